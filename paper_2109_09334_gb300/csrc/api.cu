@@ -111,6 +111,36 @@ __global__ void k_poly_dft(int n, int nout, int nfun, const cpx<double> *tw, int
     }
 }
 
+// The background functions of y (FP64 table [nfun][n1]) on the row segments:
+// per function and column c = segment * hc + m the DFT of length kSegLen of
+// the function on the segment's core, zero outside.
+template <typename T>
+__global__ void k_seg_dft(int n1, int hop, int halo, int hc, int ncol, int nfun, const double *tab, cpx<T> *out) {
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < nfun * ncol; e += gridDim.x * blockDim.x) {
+        const int q = e / ncol, c = e - q * ncol, seg = c / hc, m = c - seg * hc;
+        const int y0 = seg * hop, len = min(hop, n1 - y0);
+        double re = 0.0, im = 0.0;
+        for (int k = 0; k < len; ++k) {
+            double sn, cs;
+            sincospi(-2.0 * (double)((m * (halo + k)) % kSegLen) / kSegLen, &sn, &cs);
+            const double v = tab[(size_t)q * n1 + y0 + k];
+            re += v * cs;
+            im += v * sn;
+        }
+        out[e] = mk((T)re, (T)im);
+    }
+}
+
+// exp(-2 pi i q / n), evaluated in FP64
+template <typename T>
+__global__ void k_twiddle(int n, cpx<T> *tw) {
+    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
+        double sn, cs;
+        sincospi(-2.0 * (double)q / (double)n, &sn, &cs);
+        tw[q] = mk((T)cs, (T)sn);
+    }
+}
+
 static bool is_pow2(int v) { return v > 0 && (v & (v - 1)) == 0; }
 
 int plan_validate(const sfft_config *c) {
@@ -132,7 +162,8 @@ void plan_free(Plan *p) {
     void *bufs[] = {p->tw0, p->tw1, p->twp0, p->twp1, p->chirp1, p->bfilt1, p->twpm1, p->chirp0, p->bfilt0,
                     p->twpm0, p->kimg, p->xhat, p->yhat, p->F, p->U, p->Q, p->pairs, p->rowmom, p->lag, p->A,
                     p->Wm, p->dscale, p->r, p->xw, p->zv, p->flag, p->M_own, p->rhs_own, p->x_own, p->info_own,
-                    p->img_ref, p->img_sci, p->img_diff, p->img_mask, p->kap, p->d_int, p->ftab, p->ftab64,
+                    p->img_ref, p->img_sci, p->img_diff, p->img_mask, p->kap, p->d_int, p->ftab, p->ftab64, p->tw128,
+                    p->segy ? p->twy : nullptr,
                     p->bxy64, p->d_zdesc, p->d_rdesc, p->z0, p->cmat, p->unk, p->gam, p->bnd};
     for (void *b : bufs)
         if (b) cudaFree(b);
@@ -240,6 +271,24 @@ int plan_new(const sfft_config *cfg, cudaStream_t s, Plan **out) {
             return rc;
         }
     }
+    // Overlap-save transforms: the lag sums along x for the polynomial basis
+    // (B-spline plans need the column spectra for Lambda, and keep the row
+    // transforms these were computed from), the rows where n1 is not a power
+    // of two.
+    p->segx = p->lam_closed && p->nk <= 6;
+    p->segy = p->segx && p->gen1;
+    p->ylen = p->segy ? kSegLen : p->n1;
+    p->hc = p->ylen / 2 + 1;
+    p->nsy = 1;
+    if (p->segy) {
+        p->halo = 2 * cfg->w1;
+        const int most = kSegLen - 2 * p->halo;
+        p->nsy = (p->n1 + most - 1) / most;
+        p->hop = (p->n1 + p->nsy - 1) / p->nsy;
+        p->nsy = (p->n1 + p->hop - 1) / p->hop;  // no empty segment
+        p->offb = p->nfy;
+    }
+    p->ncol = p->nsy * p->hc;
     // gather pairs
     const int maxp = p->nk * (p->nk + 1) / 2 + p->nk * p->nbx + p->nk;
     p->host_pairs = (PairDesc *)malloc((size_t)2 * maxp * sizeof(PairDesc));
@@ -273,7 +322,7 @@ int plan_new(const sfft_config *cfg, cudaStream_t s, Plan **out) {
         // the other variants take the products one by one.
         PairDesc *g = p->host_pairs + np;
         int ng = 0, pending = -1;
-        const bool pack = !p->gen0 && p->na == 64 && 2 * cfg->w0 <= 16;
+        const bool pack = !p->segx && !p->gen0 && p->na == 64 && 2 * cfg->w0 <= 16;
         for (int k = 0; k < np; ++k) {
             const PairDesc &d = p->host_pairs[k];
             if (pack && d.kind == PK_OMEGA && d.a == d.b) {
@@ -296,7 +345,7 @@ int plan_new(const sfft_config *cfg, cudaStream_t s, Plan **out) {
     }
 
     const size_t P = (size_t)p->n0 * p->n1;
-    const size_t half = (size_t)p->h1c * p->n0;
+    const size_t half = (size_t)p->ncol * p->n0;
     const size_t csz = p->csz;
     const size_t rsz = p->fp64 ? sizeof(double) : sizeof(float);
     const int npo = p->nk * (p->nk + 1) / 2;
@@ -314,10 +363,17 @@ int plan_new(const sfft_config *cfg, cudaStream_t s, Plan **out) {
     SFFT_ALLOC(p->twp0, p->n0 * csz);
     SFFT_ALLOC(p->twp1, p->n1 * csz);
     if (!p->lam_closed) SFFT_ALLOC(p->xhat, (size_t)p->nbx * p->n0 * csz);
-    SFFT_ALLOC(p->yhat, (size_t)p->nby * p->h1c * csz);
-    SFFT_ALLOC(p->F, (size_t)(p->nfy + 1) * half * csz);
-    // the column spectra (power-of-two n0); the subtraction reuses U for D~
-    SFFT_ALLOC(p->U, (size_t)(p->gen0 ? 1 : p->nimg) * half * csz);
+    SFFT_ALLOC(p->yhat, (size_t)p->nby * p->ncol * csz);
+    SFFT_ALLOC(p->F, (size_t)(p->offb + p->nfy + 1) * half * csz);
+    // the column spectra (power-of-two n0, unless segx); the subtraction
+    // and the noise decorrelation reuse U for D~
+    {
+        const size_t dt = std::max(half, (size_t)p->h1c * p->n0);
+        SFFT_ALLOC(p->U, (p->gen0 || p->segx ? dt : (size_t)p->nimg * half) * csz);
+    }
+    if (p->segx) SFFT_ALLOC(p->tw128, 128 * csz);
+    if (p->segy) SFFT_ALLOC(p->twy, (size_t)p->ylen * csz);
+    else p->twy = p->tw1;
     SFFT_ALLOC(p->kimg, (size_t)p->L0 * p->L1 * sizeof(double));
     if (p->gen0) {
         SFFT_ALLOC(p->chirp0, (size_t)p->n0 * csz);
@@ -329,7 +385,7 @@ int plan_new(const sfft_config *cfg, cudaStream_t s, Plan **out) {
         SFFT_ALLOC(p->bfilt1, (size_t)p->m1 * csz);
         SFFT_ALLOC(p->twpm1, (size_t)p->m1 * csz);
     }
-    SFFT_ALLOC(p->Q, (size_t)p->nrows * p->h1c * csz);
+    SFFT_ALLOC(p->Q, (size_t)p->nrows * p->ncol * csz);
     SFFT_ALLOC(p->pairs, (size_t)(np + p->ngpairs) * sizeof(PairDesc));
     p->gpairs = p->pairs + np;
     SFFT_ALLOC(p->rowmom, (size_t)p->n0 * p->nmom * sizeof(double));
@@ -351,7 +407,7 @@ int plan_new(const sfft_config *cfg, cudaStream_t s, Plan **out) {
     SFFT_ALLOC(p->rhs_own, n * sizeof(double));
     SFFT_ALLOC(p->x_own, n * sizeof(double));
     SFFT_ALLOC(p->info_own, sizeof(sfft_solve_info));
-    SFFT_ALLOC(p->kap, (size_t)p->nk * p->L0 * p->h1c * csz);
+    SFFT_ALLOC(p->kap, std::max((size_t)p->nk * p->L0 * p->hc, (size_t)p->L0 * p->h1c) * csz);
 
     // constant tables
     cudaError_t err;
@@ -370,7 +426,7 @@ int plan_new(const sfft_config *cfg, cudaStream_t s, Plan **out) {
     }
     k_twiddle64<<<(p->n0 + 255) / 256, 256, 0, s>>>(p->n0, t64a);
     k_twiddle64<<<(p->n1 + 255) / 256, 256, 0, s>>>(p->n1, t64b);
-    const int bx = (p->nbx * p->n0 + 127) / 128, by = (p->nby * p->h1c + 127) / 128;
+    const int bx = (p->nbx * p->n0 + 127) / 128, by = (p->nby * p->ncol + 127) / 128;
     // the tabulated background functions (FP64)
     const double *tbx = p->bxy64, *tby = p->bxy64 + (size_t)p->nbx * p->n0;
     if (p->fp64) {
@@ -381,7 +437,13 @@ int plan_new(const sfft_config *cfg, cudaStream_t s, Plan **out) {
         if (p->xhat)
             k_poly_dft<double><<<bx, 128, 0, s>>>(p->n0, p->n0, p->nbx, t64a, p->na, p->nbk, 1, tbx,
                                                   (cpx<double> *)p->xhat);
-        k_poly_dft<double><<<by, 128, 0, s>>>(p->n1, p->h1c, p->nby, t64b, 0, 1, 0, tby, (cpx<double> *)p->yhat);
+        if (p->segy)
+            k_seg_dft<double><<<by, 128, 0, s>>>(p->n1, p->hop, p->halo, p->hc, p->ncol, p->nby, tby,
+                                             (cpx<double> *)p->yhat);
+        else
+            k_poly_dft<double><<<by, 128, 0, s>>>(p->n1, p->h1c, p->nby, t64b, 0, 1, 0, tby, (cpx<double> *)p->yhat);
+        if (p->segx) k_twiddle<double><<<1, 128, 0, s>>>(128, (cpx<double> *)p->tw128);
+        if (p->segy) k_twiddle<double><<<1, 256, 0, s>>>(p->ylen, (cpx<double> *)p->twy);
     } else {
         k_round<float><<<(p->n0 + 255) / 256, 256, 0, s>>>(p->n0, t64a, (cpx<float> *)p->tw0);
         k_round<float><<<(p->n1 + 255) / 256, 256, 0, s>>>(p->n1, t64b, (cpx<float> *)p->tw1);
@@ -390,7 +452,13 @@ int plan_new(const sfft_config *cfg, cudaStream_t s, Plan **out) {
         if (p->xhat)
             k_poly_dft<float><<<bx, 128, 0, s>>>(p->n0, p->n0, p->nbx, t64a, p->na, p->nbk, 1, tbx,
                                                  (cpx<float> *)p->xhat);
-        k_poly_dft<float><<<by, 128, 0, s>>>(p->n1, p->h1c, p->nby, t64b, 0, 1, 0, tby, (cpx<float> *)p->yhat);
+        if (p->segy)
+            k_seg_dft<float><<<by, 128, 0, s>>>(p->n1, p->hop, p->halo, p->hc, p->ncol, p->nby, tby,
+                                             (cpx<float> *)p->yhat);
+        else
+            k_poly_dft<float><<<by, 128, 0, s>>>(p->n1, p->h1c, p->nby, t64b, 0, 1, 0, tby, (cpx<float> *)p->yhat);
+        if (p->segx) k_twiddle<float><<<1, 128, 0, s>>>(128, (cpx<float> *)p->tw128);
+        if (p->segy) k_twiddle<float><<<1, 256, 0, s>>>(p->ylen, (cpx<float> *)p->twy);
     }
     for (int ax = 0; ax < 2; ++ax) {  // Bluestein tables of the axes that are not powers of two
         const bool gen = ax == 0 ? p->gen0 : p->gen1;
@@ -656,7 +724,7 @@ int sfft_plan_autotune(sfft_plan_t plan, const void *d_ref, const void *d_sci, v
     // predict the batched solves of the serving path (sfft_plan_set_tuning
     // sets it by hand).
     for (Knob &kb : knobs) {
-        if (kb.stage == SFFT_STAGE_COLS && p->gen0) continue;  // no column FFT
+        if (kb.stage == SFFT_STAGE_COLS && (p->gen0 || p->segx)) continue;  // no column FFT
         int best = 0;
         float best_ms = 1e30f;
         for (int c : kb.cand) {

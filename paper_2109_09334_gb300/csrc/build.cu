@@ -1019,7 +1019,7 @@ constexpr int kS2Out = 8;  // lag outputs per warp task in k_stage2
 constexpr int kS2Fold = 8;  // frequencies per plain partial sum in k_stage2
 
 template <typename T>
-__global__ void k_stage2(int n0, int n1, int w0, int w1, BasisView bv, int npairs,
+__global__ void k_stage2(double invP, int ylen, int hc, int ncol, int w0, int w1, BasisView bv, int npairs,
                          const PairDesc *__restrict__ pairs, const cpx<T> *__restrict__ Q,
                          const cpx<T> *__restrict__ yhat, const cpx<T> *__restrict__ tw1,
                          double *__restrict__ lag, int off_om, int off_la, int off_th) {
@@ -1030,14 +1030,13 @@ __global__ void k_stage2(int n0, int n1, int w0, int w1, BasisView bv, int npair
         if (row >= pairs[k].row0 && row < pairs[k].row0 + 2 * pairs[k].h0 + 1) pi = k;
     const PairDesc pd = pairs[pi];
     const int rho0 = row - pd.row0 - pd.h0;
-    const int h1c = n1 / 2 + 1;
     const int nk = bv.nk;
     const int nbt = bv.nb;
     const int h1 = (pd.kind == PK_OMEGA) ? 2 * w1 : w1;
     int nq = 1;
     if (pd.kind == PK_LAMBDA) nq = bv.lamn(pd.b);  // background terms whose x-function is p = b
-    const cpx<T> *q = Q + (size_t)row * h1c;
-    const double invP = 1.0 / ((double)n0 * (double)n1);
+    const cpx<T> *q = Q + (size_t)row * ncol;
+    const bool seg = ncol != hc;  // columns of several row segments
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     // outputs in chunks of up to kS2Out lags rho1 >= 0 of one q index, each
     // with its mirror -rho1 (cpq chunks per q): both come from one twiddle,
@@ -1065,16 +1064,17 @@ __global__ void k_stage2(int n0, int n1, int w0, int w1, BasisView bv, int npair
         if (act) {
             int cnt = 0;
             const int mstep = nsp * 32;
-            const int dstep = imod(mstep * r0, n1);  // change of (mm r0) mod n1 per step of mm
-            int idx0 = imod((sp * 32 + lane) * r0, n1);
-            for (int mm = sp * 32 + lane; mm < h1c; mm += mstep) {
-                cpx<T> v = q[mm];
-                if (pd.kind == PK_LAMBDA) v = cmul(v, yhat[(size_t)bv.lamq(pd.b, qi) * h1c + mm]);
-                const T wm = (mm == 0 || (2 * mm == n1)) ? (T)1 : (T)2;
+            const int dstep = imod(mstep * r0, ylen);  // change of (mm r0) mod ylen per step of mm
+            int idx0 = imod((sp * 32 + lane) * r0, ylen);
+            for (int cc = sp * 32 + lane; cc < ncol; cc += mstep) {
+                cpx<T> v = q[cc];
+                const int mm = seg ? cc % hc : cc;  // frequency of the column
+                if (pd.kind == PK_LAMBDA) v = cmul(v, yhat[(size_t)bv.lamq(pd.b, qi) * ncol + cc]);
+                const T wm = (mm == 0 || (2 * mm == ylen)) ? (T)1 : (T)2;
                 v = scale(v, wm);
-                int idx = idx0;  // (mm rho1) mod n1, stepped by mm over the chunk's lags
+                int idx = seg ? imod(mm * r0, ylen) : idx0;  // (mm rho1) mod ylen, stepped by mm over the chunk's lags
                 idx0 += dstep;
-                if (idx0 >= n1) idx0 -= n1;
+                if (idx0 >= ylen) idx0 -= ylen;
 #pragma unroll
                 for (int k = 0; k < kS2Out; ++k) {
                     if (r0 + k <= h1) {
@@ -1083,7 +1083,7 @@ __global__ void k_stage2(int n0, int n1, int w0, int w1, BasisView bv, int npair
                         pl[kS2Out + k] += v.re * e.re + v.im * e.im;
                     }
                     idx += mm;
-                    if (idx >= n1) idx -= n1;
+                    if (idx >= ylen) idx -= ylen;
                 }
                 if (++cnt == kS2Fold) {
 #pragma unroll
@@ -1220,7 +1220,10 @@ static cudaError_t launch_rows(Plan *p, const void *ref, const void *sci, const 
                                bool moments, cudaStream_t s) {
     const int nfft = (p->nfy + 2) / 2;
     const FTab<T> ft = ftab_of<T>(p);
-    if (p->gen1) {
+    if (p->segy) {
+        const cudaError_t e = rows_segments(p, ref, sci, mask, moments, s);
+        if (e != cudaSuccess) return e;
+    } else if (p->gen1) {
         const int G = p->m1 / 16;
         int TR = (sizeof(T) == 4 ? 1024 : 512) / G;
         if (TR < 1) TR = 1;
@@ -1252,7 +1255,7 @@ static cudaError_t launch_rows(Plan *p, const void *ref, const void *sci, const 
                                                               (const cpx<T> *)p->twp1, p->bspline ? ft.fy : nullptr,
                                                               kRowsPrefetch * p->sms);
     }
-    p->launches++;
+    if (!p->segy) p->launches++;
     if (moments && !p->bspline) {
         auto km = (p->cfg.dk == 2 && p->cfg.db == 2) ? k_row_moments<T, I, 5, 5, 3, 3> : k_row_moments<T, I>;
         km<<<p->n0, 256, 0, s>>>(p->n1, p->cfg.dk, p->cfg.db, (const I *)ref, (const I *)sci, mask, p->rowmom);
@@ -1275,7 +1278,7 @@ template <typename T>
 static cudaError_t launch_cols(Plan *p, cudaStream_t s) {
     k_zero_lag<<<p->nzm, 256, 0, s>>>(p->n0, p->nmom, p->d_zdesc, p->ftab64, p->rowmom, p->z0);
     p->launches++;
-    if (p->gen0) return cudaGetLastError();  // the lag sums along x need no column spectra
+    if (p->gen0 || p->segx) return cudaGetLastError();  // the lag sums along x need no column spectra
     const int G = p->n0 / 16;
     // about 256 threads per block (one 4096-point transform; the twiddles
     // come through L1, so small blocks cost no table copies), at most 4 images
@@ -1304,6 +1307,7 @@ static cudaError_t launch_cols(Plan *p, cudaStream_t s) {
 
 template <typename T>
 static cudaError_t launch_gather(Plan *p, cudaStream_t s) {
+    if (p->segx) return lag_sums_x(p, s);
     if (p->gen0) {
         const int hmax = 2 * p->cfg.w0;
         const size_t smem = (size_t)(2 * p->n0 + 2 * (hmax + 8) + 16) * sizeof(cpx<T>) + (size_t)p->n0 * sizeof(T);
@@ -1347,9 +1351,10 @@ static cudaError_t launch_gather(Plan *p, cudaStream_t s) {
 template <typename T>
 static cudaError_t launch_lags(Plan *p, double *M, double *rhs, cudaStream_t s) {
     cudaError_t err;
-    k_stage2<T><<<p->nrows, 256, 0, s>>>(p->n0, p->n1, p->cfg.w0, p->cfg.w1, p->bv, p->npairs,
-                                         p->pairs, (const cpx<T> *)p->Q, (const cpx<T> *)p->yhat,
-                                         (const cpx<T> *)p->tw1, p->lag, p->lag_om, p->lag_la, p->lag_th);
+    const int xlen = p->segx ? kLagLen : p->n0;  // length of the transforms along x
+    k_stage2<T><<<p->nrows, 256, 0, s>>>(1.0 / ((double)xlen * (double)p->ylen), p->ylen, p->hc, p->ncol, p->cfg.w0, p->cfg.w1, p->bv,
+                                         p->npairs, p->pairs, (const cpx<T> *)p->Q, (const cpx<T> *)p->yhat,
+                                         (const cpx<T> *)p->twy, p->lag, p->lag_om, p->lag_la, p->lag_th);
     p->launches++;
     if ((err = cudaGetLastError())) return err;
     LagView lv;

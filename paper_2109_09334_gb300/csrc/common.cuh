@@ -25,10 +25,34 @@ template <typename T>
 __device__ __forceinline__ cpx<T> operator+(cpx<T> a, cpx<T> b) { return mk(a.re + b.re, a.im + b.im); }
 template <typename T>
 __device__ __forceinline__ cpx<T> operator-(cpx<T> a, cpx<T> b) { return mk(a.re - b.re, a.im - b.im); }
+// In FP32 both parts in one packed instruction: the same roundings at the same
+// rate, but half the issue slots, which bound the transforms.
+__device__ __forceinline__ cpx<float> operator+(cpx<float> a, cpx<float> b) {
+    cpx<float> c;
+    asm("{\n .reg .b64 a, b, c;\n mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %5};\n add.rn.f32x2 c, a, b;\n"
+        " mov.b64 {%0, %1}, c;\n}"
+        : "=f"(c.re), "=f"(c.im)
+        : "f"(a.re), "f"(a.im), "f"(b.re), "f"(b.im));
+    return c;
+}
+__device__ __forceinline__ cpx<float> operator-(cpx<float> a, cpx<float> b) {
+    cpx<float> c;
+    asm("{\n .reg .b64 a, b, c;\n mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %5};\n sub.rn.f32x2 c, a, b;\n"
+        " mov.b64 {%0, %1}, c;\n}"
+        : "=f"(c.re), "=f"(c.im)
+        : "f"(a.re), "f"(a.im), "f"(b.re), "f"(b.im));
+    return c;
+}
 template <typename T>
 __device__ __forceinline__ cpx<T> cmul(cpx<T> a, cpx<T> b) {
     return mk(a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re);
 }
+// a + b and a - b by part: where b is a product, the compiler fuses it into
+// the sum
+template <typename T>
+__device__ __forceinline__ cpx<T> cadd(cpx<T> a, cpx<T> b) { return mk(a.re + b.re, a.im + b.im); }
+template <typename T>
+__device__ __forceinline__ cpx<T> csub(cpx<T> a, cpx<T> b) { return mk(a.re - b.re, a.im - b.im); }
 // acc + a * b and acc - a * b as four fused multiply-adds each (the
 // products are not rounded separately, so the results differ from
 // acc +- cmul(a, b) in the last bits; both are single-rounding-per-term sums)

@@ -22,11 +22,13 @@ __device__ __forceinline__ cpx<T> twiddle(const cpx<T> *__restrict__ tw, int q, 
 // 4-point DFT with sign sgn on (v0..v3) in place
 template <typename T>
 __device__ __forceinline__ void dft4(cpx<T> &v0, cpx<T> &v1, cpx<T> &v2, cpx<T> &v3, int sgn) {
-    cpx<T> a = v0 + v2, b = v0 - v2, c = v1 + v3, d = mul_i(v1 - v3, sgn);
+    cpx<T> a = v0 + v2, b = v0 - v2, c = v1 + v3, e = v1 - v3;
     v0 = a + c;
     v2 = a - c;
-    v1 = b + d;
-    v3 = b - d;
+    // b +- (sgn i) e, by part: the rotated operand needs no register moves
+    const cpx<T> p = mk(b.re - e.im, b.im + e.re), m = mk(b.re + e.im, b.im - e.re);
+    v1 = sgn > 0 ? p : m;
+    v3 = sgn > 0 ? m : p;
 }
 
 // 8-point DFT with sign sgn on v (natural order in and out): a radix-2 split

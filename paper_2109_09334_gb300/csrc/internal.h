@@ -12,6 +12,11 @@ namespace sfft {
 // r in [0, NA)): min(64, n0).
 constexpr int kMaxNA = 64;
 
+// Row segments of a row length that is not a power of two (segment.cu).
+constexpr int kSegLen = 256;
+// Window length of the lag sums along x (segment.cu).
+constexpr int kLagLen = 128;
+
 // Cooperative solve grid: at most kMaxSolveGrid blocks.  The plan's vector
 // xw holds x (n), then the solve's statistics (8) and per-block partial sums
 // (2 per block), then the subtraction's kernel sums.
@@ -102,6 +107,17 @@ struct Plan {
     // Bluestein DFTs of length n1 through FFTs of length m1; gen0: the lag
     // sums along x are direct circular correlations (k_xcorr), no column FFT.
     int gen0, gen1, m0, m1;
+    // Overlap-save transforms (segment.cu).  segx: the lag sums along x by
+    // k_lagx (polynomial basis, n_K <= 6 terms, w0 <= 16); else the column
+    // FFT and gather, or k_xcorr.  segy: the rows by segments of kSegLen
+    // (gen1 only; nsy segments of core length hop, halo 2 w1).  The row
+    // transform table F has ncol columns: column c is frequency c mod hc of a
+    // transform of length ylen (of segment c / hc).
+    int segx, segy, nsy, hop, halo;
+    int ylen, hc, ncol;
+    int offb;              // first window sequence in F (segy: after the nfy core sequences)
+    void *twy;             // twiddles of length ylen (= tw1 unless segy)
+    void *tw128;           // twiddles of length 128 (segx)
     void *chirp1, *bfilt1, *twpm1;  // Bluestein tables for n1 (compute type)
     void *chirp0, *bfilt0, *twpm0;  // Bluestein tables for n0 (noise decorrelation only)
     double *kimg;                   // L0 x L1 kernel image (noise decorrelation)
@@ -243,6 +259,11 @@ struct Coadd {
 };
 cudaError_t decorrelate(Plan *p, const double *x, double xt0, double yt0, double sigma_ref, double sigma_sci,
                         const void *diff, void *out, const Coadd *co, cudaStream_t s);
+// overlap-save transforms (segment.cu)
+cudaError_t lag_sums_x(Plan *p, cudaStream_t s);
+cudaError_t rows_segments(Plan *p, const void *ref, const void *sci, const uint8_t *mask, bool core,
+                          cudaStream_t s);
+cudaError_t rows_inv_segments(Plan *p, void *diff, cudaStream_t s);
 cudaError_t subtract_from_rows(Plan *p, const double *x, void *diff, cudaStream_t s);
 cudaError_t plan_tables(Plan *p, cudaStream_t s);
 

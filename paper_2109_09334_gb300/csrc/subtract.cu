@@ -43,10 +43,10 @@ __global__ void k_kernel_sums(BasisView bv, const double *__restrict__ x, double
 
 // kap[t][a + w0][m]
 template <typename T>
-__global__ void k_kernel_table(int n1, BasisView bv, const double *__restrict__ x, const double *__restrict__ ksum,
+__global__ void k_kernel_table(int ylen, BasisView bv, const double *__restrict__ x, const double *__restrict__ ksum,
                                const cpx<T> *__restrict__ tw1, cpx<T> *__restrict__ kap) {
     const int w0 = bv.w0, w1 = bv.w1;
-    const int h1c = n1 / 2 + 1, L0 = 2 * w0 + 1;
+    const int h1c = ylen / 2 + 1, L0 = 2 * w0 + 1;
     const size_t total = (size_t)bv.nk * L0 * h1c;
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
         const int m = (int)(e % h1c);
@@ -57,7 +57,7 @@ __global__ void k_kernel_table(int n1, BasisView bv, const double *__restrict__ 
             const int u = bv.unknown(t, a, b);
             double c = u >= 0 ? x[u] : 0.0;
             if (a == 0 && b == 0) c -= ksum[t];
-            cpx<T> w = tw1[imod(m * b, n1)];  // exp(-2 pi i m b / n1)
+            cpx<T> w = tw1[imod(m * b, ylen)];  // exp(-2 pi i m b / ylen)
             re += (T)c * w.re;
             im += (T)c * w.im;
         }
@@ -78,7 +78,7 @@ __host__ __device__ constexpr int sub_q() { return sizeof(T) == 4 ? 4 : 8; }
 // W0 >= 0: the kernel half-width is the compile-time W0 (the tap loop unrolls
 // completely, so the window shifts are register renames); W0 < 0: w0 at run time.
 template <typename T, bool P2, int W0>
-__global__ void __launch_bounds__(sizeof(T) == 4 ? 1024 : 512) k_sub_cols(int n0, int n1, BasisView bv, FTab<T> ft,
+__global__ void __launch_bounds__(sizeof(T) == 4 ? 1024 : 512) k_sub_cols(int n0, int hc, int ncol, int offb, BasisView bv, FTab<T> ft,
                                                                          int w0, int nbkg_off,
                                                                          const cpx<T> *__restrict__ F,
                                                                          const cpx<T> *__restrict__ kap,
@@ -93,30 +93,29 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? 1024 : 512) k_sub_cols(int n0
     constexpr int Q = sub_q<T>();
     cpx<T> *Wb = kp + nk * L0;  // two buffers of n0 + n0 / Q (padded), alternating by term
     auto padq = [](int v) { return v + v / Q; };
-    const int m = blockIdx.x, tid = threadIdx.x, nthr = blockDim.x;
-    const int h1c = n1 / 2 + 1;
+    const int col = blockIdx.x, m = col % hc, tid = threadIdx.x, nthr = blockDim.x;
     const int msk = n0 - 1;
     // index mod n0 for -n0 <= v < 2 n0 (P2: n0 is a power of two)
     auto wrapx = [&](int v) { return P2 ? (v & msk) : (v < 0 ? v + n0 : (v >= n0 ? v - n0 : v)); };
     const int x0 = Q * tid;  // outputs x0 .. x0 + Q - 1 below n0
-    for (int e = tid; e < nk * L0; e += nthr) kp[e] = kap[(size_t)e * h1c + m];
+    for (int e = tid; e < nk * L0; e += nthr) kp[e] = kap[(size_t)e * hc + m];
     T xt[Q];
 #pragma unroll
     for (int q = 0; q < Q; ++q) xt[q] = coord<T>(x0 + q, n0);
     // S~ minus the background B~(x, m) = sum_s b_s bx_p(x) Y_q(m)
     cpx<T> acc[Q];
     {
-        const cpx<T> *Sc = F + ((size_t)bv.nfy * h1c + m) * n0 + x0;
+        const cpx<T> *Sc = F + ((size_t)(offb + bv.nfy) * ncol + col) * n0 + x0;
 #pragma unroll
         for (int q = 0; q < Q; ++q) acc[q] = (P2 || x0 + q < n0) ? Sc[q] : mk((T)0, (T)0);
         for (int s = 0; s < nbt; ++s) {
             const int p = bv.sp(s), qq = bv.sq(s);
-            const cpx<T> yq = yhat[(size_t)qq * h1c + m];
+            const cpx<T> yq = yhat[(size_t)qq * ncol + col];
             const T bpq = (T)x[nbkg_off + s];
 #pragma unroll
             for (int q = 0; q < Q; ++q) {
                 const T wx = ft.bx ? ((P2 || x0 + q < n0) ? ft.bx[(size_t)p * n0 + x0 + q] : (T)0) : ipow(xt[q], p);
-                acc[q] = acc[q] - scale(yq, bpq * wx);
+                acc[q] = csub(acc[q], scale(yq, bpq * wx));
             }
         }
     }
@@ -129,7 +128,7 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? 1024 : 512) k_sub_cols(int n0
         const int ncj = bv.jcnt(j);
         if (ncj == 0) continue;
         cpx<T> f[Q];
-        const cpx<T> *Fj = F + ((size_t)j * h1c + m) * n0 + x0;
+        const cpx<T> *Fj = F + ((size_t)(offb + j) * ncol + col) * n0 + x0;
 #pragma unroll
         for (int q = 0; q < Q; ++q) f[q] = (P2 || x0 + q < n0) ? Fj[q] : mk((T)0, (T)0);
         for (int k = 0; k < ncj; ++k) {
@@ -157,7 +156,7 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? 1024 : 512) k_sub_cols(int n0
             }
         }
     }
-    cpx<T> *out = Dt + (size_t)m * n0 + x0;
+    cpx<T> *out = Dt + (size_t)col * n0 + x0;
 #pragma unroll
     for (int q = 0; q < Q; ++q)
         if (P2 || x0 + q < n0) out[q] = acc[q];
@@ -333,10 +332,10 @@ static cudaError_t sub_t(Plan *p, const double *x, void *diff, cudaStream_t s) {
     double *ksum = p->xw + p->n + kSolveTail;  // after the solve's statistics and partial sums
     p->launches += 4;
     k_kernel_sums<<<p->nk, 256, 0, s>>>(p->bv, x, ksum);
-    const size_t tot = (size_t)p->nk * p->L0 * p->h1c;
+    const size_t tot = (size_t)p->nk * p->L0 * p->hc;
     int blocks = (int)((tot + 255) / 256);
     if (blocks > 8192) blocks = 8192;
-    k_kernel_table<T><<<blocks, 256, 0, s>>>(p->n1, p->bv, x, ksum, (const cpx<T> *)p->tw1, (cpx<T> *)p->kap);
+    k_kernel_table<T><<<blocks, 256, 0, s>>>(p->ylen, p->bv, x, ksum, (const cpx<T> *)p->twy, (cpx<T> *)p->kap);
     if ((err = cudaGetLastError())) return err;
     {
         const int nthr = (p->n0 + sub_q<T>() - 1) / sub_q<T>();
@@ -353,13 +352,13 @@ static cudaError_t sub_t(Plan *p, const double *x, void *diff, cudaStream_t s) {
             default: break;
         }
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        kern<<<p->h1c, nthr, smem, s>>>(p->n0, p->n1, p->bv, ftab_of<T>(p), p->cfg.w0, nbkg_off,
+        kern<<<p->ncol, nthr, smem, s>>>(p->n0, p->hc, p->ncol, p->offb, p->bv, ftab_of<T>(p), p->cfg.w0, nbkg_off,
                                         (const cpx<T> *)p->F, (const cpx<T> *)p->kap, (const cpx<T> *)p->yhat, x,
                                         (cpx<T> *)p->U);
         if ((err = cudaGetLastError())) return err;
     }
-    if ((err = launch_rows_inv<T>(p, diff, s))) return err;
-    return cudaGetLastError();
+    if (p->segy) return rows_inv_segments(p, diff, s);
+    return launch_rows_inv<T>(p, diff, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -419,7 +418,7 @@ __global__ void k_decorr_kappa(int n1, int nkern, int na, int w0, int w1, const 
         const int c = ca / L0, a = ca - c * L0;
         const double *k = c < na ? kimg_a + (size_t)c * L0 * L1 : kimg_b + (size_t)(c - na) * L0 * L1;
         cpx<T> v = mk((T)0, (T)0);
-        for (int bi = 0; bi < L1; ++bi) v = v + scale(tw1[imod(m * (bi - w1), n1)], (T)k[a * L1 + bi]);
+        for (int bi = 0; bi < L1; ++bi) v = cadd(v, scale(tw1[imod(m * (bi - w1), n1)], (T)k[a * L1 + bi]));
         kap[e] = v;
     }
 }
@@ -502,7 +501,7 @@ __global__ void __launch_bounds__(512) k_decorr_cols(int n0, int n1, int mlen, i
         const T num = (T)(ss2 + sr2 * k00 * k00);
         for (int l = tid; l < n0; l += G) {
             cpx<T> kh = mk((T)0, (T)0);
-            for (int a = 0; a < L0; ++a) kh = kh + cmul(kp[a], tw0[imod(l * (a - w0), n0)]);
+            for (int a = 0; a < L0; ++a) kh = cadd(kh, cmul(kp[a], tw0[imod(l * (a - w0), n0)]));
             const T q = sqrt(num / ((T)ss2 + (T)sr2 * (kh.re * kh.re + kh.im * kh.im)));
             zr[pad16(l)] = scale(zr[pad16(l)], q);
         }
@@ -518,11 +517,11 @@ __global__ void __launch_bounds__(512) k_decorr_cols(int n0, int n1, int mlen, i
         const T num = (T)(ds + k00 * k00 * dr);
         for (int l = tid; l < n0; l += G) {
             cpx<T> kh = mk((T)0, (T)0);
-            for (int a = 0; a < L0; ++a) kh = kh + cmul(kp[a], tw0[imod(l * (a - w0), n0)]);
+            for (int a = 0; a < L0; ++a) kh = cadd(kh, cmul(kp[a], tw0[imod(l * (a - w0), n0)]));
             T es = (T)0, er = (T)0;
             for (int c = 0; c < nc; ++c) {
                 cpx<T> gh = mk((T)0, (T)0);
-                for (int a = 0; a < Lg; ++a) gh = gh + cmul(gp[c * Lg + a], tw0[imod(l * (a - cd.g0), n0)]);
+                for (int a = 0; a < Lg; ++a) gh = cadd(gh, cmul(gp[c * Lg + a], tw0[imod(l * (a - cd.g0), n0)]));
                 const T e2 = (T)cd.s2[c] * (gh.re * gh.re + gh.im * gh.im);
                 if (c < cd.ns) es += e2;
                 else er += e2;
