@@ -441,13 +441,11 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? 1024 : 512) k_decorr_rows(int
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int G = mlen / 16;
     const int np = padded_len(mlen);
-    const int ntw = BLU ? 0 : pass_table_len(n1);
-    cpx<T> *tw = reinterpret_cast<cpx<T> *>(smem_raw);  // pass table (pow2)
-    cpx<T> *Z = tw + ntw;                                // NG * np
-    const int tid = threadIdx.x, nthr = blockDim.x;
+    const cpx<T> *tw = twg;                              // pass table (pow2), read through L1
+    cpx<T> *Z = reinterpret_cast<cpx<T> *>(smem_raw);   // NG * np
+    const int tid = threadIdx.x;
     const int grp = tid / G, gt = tid - grp * G;
     const int xa = (blockIdx.x * NG + grp) * 2, xb = xa + 1;
-    for (int q = tid; q < ntw; q += nthr) tw[q] = twg[q];
     cpx<T> *zr = Z + (size_t)grp * np;
     for (int y = gt; y < n1; y += G) {
         const T a = xa < n0 ? (T)D[(size_t)xa * n1 + y] : (T)0;
@@ -457,12 +455,16 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? 1024 : 512) k_decorr_rows(int
     __syncthreads();
     if (BLU) bluestein(zr, n1, mlen, -1, chirp, bfilt, twg, gt, G);
     else group_fft(zr, n1, -1, tw, gt, G);
+    // the block's 2 NG rows (a power of two) side by side along x
     const int h1c = n1 / 2 + 1;
-    for (int m = gt; m < h1c; m += G) {
-        const cpx<T> z = zr[pad16(m)];
-        const cpx<T> zc = conj(zr[pad16(m == 0 ? 0 : n1 - m)]);
-        if (xa < n0) Dt[(size_t)m * n0 + xa] = scale(z + zc, (T)0.5);
-        if (xb < n0) Dt[(size_t)m * n0 + xb] = mul_i(scale(z - zc, (T)0.5), -1);
+    const int nr = 2 * NG, total = h1c * nr;
+    for (int e = tid; e < total; e += NG * G) {
+        const int r = e & (nr - 1), m = e / nr, x = blockIdx.x * nr + r;
+        if (x >= n0) continue;
+        const cpx<T> *zz = Z + (size_t)(r >> 1) * np;
+        const cpx<T> z = zz[pad16(m)];
+        const cpx<T> zc = conj(zz[pad16(m == 0 ? 0 : n1 - m)]);
+        Dt[(size_t)m * n0 + x] = (r & 1) ? mul_i(scale(z - zc, (T)0.5), -1) : scale(z + zc, (T)0.5);
     }
 }
 
@@ -477,54 +479,97 @@ __global__ void __launch_bounds__(512) k_decorr_cols(int n0, int n1, int mlen, i
                                                       CoaddDesc cd, const cpx<T> *__restrict__ gam) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int G = mlen / 16;
-    const int ntw = BLU ? 0 : pass_table_len(n0);
     const int L0 = 2 * w0 + 1;
     const int nc = cd.ns + cd.nr, Lg = 2 * cd.g0 + 1;  // nc = 0: the one-pair form
-    cpx<T> *tw = reinterpret_cast<cpx<T> *>(smem_raw);  // pass table (pow2)
-    cpx<T> *kp = tw + ntw;                               // L0: kappa(a, m)
+    const cpx<T> *tw = twg;                               // pass table (pow2), read through L1
+    cpx<T> *kp = reinterpret_cast<cpx<T> *>(smem_raw);   // L0: kappa(a, m)
     cpx<T> *gp = kp + L0;                                // nc * Lg: gamma_c(a, m)
     cpx<T> *zr = gp + nc * Lg;                           // padded mlen
     const int tid = threadIdx.x, m = blockIdx.x;
     const int h1c = n1 / 2 + 1;
-    for (int q = tid; q < ntw; q += G) tw[q] = twg[q];
     for (int a = tid; a < L0; a += G) kp[a] = kap[(size_t)a * h1c + m];
     for (int e = tid; e < nc * Lg; e += G) gp[e] = gam[(size_t)e * h1c + m];
-    double k00 = 0.0;  // K^(0, 0): the kernel sum
-    for (int a = 0; a < L0; ++a) k00 += (double)kap[(size_t)a * h1c].re;
+    // K^(0, 0) (kernel nc) and the sums of the homogenisation kernels, one
+    // thread each: FP64 sums in every thread took as long as the transforms
+    __shared__ double ksums[2 * kMaxCoadd + 1];
+    __shared__ double numer;  // the filter's numerator: its denominator at frequency 0
+    for (int c = tid; c <= nc; c += G) {
+        double v = 0.0;
+        if (c == nc) {
+            for (int a = 0; a < L0; ++a) v += (double)kap[(size_t)a * h1c].re;
+        } else {
+            for (int a = 0; a < Lg; ++a) v += (double)gam[((size_t)c * Lg + a) * h1c].re;
+        }
+        ksums[c] = v;
+    }
     cpx<T> *col = Dt + (size_t)m * n0;
     for (int x = tid; x < n0; x += G) zr[pad16(x)] = col[x];
     __syncthreads();
+    if (tid == 0) {
+        const double k00 = ksums[nc];
+        if (nc == 0) {
+            const double ss2 = sigma_sci * sigma_sci, sr2 = sigma_ref * sigma_ref;
+            numer = ss2 + sr2 * k00 * k00;
+        } else {
+            double ds = 0.0, dr = 0.0;
+            for (int c = 0; c < nc; ++c) {
+                const double g00 = ksums[c];
+                (c < cd.ns ? ds : dr) += cd.s2[c] * g00 * g00;
+            }
+            numer = ds + k00 * k00 * dr;
+        }
+    }
     if (BLU) bluestein(zr, n0, mlen, -1, chirp, bfilt, twg, tid, G);
     else group_fft(zr, n0, -1, tw, tid, G);
+    // K^(l, m) = sum_a kappa(a, m) e^(-2 pi i l a / N0): the twiddle index steps by l
+    auto khat = [&](int l) {
+        cpx<T> kh = mk((T)0, (T)0);
+        int idx = imod(-l * w0, n0);
+        for (int a = 0; a < L0; ++a) {
+            kh = cadd(kh, cmul(kp[a], tw0[idx]));
+            idx += l;
+            if (idx >= n0) idx -= n0;
+        }
+        return kh;
+    };
     if (nc == 0) {
         const double ss2 = sigma_sci * sigma_sci, sr2 = sigma_ref * sigma_ref;
-        const T num = (T)(ss2 + sr2 * k00 * k00);
+        const T num = (T)numer;
         for (int l = tid; l < n0; l += G) {
-            cpx<T> kh = mk((T)0, (T)0);
-            for (int a = 0; a < L0; ++a) kh = cadd(kh, cmul(kp[a], tw0[imod(l * (a - w0), n0)]));
+            const cpx<T> kh = khat(l);
             const T q = sqrt(num / ((T)ss2 + (T)sr2 * (kh.re * kh.re + kh.im * kh.im)));
             zr[pad16(l)] = scale(zr[pad16(l)], q);
         }
     } else {
         // Eq. 23-24 in full: den = sum_j s_Sj^2 |G^_j|^2 + |K^|^2 sum_i s_Ri^2 |H^_i|^2,
-        // normalised by its value at frequency 0 (unit kernel sum)
-        double ds = 0.0, dr = 0.0;
-        for (int c = 0; c < nc; ++c) {
-            double g00 = 0.0;
-            for (int a = 0; a < Lg; ++a) g00 += (double)gam[((size_t)c * Lg + a) * h1c].re;
-            (c < cd.ns ? ds : dr) += cd.s2[c] * g00 * g00;
-        }
-        const T num = (T)(ds + k00 * k00 * dr);
+        // normalised by its value at frequency 0 (unit kernel sum).  Eight
+        // kernels at a time share each twiddle.
+        const T num = (T)numer;
+        constexpr int kC = 8;
         for (int l = tid; l < n0; l += G) {
-            cpx<T> kh = mk((T)0, (T)0);
-            for (int a = 0; a < L0; ++a) kh = cadd(kh, cmul(kp[a], tw0[imod(l * (a - w0), n0)]));
+            const cpx<T> kh = khat(l);
             T es = (T)0, er = (T)0;
-            for (int c = 0; c < nc; ++c) {
-                cpx<T> gh = mk((T)0, (T)0);
-                for (int a = 0; a < Lg; ++a) gh = cadd(gh, cmul(gp[c * Lg + a], tw0[imod(l * (a - cd.g0), n0)]));
-                const T e2 = (T)cd.s2[c] * (gh.re * gh.re + gh.im * gh.im);
-                if (c < cd.ns) es += e2;
-                else er += e2;
+            const int idx0 = imod(-l * cd.g0, n0);
+            for (int c0 = 0; c0 < nc; c0 += kC) {
+                cpx<T> gh[kC];
+#pragma unroll
+                for (int j = 0; j < kC; ++j) gh[j] = mk((T)0, (T)0);
+                int idx = idx0;
+                for (int a = 0; a < Lg; ++a) {
+                    const cpx<T> w = tw0[idx];
+#pragma unroll
+                    for (int j = 0; j < kC; ++j)
+                        if (c0 + j < nc) gh[j] = cadd(gh[j], cmul(gp[(c0 + j) * Lg + a], w));
+                    idx += l;
+                    if (idx >= n0) idx -= n0;
+                }
+#pragma unroll
+                for (int j = 0; j < kC; ++j) {
+                    if (c0 + j >= nc) break;
+                    const T e2 = (T)cd.s2[c0 + j] * (gh[j].re * gh[j].re + gh[j].im * gh[j].im);
+                    if (c0 + j < cd.ns) es += e2;
+                    else er += e2;
+                }
             }
             const T q = sqrt(num / (es + (kh.re * kh.re + kh.im * kh.im) * er));
             zr[pad16(l)] = scale(zr[pad16(l)], q);
@@ -568,8 +613,7 @@ static cudaError_t decorr_t(Plan *p, const double *x, double xt0, double yt0, do
         if (NG < 1) NG = 1;
         if (NG > 4) NG = 4;
         if (NG > (p->n0 + 1) / 2) NG = (p->n0 + 1) / 2;
-        const int ntw = p->gen1 ? 0 : pass_table_len(p->n1);
-        auto smem_of = [&](int ng) { return ((size_t)ntw + (size_t)ng * padded_len(p->m1)) * sizeof(cpx<T>); };
+        auto smem_of = [&](int ng) { return (size_t)ng * padded_len(p->m1) * sizeof(cpx<T>); };
         while (NG > 1 && smem_of(NG) > 200 * 1024) NG /= 2;
         const size_t smem = smem_of(NG);
         const int blocks = (p->n0 + 2 * NG - 1) / (2 * NG);
@@ -595,9 +639,8 @@ static cudaError_t decorr_t(Plan *p, const double *x, double xt0, double yt0, do
     }
     {  // columns
         const int G = p->m0 / 16;
-        const int ntw = p->gen0 ? 0 : pass_table_len(p->n0);
         const int ncg = (cd.ns + cd.nr) * (2 * cd.g0 + 1);
-        const size_t smem = ((size_t)ntw + p->L0 + ncg + padded_len(p->m0)) * sizeof(cpx<T>);
+        const size_t smem = ((size_t)p->L0 + ncg + padded_len(p->m0)) * sizeof(cpx<T>);
         auto kern = p->gen0 ? k_decorr_cols<T, true> : k_decorr_cols<T, false>;
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         kern<<<p->h1c, G, smem, s>>>(p->n0, p->n1, p->m0, w0, sr, ss, (const cpx<T> *)p->kap, (const cpx<T> *)p->tw0,
