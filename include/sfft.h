@@ -137,15 +137,12 @@ int sfft_plan_destroy(sfft_plan_t plan);
 int sfft_plan_workspace_bytes(sfft_plan_t plan, uint64_t *bytes);
 
 /*
- * Panel width of the blocked Cholesky factorisation of the FP32 solve (the
- * solve of Eq. 18; FP64 plans always use 32): 32 (the default) or 64.  With
- * 64 a solve needs half the grid barriers and half the passes over the
- * trailing matrix but a longer serial chain per diagonal block: faster when
- * several systems share a launch (sfft_run_pairs, batches, servers), slower
- * for one system alone.  The widths round differently (both meet the
- * solve's tolerance); systems solved in one launch must share the width
- * (SFFT_ERR_INVALID otherwise).  Server slots and pool lanes that batch
- * four or more pairs (batch >= 4) use 64.  SFFT_ERR_INVALID for another width.
+ * Panel width setting of the FP32 solve (the solve of Eq. 18): 32 (the
+ * default) or 64.  The factorisation does the arithmetic of 32-wide panels,
+ * two to a step, for both, so the results do not depend on the setting;
+ * systems solved in one launch must share it (SFFT_ERR_INVALID otherwise).
+ * Server slots and pool lanes that batch four or more pairs (batch >= 4) set
+ * 64.  SFFT_ERR_INVALID for another width.
  */
 int sfft_plan_set_solve_panel(sfft_plan_t plan, int32_t width);
 int sfft_plan_solve_panel(sfft_plan_t plan, int32_t *width);

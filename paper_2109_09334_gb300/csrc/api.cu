@@ -161,7 +161,7 @@ int plan_validate(const sfft_config *c) {
 void plan_free(Plan *p) {
     void *bufs[] = {p->tw0, p->tw1, p->twp0, p->twp1, p->chirp1, p->bfilt1, p->twpm1, p->chirp0, p->bfilt0,
                     p->twpm0, p->kimg, p->xhat, p->yhat, p->F, p->U, p->Q, p->pairs, p->rowmom, p->lag, p->A,
-                    p->Wm, p->dscale, p->r, p->xw, p->zv, p->flag, p->M_own, p->rhs_own, p->x_own, p->info_own,
+                    p->dscale, p->r, p->xw, p->zv, p->flag, p->M_own, p->rhs_own, p->x_own, p->info_own,
                     p->img_ref, p->img_sci, p->img_diff, p->img_mask, p->kap, p->d_int, p->ftab, p->ftab64, p->tw128,
                     p->segy ? p->twy : nullptr,
                     p->bxy64, p->d_zdesc, p->d_rdesc, p->z0, p->cmat, p->unk, p->gam, p->bnd};
@@ -390,8 +390,7 @@ int plan_new(const sfft_config *cfg, cudaStream_t s, Plan **out) {
     p->gpairs = p->pairs + np;
     SFFT_ALLOC(p->rowmom, (size_t)p->n0 * p->nmom * sizeof(double));
     SFFT_ALLOC(p->lag, nlag * sizeof(double));
-    SFFT_ALLOC(p->A, n * n * rsz);
-    SFFT_ALLOC(p->Wm, n * n * rsz);
+    SFFT_ALLOC(p->A, solve_matrix_elems((int)n, p->fp64) * rsz);
     p->solve_grid = solve_grid_size(p->fp64);
     p->solve_grid_tc = p->fp64 ? 0 : solve_grid_size(false, true);
     if (p->solve_grid <= 0 || p->solve_grid > kMaxSolveGrid) {

@@ -125,7 +125,8 @@ struct Plan {
     // tune_tc: 0 or 1 the solve's tile products on the CUDA cores, 2 on the
     // tensor cores (FP32 plans only; see solve.cu)
     int tune_tr, tune_gi, tune_ng, tune_sgrid, tune_tc;
-    // panel width of the FP32 blocked Cholesky: 32 (default) or 64 (solve.cu)
+    // panel width setting (32, the default, or 64): must agree within a batch;
+    // the factorisation takes 64-wide steps for both (solve.cu)
     int solve_panel;
     int sms;  // multiprocessors of the device the plan was created on
     // basis (see BasisView); the tables are built at plan creation
@@ -161,8 +162,7 @@ struct Plan {
     double *lag;           // lag tables (Omega, Lambda, Theta), FP64
     int lag_om, lag_la, lag_th;  // offsets into lag
     // solve workspace
-    void *A;               // n*n factor (compute type)
-    void *Wm;              // n*n: W = L^-1 (compute type)
+    void *A;               // the solve's tiles, panel and diagonal blocks (solve_matrix_elems, compute type)
     int solve_grid;        // blocks of the cooperative solve kernel
     int solve_grid_tc;     // blocks of its tensor-core variant (one per SM), 0 for FP64
     double *dscale;        // n Jacobi scales
@@ -237,13 +237,14 @@ cudaError_t solve_batch(Plan *const *plans, int count, const double *const *M, c
                         double *const *x, sfft_solve_info *const *info, cudaStream_t s);
 int solve_grid_size(bool fp64, bool tc = false);
 size_t solve_vec_elems(int n);
+size_t solve_matrix_elems(int n, bool fp64);
 // Solve workspace given by the caller instead of a plan (sizes for n
-// unknowns in the compute type: A, W n*n; zv solve_vec_elems(n); dsc, r n
+// unknowns in the compute type: A solve_matrix_elems(n); zv solve_vec_elems(n); dsc, r n
 // doubles; xw n + 8 + 2*grid doubles; flag 4 ints).
 struct SolveBuffers {
     int n, grid;
     bool fp64;
-    void *A, *W, *zv;
+    void *A, *zv;
     double *dsc, *r, *xw;
     int *flag;
 };

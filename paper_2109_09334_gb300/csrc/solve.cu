@@ -7,30 +7,44 @@
 //     r = rhs - M x (FP64),  x += D W^T W D r,
 // until ||r|| / ||rhs|| <= 1e-12.
 //
-// Everything runs in one cooperative (grid-synchronised) kernel with two
-// blocks per SM (FP32; one in FP64), so the ~n/NB dependent block steps cost
-// a grid barrier each instead of a kernel launch:
-//   * Cholesky, right-looking with NB-wide panels, NB = 32 (the default) or
-//     64 (per plan; fewer barriers and trailing passes, a longer chain per
-//     step: faster when several systems share a launch).  One block applies
-//     the last update to the next diagonal block itself, factors it right
-//     away and inverts the factor in the same sweep (factor_inv: eight steps
-//     of four columns per 32x32 block, exchanging through shared memory;
-//     factor64 builds the 64x64 block from two of them).  Phase P then forms
-//     the panel L_ik = A_ik L_kk^-T as 64xNB GEMM tiles; phase U applies
-//     A_ij -= L_ik L_jk^T to the trailing lower triangle in 64x64 tiles, on
-//     the CUDA cores or, in the FP32 variant that asks for it, on the tensor
-//     cores (tcgen05, 3xTF32 split; see tile_gemm_tc).
-//   * W = L^-1 is formed in the same sweep (block forward elimination applied
-//     to the identity): W_kk = L_kk^-1 from the diagonal factorisation, phase
-//     P sets W_k[:, 0:k0] = L_kk^-1 W_k[:, 0:k0] and phase U applies
-//     W_i -= L_ik W_k below.
+// Everything runs in one cooperative (grid-synchronised) kernel.  The
+// factorisation and the inverse are one in-place sweep over an array X of
+// TS x TS tiles (TS = 64 in FP32, 32 in FP64; rows padded to whole tiles, so
+// that every load is a whole vector): at step k the lower triangle of X holds
+// W in the block columns before k and the trailing A from there on.  A
+// step is
+//   * phase P: the panel of this step, TS rows over all columns c:
+//       P(:, c) = Dk X(k, c)          (c before block k: row block k of W),
+//       P(:, k) = Dk = L_kk^-1,
+//       P(:, c) = Dk X(c, k)^T        (c after block k: L_ck^T);
+//     row block k of X becomes its final W;
+//   * phase U: X(i, j) -= P(:, i)^T P(:, j) for every tile j <= i, i > k (the
+//     old values of block column k count as zero).  The same product updates
+//     the trailing A (j > k) and W (j <= k).
+// The arithmetic is that of 32-wide steps whatever TS: with TS = 64 a step is
+// two of them, Dk = [D1 0; * D2] stays in its 32 x 32 parts D1, D2 and L21,
+//     P1 = D1 X1,  P2 = D2 (X2 - L21 P1),
+// and phase U subtracts the products of the two halves one after the other.
+// Half the barriers and passes over X, the same roundings.
+// Meanwhile one block per system, which takes no tasks, forms the next
+// diagonal block from the tiles as the step found them: L_{k+1,k}, the last
+// update of X(k+1, k+1), its factor and the inverses of that.  It arrives at
+// the barrier between P and U as soon as it has read its two tiles and waits
+// there only when it is done, so that its chain runs beside both phases.
+//
+// What bounds it (n = 1735, 27 steps): one system alone by the step's latency
+// (the chain, or P, one to three rounds of tiles and two grid barriers);
+// eight systems by the tiles' FP32 products and their shared-memory reads.
+// One system 907 -> 545 us, eight of 507 to 1735 unknowns 1510 -> 947 us against
+// 32-wide steps with two whole-grid barriers, the chain inside phase U.
 //   * refinement: residual GEMV in FP64 and two GEMVs with W.
 // Every control decision after a barrier uses values written before it, so
 // all blocks execute the same sequence of barriers.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
+#include <limits.h>
 #include <math.h>
+
 
 #include "common.cuh"
 #include "internal.h"
@@ -39,152 +53,127 @@ namespace cg = cooperative_groups;
 
 namespace sfft {
 
-// Cholesky panel width NB (template parameter of the kernel): 32 or 64
-constexpr int kNBMax = 64;
-constexpr int kDB = 32;         // sub-block of the diagonal block factored in one sweep
-constexpr int kKC = 32;         // k chunk of a tile product staged at once
-constexpr int kTile = 64;       // trailing-update and GEMM output tile
+constexpr int kDB = 32;         // order of a block factored by one warp
+constexpr int kKC = 32;         // k chunk of a tensor-core tile product
+constexpr int kTile = 64;       // FP32 tile
 constexpr int kMaxIters = 12;   // refinement iterations
 constexpr double kTol = 1e-12;  // ||r|| / ||rhs||
 constexpr int kThreads = 256;
 constexpr int kBlocksPerSM = 2;  // resident FP32 solve blocks per SM (more loads in flight); FP64 takes 1
-constexpr int kSeg = 8;         // row segments of the W^T y product
+constexpr int kSeg = 8;        // row segments of the W^T y product
 constexpr int kWDepth32 = 16;   // FP32 loads in flight per lane in the products with W
 constexpr int kMaxBatch = kMaxSolveBatch;  // systems solved together by one launch
 
+// Tile edge TS (also the width of a step); R x R outputs per thread of a tile
+// product; KV values per 16-byte vector.  FP64 tiles are smaller because the FP64 units set their time: more
+// blocks share it.
+template <typename T>
+struct Shape {
+    static constexpr int TS = sizeof(T) == 4 ? kTile : kDB;
+    static constexpr int R = TS / 16;
+    static constexpr int KV = 16 / sizeof(T);
+    static constexpr int LDD = kDB + KV;         // pitch of a 32 x 32 block held by the chain
+    static constexpr int kDiag = TS == kDB ? 1 : 3;  // blocks of a diagonal block: D1, D2, L21
+};
+
 template <typename T>
 struct SolveArgs {
-    int n;
+    int n, ld;  // unknowns; rows and columns of X in whole tiles
     const double *M, *rhs;
     double *dsc, *x, *r, *stats;  // stats[0..3]
-    T *A, *W, *z, *y, *wseg;
-    int *flag;  // [0] status (0 running, 1 converged, <0 failure), [1] iterations
+    T *X, *P, *D;  // [ld][ld]; [TS][ld]; two buffers of a diagonal block, [kDiag][32][32]
+    T *z, *y, *wseg;
+    // [0] status (0 running, 1 converged, <0 failure), [1] iterations, [2]
+    // first diagonal block with a pivot that is not positive (INT_MAX: none)
+    int *flag;
     double *xout;
     sfft_solve_info *info;
 };
 
+// 16 bytes of T
 template <typename T>
-struct TileSmem {
-    T a[kTile][kKC + 1];  // a(i, p)
-    T b[kKC][kTile + 1];  // b(p, j)
+struct alignas(16) Vec {
+    T v[Shape<T>::KV];
 };
-
-// four consecutive values of shared memory (16-byte aligned)
-__device__ __forceinline__ void ld4(const float *p, float (&o)[4]) {
-    const float4 v = *reinterpret_cast<const float4 *>(p);
-    o[0] = v.x;
-    o[1] = v.y;
-    o[2] = v.z;
-    o[3] = v.w;
-}
-__device__ __forceinline__ void ld4(const double *p, double (&o)[4]) {
-    const double2 a = reinterpret_cast<const double2 *>(p)[0], b = reinterpret_cast<const double2 *>(p)[1];
-    o[0] = a.x;
-    o[1] = a.y;
-    o[2] = b.x;
-    o[3] = b.y;
-}
-
-// Operands of one 32-deep chunk of a 64x64 tile product, loaded into
-// registers (kLdOps elements of each per thread): all loads of a chunk are
-// in flight before the first store to shared memory.
-constexpr int kLdOps = kTile * kKC / kThreads;
 template <typename T>
-struct TileOps {
-    T ra[kLdOps], rb[kLdOps];
-};
-
-// chunk [kk, kk + kn) of the operands of tile_gemm (same a, b, bounds)
-template <bool TB, typename T>
-__device__ __forceinline__ void tile_load(TileOps<T> &o, const T *Ag, int lda, int arow0, int arows, const T *Bg,
-                                          int ldb, int bcol0, int bcols, int kk, int kn) {
-    const int tid = threadIdx.x;
-#pragma unroll
-    for (int q = 0; q < kLdOps; ++q) {
-        const int e = tid + q * kThreads, i = e / kKC, p = e % kKC;
-        o.ra[q] = (i < arows && p < kn) ? Ag[(size_t)(arow0 + i) * lda + kk + p] : (T)0;
-    }
-    if constexpr (TB) {
-#pragma unroll
-        for (int q = 0; q < kLdOps; ++q) {
-            const int e = tid + q * kThreads, j = e / kKC, p = e % kKC;
-            o.rb[q] = (j < bcols && p < kn) ? Bg[(size_t)(bcol0 + j) * ldb + kk + p] : (T)0;
-        }
-    } else {
-#pragma unroll
-        for (int q = 0; q < kLdOps; ++q) {
-            const int e = tid + q * kThreads, p = e / kTile, j = e % kTile;
-            o.rb[q] = (j < bcols && p < kn) ? Bg[(size_t)(kk + p) * ldb + bcol0 + j] : (T)0;
-        }
-    }
+__device__ __forceinline__ Vec<T> ldv(const T *p) {
+    return *reinterpret_cast<const Vec<T> *>(p);
 }
-
-// acc += the product of one loaded chunk: stage it in shared memory
-// (tile_stage), then each thread accumulates its 4x4 outputs (rows 4 tr + u,
-// columns tc + 16 v) over the 32 values of k in order (tile_compute).
-template <bool TB, typename T>
-__device__ __forceinline__ void tile_stage(TileSmem<T> &sm, const TileOps<T> &o) {
-    const int tid = threadIdx.x;
-#pragma unroll
-    for (int q = 0; q < kLdOps; ++q) {
-        const int e = tid + q * kThreads;
-        sm.a[e / kKC][e % kKC] = o.ra[q];
-        if constexpr (TB)
-            sm.b[e % kKC][e / kKC] = o.rb[q];
-        else
-            sm.b[e / kTile][e % kTile] = o.rb[q];
-    }
-    __syncthreads();
-}
-
 template <typename T>
-__device__ __forceinline__ void tile_compute(T (&acc)[4][4], const TileSmem<T> &sm) {
-    const int tid = threadIdx.x;
-    const int tr = tid / 16, tc = tid % 16;
+__device__ __forceinline__ void stv(T *p, const Vec<T> &v) {
+    *reinterpret_cast<Vec<T> *>(p) = v;
+}
+// from global memory, past L1 (other blocks wrote it in this launch)
+__device__ __forceinline__ Vec<float> ldg_cg(const float *p) {
+    const float4 f = __ldcg(reinterpret_cast<const float4 *>(p));
+    return {{f.x, f.y, f.z, f.w}};
+}
+__device__ __forceinline__ Vec<double> ldg_cg(const double *p) {
+    const double2 f = __ldcg(reinterpret_cast<const double2 *>(p));
+    return {{f.x, f.y}};
+}
+__device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(smem)),
+                 "l"(gmem));
+}
+
+// The thread's R x R outputs of a TS x TS tile start at (tile_row, tile_col):
+// a warp covers 8 x 4 threads, row and column bits interleaved in the lane
+// number, so that lanes 2 apart share their column vector and lanes 1 apart
+// their row vector.  Shared memory then delivers a half-warp's vectors in one
+// pass.
+template <typename T>
+__device__ __forceinline__ int tile_row() {
+    const int w = threadIdx.x >> 5, l = threadIdx.x;
+    return Shape<T>::R * ((w & 1) * 8 + (((l >> 1) & 1) | ((l >> 2) & 6)));
+}
+template <typename T>
+__device__ __forceinline__ int tile_col() {
+    const int w = threadIdx.x >> 5, l = threadIdx.x;
+    return Shape<T>::R * ((w >> 1) * 4 + ((l & 1) | ((l >> 1) & 2)));
+}
+
+// acc(u, v) = sum_p a[p][tile_row + u] b[p][tile_col + v], p < 32 in order, both
+// operands k-major with pitch TS
+template <typename T>
+__device__ __forceinline__ void tile_mul(T (&acc)[Shape<T>::R][Shape<T>::R], const T *a, const T *b) {
+    using S = Shape<T>;
+    const T *pa = a + tile_row<T>(), *pb = b + tile_col<T>();
+#pragma unroll
+    for (int u = 0; u < S::R; ++u)
+#pragma unroll
+        for (int v = 0; v < S::R; ++v) acc[u][v] = (T)0;
 #pragma unroll 8
-    for (int p = 0; p < kKC; ++p) {
-        T av[4], bv[4];
+    for (int p = 0; p < kDB; ++p) {
+        const Vec<T> av = ldv(pa + p * S::TS), bv = ldv(pb + p * S::TS);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) av[u] = sm.a[tr * 4 + u][p];
+        for (int u = 0; u < S::R; ++u)
 #pragma unroll
-        for (int v = 0; v < 4; ++v) bv[v] = sm.b[p][tc + 16 * v];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int v = 0; v < 4; ++v) acc[u][v] += av[u] * bv[v];
+            for (int v = 0; v < S::R; ++v) acc[u][v] += av.v[u] * bv.v[v];
     }
-    __syncthreads();
 }
 
-template <bool TB, typename T>
-__device__ __forceinline__ void tile_mul(T (&acc)[4][4], TileSmem<T> &sm, const TileOps<T> &o) {
-    tile_stage<TB>(sm, o);
-    tile_compute(acc, sm);
-}
-
-// 64x64 tile:  acc(i, j) += sum_{k0 <= k < k1} a(i, k) b(k, j)
-//   a(i, k) = Ag[(arow0 + i) * lda + k]
-//   b(k, j) = transB ? Bg[(bcol0 + j) * ldb + k] : Bg[k * ldb + bcol0 + j]
-// rows i >= arows and columns j >= bcols read as zero.  All loads of a
-// 32-deep chunk are issued before the first store to shared memory, so that
-// their latencies overlap.
-template <typename T>
-__device__ void tile_gemm(T (&acc)[4][4], TileSmem<T> &sm, const T *Ag, int lda, int arow0, int arows,
-                          const T *Bg, int ldb, int bcol0, int bcols, bool transB, int k0, int k1) {
-    for (int kk = k0; kk < k1; kk += kKC) {
-        TileOps<T> o;
-        if (transB) {
-            tile_load<true>(o, Ag, lda, arow0, arows, Bg, ldb, bcol0, bcols, kk, min(kKC, k1 - kk));
-            tile_mul<true>(acc, sm, o);
-        } else {
-            tile_load<false>(o, Ag, lda, arow0, arows, Bg, ldb, bcol0, bcols, kk, min(kKC, k1 - kk));
-            tile_mul<false>(acc, sm, o);
+// acc(v) = sum_p a[p * astep] b[p * bstep + v], p < 32 in order: a points at
+// this lane's row, b at this warp's NC columns
+template <typename T, int NC>
+__device__ __forceinline__ void lane_mul(T (&acc)[NC], const T *a, int astep, const T *b, int bstep) {
+    constexpr int KV = Shape<T>::KV;
+#pragma unroll
+    for (int v = 0; v < NC; ++v) acc[v] = (T)0;
+#pragma unroll 8
+    for (int p = 0; p < kDB; ++p) {
+        const T av = a[p * astep];
+#pragma unroll
+        for (int v = 0; v < NC; v += KV) {
+            const Vec<T> w = ldv(b + p * bstep + v);
+#pragma unroll
+            for (int i = 0; i < KV; ++i) acc[v + i] += av * w.v[i];
         }
     }
 }
 
 // ---- the FP32 tile GEMM on the tensor cores (tcgen05, sm_100 family) --------
-// The 64x64x32 tile products of the trailing update run as tcgen05.mma of
+// The tile products of phase U run, in chunks of 32 panel rows, as tcgen05.mma of
 // kind::tf32 (M = N = 64, K = 8 per instruction) with the accumulator in
 // tensor memory.  TF32 keeps 10 mantissa bits, too few for a factor that
 // must seed the FP64 refinement at a Jacobi-scaled condition number near
@@ -196,10 +185,10 @@ __device__ void tile_gemm(T (&acc)[4][4], TileSmem<T> &sm, const T *Ag, int lda,
 // K-major layout without swizzle: core matrices of 8 rows x 16 bytes, the
 // next core matrix along K at +128 bytes (leading byte offset), the next
 // 8-row group at +1024 bytes (stride byte offset, 32 K values per row).  One
-// elected thread issues the 12 MMAs of a tile and commits them to an
+// elected thread issues the 12 MMAs of a chunk and commits them to an
 // mbarrier; the block waits on it (bounded by a clock limit), reads the
 // accumulator back with tcgen05.ld and hands it to the caller in the
-// register layout of tile_gemm, through a shared transpose.  In tensor
+// register layout of tile_mul, through a shared transpose.  In tensor
 // memory an M = 64 accumulator holds row 16 q + l in lane 32 q + l (q < 4,
 // l < 16) and column j in column j.
 constexpr int kTcCols = 64;                    // tensor-memory columns per block
@@ -283,18 +272,18 @@ __device__ void tc_release(TcState &st) {
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(st.tmem), "n"(kTcCols));
 }
 
-// tile_gemm on the tensor cores for one chunk of at most kKC values of k
-// (k1 - k0 <= kKC), same operands and result layout.  Returns false if the
-// MMAs did not complete within the wait limit (acc is then not valid).
-__device__ bool tile_gemm_tc(float (&acc)[4][4], TcSmem &tc, TcState &st, const float *Ag, int lda, int arow0,
-                             int arows, const float *Bg, int ldb, int bcol0, int bcols, bool transB, int k0, int k1) {
-    constexpr int kLd = kLdOps;
-    const int tid = threadIdx.x, tr = tid / 16, tc16 = tid % 16;
-    const int kn = min(kKC, k1 - k0);
+// One chunk of kKC panel rows of a 64x64 tile product on the tensor cores:
+// acc(i, j) = sum_k P[k][i0 + i] P[k][j0 + j], k0 <= k < k0 + kKC, in the
+// thread layout of tile_mul.  Returns false if the MMAs did not complete
+// within the wait limit (acc is then not valid).
+__device__ bool tile_mul_tc(float (&acc)[4][4], TcSmem &tc, TcState &st, const float *P, int ld, int i0, int j0,
+                            int k0) {
+    constexpr int kLd = kTile * kKC / kThreads;
+    const int tid = threadIdx.x;
     // element e = tid + q * kThreads of a 64 x 32 operand is (row, k) with
     // the lane choosing (row mod 8, k mod 4) and the rest (row / 8, k / 4):
     // a warp then stores one whole core matrix (32 consecutive words, no
-    // bank conflict) and reads 8 rows x 16 bytes (or 4 k-rows x 32 bytes)
+    // bank conflict) and reads 4 k-rows x 32 bytes
     float ra[kLd], rb[kLd];
     int ri[kLd], rk[kLd];
 #pragma unroll
@@ -305,11 +294,9 @@ __device__ bool tile_gemm_tc(float (&acc)[4][4], TcSmem &tc, TcState &st, const 
     }
 #pragma unroll
     for (int q = 0; q < kLd; ++q) {
-        const int i = ri[q], pp = rk[q];
-        ra[q] = (i < arows && pp < kn) ? Ag[(size_t)(arow0 + i) * lda + k0 + pp] : 0.f;
-        rb[q] = (i < bcols && pp < kn)
-                    ? (transB ? Bg[(size_t)(bcol0 + i) * ldb + k0 + pp] : Bg[(size_t)(k0 + pp) * ldb + bcol0 + i])
-                    : 0.f;
+        const float *row = P + (size_t)(k0 + rk[q]) * ld + ri[q];
+        ra[q] = __ldcg(row + i0);
+        rb[q] = __ldcg(row + j0);
     }
 #pragma unroll
     for (int q = 0; q < kLd; ++q) {
@@ -378,325 +365,449 @@ __device__ bool tile_gemm_tc(float (&acc)[4][4], TcSmem &tc, TcState &st, const 
 #pragma unroll
     for (int u = 0; u < 4; ++u)
 #pragma unroll
-        for (int w = 0; w < 4; ++w) acc[u][w] = Cs[(tr * 4 + u) * (kTile + 1) + tc16 + 16 * w];
+        for (int w = 0; w < 4; ++w) acc[u][w] = Cs[(tile_row<float>() + u) * (kTile + 1) + tile_col<float>() + w];
     __syncthreads();  // the shared tiles are refilled by the next call
     return true;
 }
-
-// Shared memory of the diagonal-block factorisation (aliases the GEMM tiles):
-// four columns of S (by row) and four rows of Y (by column) per step,
-// double-buffered by step parity.
-template <typename T>
-struct __align__(16) FactorSmem {
-    T col[2][kDB][4];
-    T row[2][kDB][4];
-    T lp[kNBMax][kKC + 1];  // staged operands (panel rows of the last update; 32 x 32 products)
-    T s1[kDB][kDB + 1];  // L21
-    T s2[kDB][kDB + 1];  // L21 L11^-1
-};
-
-template <typename T>
-union SolveSmem {
-    TileSmem<T> tile;
-    FactorSmem<T> fac;
-    TcSmem tc;  // FP32 only (the tensor-core tile GEMM)
-};
-
-template <typename T>
-__device__ __forceinline__ T pick4(const T (&v)[4], int q) {
-    return q == 0 ? v[0] : (q == 1 ? v[1] : (q == 2 ? v[2] : v[3]));
-}
-
 // 1 / sqrt(d): the FP32 factor only seeds the FP64 refinement, so the
 // hardware approximation serves; FP64 takes the correctly rounded path.
-__device__ __forceinline__ float inv_sqrt(float d) { return rsqrtf(d); }
+__device__ __forceinline__ float inv_sqrt(float d) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+    return r;
+}
 __device__ __forceinline__ double inv_sqrt(double d) { return 1.0 / sqrt(d); }
 
-// The whole block factors the 32x32 block of A at (k0, k0) (nb <= 32 rows
-// inside the matrix) and inverts its factor in the same sweep, four columns
-// per step.  With kp >= 0 the block first applies the last update of that
-// block itself, S = A_kk - L L^T with L = A[k0:k0+32, kp:kp+32] (the panel
-// of a 32-wide step kp), in the operation order of the trailing-update
-// tiles; with kp < 0 A_kk is already fully updated.  Then:
-// every thread factors the 4x4 pivot block itself, forms the L entries of the
-// rows it needs by forward substitution, and applies the rank-4 update to S
-// and the matching block forward elimination to Y (L Y = I, so Y ends as
-// L^-1).  Thread (t, u) = (tid / 8, tid % 8) keeps row t, columns u, u+8,
-// u+16, u+24 of S and Y in registers; each step publishes the next four
-// columns of S and rows of Y through shared memory (one barrier per step).
-// Writes L_kk into A and L_kk^-1 into W (zeros above the diagonal) and flags
-// a non-positive pivot.
+// named barriers: 1..8 pass the steps of a factorisation from warp 0 to warp
+// 1, kBarHelp joins the helper warps of the chain; 0 is __syncthreads
+constexpr int kBarHelp = 9;
+__device__ __forceinline__ void bar_sync(int id, int threads) {
+    asm volatile("barrier.cta.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(int id, int threads) {
+    asm volatile("barrier.cta.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+// Two warps factor the 32x32 block A (lower triangle at s, pitch lds) and
+// invert its factor, four columns per step.  Warp 0: lane r holds row r of A;
+// every lane factors the 4x4 pivot block itself, and the four L entries of
+// each row pass through shared memory (ex: a vector per row, then the four
+// reciprocal pivots).  Warp 1 follows a step behind with the forward
+// elimination of the identity, column r of Y in lane r (L Y = I); Y(r, c) goes
+// to dt[c * ldd + r], zeros above the diagonal included.  Rows nb and up are
+// the identity's (the caller sets them); a pivot that is not positive sets
+// bad; minpiv takes the smallest of the rest.  Bound by the chain of pivots.
+// (5.2 k cycles; a whole block taking four columns a step, with a barrier and
+// an exchange each, took 12 k.)
+constexpr int kExStep = kDB * 4 + 4;
 template <typename T>
-__device__ void factor_inv(const SolveArgs<T> &s, FactorSmem<T> &f, int k0, int nb, int kp) {
-    const int tid = threadIdx.x;
-    const int n = s.n;
-    const int t = tid >> 3, u = tid & 7;
-    T sv[4], yv[4];
+__device__ __forceinline__ void get4(const T *p, T (&o)[4]) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int c = u + 8 * q;
-        T v = (T)0;
-        if (t < nb && c <= t) v = s.A[(size_t)(k0 + t) * n + k0 + c];  // the lower triangle only
-        else if (t == c) v = (T)1;  // identity beyond the matrix edge
-        sv[q] = v;
-        yv[q] = (t == c) ? (T)1 : (T)0;
+    for (int v = 0; v < 4; v += Shape<T>::KV) {
+        const Vec<T> w = ldv(p + v);
+#pragma unroll
+        for (int i = 0; i < Shape<T>::KV; ++i) o[v + i] = w.v[i];
     }
-    if (kp >= 0) {
+}
+template <typename T>
+__device__ __forceinline__ void put4(T *p, const T (&o)[4]) {
 #pragma unroll
-        for (int q = 0; q < kDB * kDB / kThreads; ++q) {
-            const int e = tid + q * kThreads, r = e / kDB, p = e % kDB;
-            f.lp[r][p] = r < nb ? s.A[(size_t)(k0 + r) * n + kp + p] : (T)0;
-        }
-        __syncthreads();
-        T acc[4] = {};
-#pragma unroll 8
-        for (int p = 0; p < kDB; ++p) {
-            const T a = f.lp[t][p];
+    for (int v = 0; v < 4; v += Shape<T>::KV) {
+        Vec<T> w;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) acc[q] += a * f.lp[u + 8 * q][p];
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            if (t < nb && u + 8 * q <= t) sv[q] = sv[q] - acc[q];
+        for (int i = 0; i < Shape<T>::KV; ++i) w.v[i] = o[v + i];
+        stv(p + v, w);
     }
-    if (u < 4) f.col[0][t][u] = sv[0];
-    if (t < 4) {
+}
+// L entries in columns jb..jb+3 of a row from its entries r there, by the
+// pivot block's L entries and reciprocal pivots
+template <typename T>
+__device__ __forceinline__ void lrow(const T (&r)[4], T i0, T i1, T i2, T i3, T l10, T l20, T l21, T l30, T l31, T l32,
+                                     T (&l)[4]) {
+    l[0] = r[0] * i0;
+    l[1] = (r[1] - l[0] * l10) * i1;
+    l[2] = (r[2] - l[0] * l20 - l[1] * l21) * i2;
+    l[3] = (r[3] - l[0] * l30 - l[1] * l31 - l[2] * l32) * i3;
+}
+
+template <typename T>
+__device__ __noinline__ void factor_rows(const T *s, int lds, T *ex, int nb, bool &bad, T &minpiv) {
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    T a[kDB], low = (T)1e30;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) f.row[0][u + 8 * q][t] = yv[q];
-    }
-    bool bad = false;
-    T minpiv = (T)1e30;
-    // unrolled: buffer indices, register picks and row tests become constants
-    // (one system 0.941 -> 0.912 ms at n = 1735)
+    for (int c = 0; c < kDB; ++c) a[c] = s[lane * lds + c];
 #pragma unroll
     for (int jb = 0; jb < kDB; jb += 4) {
-        __syncthreads();  // columns jb..jb+3 of S and rows jb..jb+3 of Y are published
-        const int b = (jb >> 2) & 1;
-        T p0[4], p1[4], p2[4], p3[4], st[4], sc[4][4], yc[4][4];
-        ld4(f.col[b][jb], p0);
-        ld4(f.col[b][jb + 1], p1);
-        ld4(f.col[b][jb + 2], p2);
-        ld4(f.col[b][jb + 3], p3);
-        ld4(f.col[b][t], st);
+        T pv[4][4];  // rows jb..jb+3 of the pivot block
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            ld4(f.col[b][u + 8 * q], sc[q]);
-            ld4(f.row[b][u + 8 * q], yc[q]);
-        }
-        // 4x4 Cholesky of the pivot block
-        const T d0 = p0[0];
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int c = 0; c <= r; ++c) pv[r][c] = __shfl_sync(kAll, a[jb + c], jb + r);
+        const T d0 = pv[0][0];
         const T i0 = inv_sqrt(d0 > (T)0 ? d0 : (T)1);
-        const T l10 = p1[0] * i0, l20 = p2[0] * i0, l30 = p3[0] * i0;
-        const T d1 = p1[1] - l10 * l10;
+        const T l10 = pv[1][0] * i0, l20 = pv[2][0] * i0, l30 = pv[3][0] * i0;
+        const T d1 = pv[1][1] - l10 * l10;
         const T i1 = inv_sqrt(d1 > (T)0 ? d1 : (T)1);
-        const T l21 = (p2[1] - l20 * l10) * i1, l31 = (p3[1] - l30 * l10) * i1;
-        const T d2 = p2[2] - l20 * l20 - l21 * l21;
+        const T l21 = (pv[2][1] - l20 * l10) * i1, l31 = (pv[3][1] - l30 * l10) * i1;
+        const T d2 = pv[2][2] - l20 * l20 - l21 * l21;
         const T i2 = inv_sqrt(d2 > (T)0 ? d2 : (T)1);
-        const T l32 = (p3[2] - l30 * l20 - l31 * l21) * i2;
-        const T d3 = p3[3] - l30 * l30 - l31 * l31 - l32 * l32;
+        const T l32 = (pv[3][2] - l30 * l20 - l31 * l21) * i2;
+        const T d3 = pv[3][3] - l30 * l30 - l31 * l31 - l32 * l32;
         const T i3 = inv_sqrt(d3 > (T)0 ? d3 : (T)1);
+        const T r[4] = {a[jb], a[jb + 1], a[jb + 2], a[jb + 3]};
+        T lt[4];
+        lrow(r, i0, i1, i2, i3, l10, l20, l21, l30, l31, l32, lt);
+        T *e = ex + (jb >> 2) * kExStep;
+        put4(e + lane * 4, lt);
+        if (lane == 0) {
+            const T iv[4] = {i0, i1, i2, i3};
+            put4(e + kDB * 4, iv);
+        }
+        __syncwarp();
+        bar_arrive(1 + (jb >> 2), 64);
         const T dp[4] = {d0, d1, d2, d3};
 #pragma unroll
         for (int p = 0; p < 4; ++p) {
             if (!(dp[p] > (T)0)) bad = true;
-            if (jb + p < nb && dp[p] < minpiv) minpiv = dp[p];
+            if (jb + p < nb && dp[p] < low) low = dp[p];
         }
-        // L entries in columns jb..jb+3 of a row from its S entries there
-        auto lrow = [&](const T (&r)[4], T (&l)[4]) {
-            l[0] = r[0] * i0;
-            l[1] = (r[1] - l[0] * l10) * i1;
-            l[2] = (r[2] - l[0] * l20 - l[1] * l21) * i2;
-            l[3] = (r[3] - l[0] * l30 - l[1] * l31 - l[2] * l32) * i3;
-        };
-        T lt[4];
-        lrow(st, lt);  // row t of L (entries right of the diagonal are not used)
-        if (u < 4 && t < nb && jb + u < nb)
-            s.A[(size_t)(k0 + t) * n + k0 + jb + u] = (t >= jb + u) ? pick4(lt, u) : (T)0;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int c = u + 8 * q;
-            // rows jb..jb+3 of X = L^-1 in column c: block forward substitution
-            T x[4];
-            lrow(yc[q], x);
-            if (t >= jb && t < jb + 4 && c <= t && t < nb && c < nb)
-                s.W[(size_t)(k0 + t) * n + k0 + c] = pick4(x, t - jb);
-            if (t > jb + 3) {
-                if (c > jb + 3 && c <= t) {
-                    T lc[4];
-                    lrow(sc[q], lc);
-                    sv[q] -= lt[0] * lc[0] + lt[1] * lc[1] + lt[2] * lc[2] + lt[3] * lc[3];
-                }
-                if (c <= jb + 3) yv[q] -= lt[0] * x[0] + lt[1] * x[1] + lt[2] * x[2] + lt[3] * x[3];
-            }
-        }
-        // publish columns jn..jn+3 of S and rows jn..jn+3 of Y (the other buffer)
-        const int jn = jb + 4;
-        if (jn < kDB) {
-            const int u0 = jn & 7;
-            if (u >= u0 && u < u0 + 4) f.col[b ^ 1][t][u - u0] = pick4(sv, jn >> 3);
-            if (t >= jn && t < jn + 4) {
-#pragma unroll
-                for (int q = 0; q < 4; ++q) f.row[b ^ 1][u + 8 * q][t - jn] = yv[q];
-            }
+        for (int c = jb + 4; c < kDB; ++c) {
+            T lc[4];
+            get4(e + c * 4, lc);
+            a[c] -= lt[0] * lc[0] + lt[1] * lc[1] + lt[2] * lc[2] + lt[3] * lc[3];
         }
     }
-    // zeros above the diagonal of both blocks
+    if (!bad && low < minpiv) minpiv = low;
+}
+template <typename T>
+__device__ __noinline__ void invert_rows(const T *ex, T *dt, int ldd) {
+    const int lane = threadIdx.x & 31;
+    T y[kDB];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int c = u + 8 * q;
-        if (c > t && t < nb && c < nb) {
-            s.A[(size_t)(k0 + t) * n + k0 + c] = (T)0;
-            s.W[(size_t)(k0 + t) * n + k0 + c] = (T)0;
+    for (int c = 0; c < kDB; ++c) y[c] = c == lane ? (T)1 : (T)0;
+#pragma unroll
+    for (int jb = 0; jb < kDB; jb += 4) {
+        const T *e = ex + (jb >> 2) * kExStep;
+        bar_sync(1 + (jb >> 2), 64);
+        T iv[4], l1[4], l2[4], l3[4], x[4];
+        get4(e + kDB * 4, iv);
+        get4(e + (jb + 1) * 4, l1);
+        get4(e + (jb + 2) * 4, l2);
+        get4(e + (jb + 3) * 4, l3);
+        const T r[4] = {y[jb], y[jb + 1], y[jb + 2], y[jb + 3]};
+        lrow(r, iv[0], iv[1], iv[2], iv[3], l1[0], l2[0], l2[1], l3[0], l3[1], l3[2], x);
+        put4(dt + lane * ldd + jb, x);
+#pragma unroll
+        for (int c = jb + 4; c < kDB; ++c) {
+            T lc[4];
+            get4(e + c * 4, lc);
+            y[c] -= lc[0] * x[0] + lc[1] * x[1] + lc[2] * x[2] + lc[3] * x[3];
         }
     }
-    if (tid == 0) {
-        if (bad) s.flag[0] = SFFT_ERR_SINGULAR;
-        else if ((double)minpiv < s.stats[0]) s.stats[0] = (double)minpiv;
+}
+
+// Shared memory of the block that forms the diagonal blocks of its system.
+// d is kept from step to step: [q][p] of D1(p, q), and for TS = 64 of
+// D2(p, q) and L21(p, q).
+template <typename T>
+struct ChainSmem {
+    using S = Shape<T>;
+    T d[S::kDiag][kDB * S::LDD];
+    T d1[kDB * S::LDD];  // the new D1 while the old one is in use
+    T xt[S::TS * S::TS];  // X(k+1, k) by columns
+    T lt[S::TS * S::TS];  // L_{k+1,k} by columns
+    T ex[8 * kExStep];
+    T s[S::TS * (S::TS + 1)];  // X(k+1, k+1) by rows
+};
+
+// 32 rows (from row r0; a lane each) and this warp's NC columns from c0 of the
+// products that give L_{k+1,k}, each followed by sync()
+template <typename T, int NC, typename F>
+__device__ __forceinline__ void chain_panel(ChainSmem<T> &c, int r0, int c0, F sync) {
+    using S = Shape<T>;
+    constexpr int TS = S::TS, LDD = S::LDD;
+    const int i = r0 + (threadIdx.x & 31);
+    T o[NC];
+    lane_mul<T, NC>(o, c.xt + i, TS, c.d[0] + c0, LDD);  // L1(i, p) = sum_q X1(i, q) D1(p, q)
+#pragma unroll
+    for (int v = 0; v < NC; ++v) c.lt[(c0 + v) * TS + i] = o[v];
+    sync();
+    if constexpr (TS == 2 * kDB) {
+        T *x2 = c.xt + kDB * TS;
+        lane_mul<T, NC>(o, c.lt + i, TS, c.d[2] + c0, LDD);  // X2 -= L1 L21^T
+#pragma unroll
+        for (int v = 0; v < NC; ++v) x2[(c0 + v) * TS + i] -= o[v];
+        sync();
+        lane_mul<T, NC>(o, x2 + i, TS, c.d[1] + c0, LDD);  // L2 = X2 D2^T
+#pragma unroll
+        for (int v = 0; v < NC; ++v) c.lt[(kDB + c0 + v) * TS + i] = o[v];
+        sync();
     }
+}
+// the same rows and columns (from j0) of the diagonal block's last update
+template <typename T, int NC>
+__device__ __forceinline__ void chain_update(ChainSmem<T> &c, int r0, int j0) {
+    using S = Shape<T>;
+    constexpr int TS = S::TS, LDS = TS + 1;
+    const int i = r0 + (threadIdx.x & 31);
+    T *s = c.s + i * LDS + j0;
+#pragma unroll
+    for (int h = 0; h < TS / kDB; ++h) {
+        const T *l = c.lt + h * kDB * TS;
+        T o[NC];
+        lane_mul<T, NC>(o, l + i, TS, l + j0, TS);
+#pragma unroll
+        for (int v = 0; v < NC; ++v) s[v] -= o[v];
+    }
+}
+
+// Forms diagonal block kb: with `update` its last update from step kb - 1
+// (whose blocks are in c.d) first; then its own blocks into c.d and
+// s.D[kb & 1].  arrive() is called once both tiles have been read.  The first
+// 32 rows go first; warps 4..7 update the other rows while warps 0 and 1
+// factor.
+template <typename T, typename F>
+__device__ __forceinline__ void chain_block(const SolveArgs<T> &s, ChainSmem<T> &c, int kb, bool update, bool &bad,
+                                            T &minpiv, F arrive) {
+    using S = Shape<T>;
+    constexpr int TS = S::TS, KV = S::KV, LDD = S::LDD, LDS = TS + 1, NV = TS * TS / KV / kThreads, VR = TS / KV;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int k0 = kb * TS, nb = min(TS, s.n - k0), ld = s.ld;
+    Vec<T> sv[NV], xv[NV];
+    if (update) {
+#pragma unroll
+        for (int q = 0; q < NV; ++q) {
+            const int e = tid + q * kThreads, i = e % TS, g = e / TS;
+            xv[q] = ldg_cg(s.X + (size_t)(k0 + i) * ld + k0 - TS + g * KV);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+        const int e = tid + q * kThreads;
+        sv[q] = ldg_cg(s.X + (size_t)(k0 + e / VR) * ld + k0 + (e % VR) * KV);
+    }
+    if (update) {
+#pragma unroll
+        for (int q = 0; q < NV; ++q) {
+            const int e = tid + q * kThreads, i = e % TS, g = e / TS;
+#pragma unroll
+            for (int v = 0; v < KV; ++v) c.xt[(g * KV + v) * TS + i] = xv[q].v[v];
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+        const int e = tid + q * kThreads, r = e / VR, j = (e % VR) * KV;
+#pragma unroll
+        for (int v = 0; v < KV; ++v) c.s[r * LDS + j + v] = r < nb ? sv[q].v[v] : (r == j + v ? (T)1 : (T)0);
+    }
+    __syncthreads();
+    arrive();
+    if (update) {
+        chain_panel<T, 4>(c, 0, 4 * warp, [] { __syncthreads(); });
+        chain_update<T, 4>(c, 0, 4 * warp);
+        __syncthreads();
+    }
+    if (warp == 0) factor_rows<T>(c.s, LDS, c.ex, nb, bad, minpiv);
+    else if (warp == 1) invert_rows<T>(c.ex, c.d1, LDD);  // (the other warps still read the old D1)
+    if constexpr (TS == 2 * kDB) {
+        if (update && warp >= 4) {
+            chain_panel<T, 8>(c, kDB, 8 * (warp - 4), [] { bar_sync(kBarHelp, 128); });
+            chain_update<T, 8>(c, kDB, 8 * (warp - 4));
+            chain_update<T, 8>(c, kDB, kDB + 8 * (warp - 4));
+        }
+    }
+    __syncthreads();
+    for (int e = tid; e < kDB * LDD / KV; e += kThreads) stv(c.d[0] + e * KV, ldv(c.d1 + e * KV));
+    if constexpr (TS == 2 * kDB) {
+        T w[4];
+        lane_mul<T, 4>(w, c.s + (kDB + lane) * LDS, 1, c.d1 + 4 * warp, LDD);  // L21 = A21 D1^T
+#pragma unroll
+        for (int v = 0; v < 4; ++v) c.d[2][(4 * warp + v) * LDD + lane] = w[v];
+        __syncthreads();
+        lane_mul<T, 4>(w, c.d[2] + lane, LDD, c.d[2] + 4 * warp, LDD);  // A22 -= L21 L21^T
+#pragma unroll
+        for (int v = 0; v < 4; ++v) c.s[(kDB + lane) * LDS + kDB + 4 * warp + v] -= w[v];
+        __syncthreads();
+        if (warp == 0) factor_rows<T>(c.s + kDB * LDS + kDB, LDS, c.ex, nb - kDB, bad, minpiv);
+        else if (warp == 1) invert_rows<T>(c.ex, c.d[1], LDD);
+        __syncthreads();
+    }
+    if constexpr (TS == kDB) __syncthreads();
+    T *D = s.D + (size_t)(kb & 1) * S::kDiag * kDB * kDB;
+    for (int e = tid; e < S::kDiag * kDB * kDB / KV; e += kThreads) {
+        const int q = e / (kDB / KV), g = e % (kDB / KV);
+        stv(D + q * kDB + g * KV, ldv(c.d[0] + q * LDD + g * KV));
+    }
+    if (tid == 0 && bad && s.flag[2] > kb) s.flag[2] = kb;
     __syncthreads();
 }
 
-// 32x32 block product in the thread layout of factor_inv (thread (t, u)
-// holds row t, columns u + 8 q): out(t, c) = sum_{p < 32} a(t, p) b(p, c),
-// a at f.lp[0..31][p], b at f.lp[32 + p][c], accumulated over p in order.
+// Phase P task: 32 columns of the panel of step kb (column `lane` and rows
+// 4 warp + v per thread).
 template <typename T>
-__device__ __forceinline__ void mm32(const FactorSmem<T> &f, T (&out)[4]) {
-    const int tid = threadIdx.x, t = tid >> 3, u = tid & 7;
+struct PanelSmem {
+    T d[Shape<T>::kDiag][kDB * kDB];
+    T x[Shape<T>::TS][kDB];  // X1, X2: the chunk's rows q of X(k, :), or its columns of X(:, k)
+    T p1[kDB][kDB];
+};
+template <typename T>
+__device__ __forceinline__ void panel_task(const SolveArgs<T> &s, PanelSmem<T> &sm, int kb, int task) {
+    using S = Shape<T>;
+    constexpr int TS = S::TS, KV = S::KV, H = TS / kDB, VR = kDB / KV;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, ld = s.ld;
+    const int k0 = kb * TS, c0 = task * kDB;
+    const T *D = s.D + (size_t)(kb & 1) * S::kDiag * kDB * kDB;
+    constexpr int ND = S::kDiag * kDB * kDB / KV / kThreads, NX = TS * kDB / KV / kThreads;
+    Vec<T> dv[ND], xv[NX];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) out[q] = (T)0;
-#pragma unroll 8
-    for (int p = 0; p < kDB; ++p) {
-        const T a = f.lp[t][p];
+    for (int q = 0; q < ND; ++q) dv[q] = ldg_cg(D + (size_t)(tid + q * kThreads) * KV);
+    const int half = (c0 - k0) / kDB;  // of the diagonal block (diag)
+    const bool diag = c0 >= k0 && c0 < k0 + TS;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) out[q] += a * f.lp[kDB + p][u + 8 * q];
+    for (int q = 0; q < NX; ++q) {
+        const int e = tid + q * kThreads;
+        if (diag) xv[q] = {};
+        else
+            xv[q] = c0 < k0 ? ldg_cg(s.X + (size_t)(k0 + e / VR) * ld + c0 + (e % VR) * KV)
+                            : ldg_cg(s.X + (size_t)(c0 + lane) * ld + k0 + (e / kDB) * KV);
     }
-}
-
-// The 64x64 diagonal block kb: with kp >= 0 the block first applies its last
-// update A_kk -= L L^T, L = A[k0:k0+64, kp:kp+64] (the panel of step kp, two
-// chunks of 32 in order, as the trailing-update tiles), to its lower
-// triangle.  Then, with [L11 0; L21 L22] its factor,
-//   L11 (factor_inv), L21 = A21 L11^-T, A22 -= L21 L21^T, L22 (factor_inv),
-//   W21 = -L22^-1 (L21 L11^-1),
-// so that W_kk = [L11^-1 0; W21 L22^-1] = L_kk^-1.  L_kk goes into A, L_kk^-1
-// into W (zeros above the diagonal of both, over the whole 64x64 block).
-template <typename T>
-__device__ void factor64(const SolveArgs<T> &s, FactorSmem<T> &f, int kb, int kp) {
-    constexpr int kNB = 64;
-    const int tid = threadIdx.x, n = s.n;
-    const int k0 = kb * kNB, nb = min(kNB, n - k0);
-    if (kp >= 0) {
-        const int tr = tid / 16, tc = tid % 16;  // rows 4 tr + a, columns tc + 16 v
-        T acc[4][4] = {};
-        for (int kc = 0; kc < kNB; kc += kKC) {
-            for (int e = tid; e < kNB * kKC; e += kThreads) {
-                const int r = e / kKC, p = e % kKC;
-                f.lp[r][p] = r < nb ? s.A[(size_t)(k0 + r) * n + kp + kc + p] : (T)0;
-            }
-            __syncthreads();
-#pragma unroll 8
-            for (int p = 0; p < kKC; ++p) {
-                T av[4], bv[4];
+    __syncthreads();  // the reads of the task before are done
 #pragma unroll
-                for (int a = 0; a < 4; ++a) av[a] = f.lp[tr * 4 + a][p];
+    for (int q = 0; q < ND; ++q) stv(sm.d[0] + (tid + q * kThreads) * KV, dv[q]);
 #pragma unroll
-                for (int v = 0; v < 4; ++v) bv[v] = f.lp[tc + 16 * v][p];
+    for (int q = 0; q < NX; ++q) {
+        const int e = tid + q * kThreads;
+        if (c0 < k0 || diag) {
+            stv(&sm.x[0][0] + e * KV, xv[q]);
+        } else {
 #pragma unroll
-                for (int a = 0; a < 4; ++a)
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) acc[a][v] += av[a] * bv[v];
-            }
-            __syncthreads();
+            for (int v = 0; v < KV; ++v) sm.x[(e / kDB) * KV + v][lane] = xv[q].v[v];
         }
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                const int r = tr * 4 + a, c = tc + 16 * v;
-                if (r < nb && c <= r) {
-                    T *p = s.A + (size_t)(k0 + r) * n + k0 + c;
-                    *p = *p - acc[a][v];
-                }
-            }
-        __syncthreads();  // the updated block is visible to the whole block
     }
-    factor_inv(s, f, k0, min(kDB, nb), -1);
-    const int n2 = nb - kDB;
-    if (n2 <= 0) return;
-    const int t = tid >> 3, u = tid & 7;
+    __syncthreads();
     T o[4];
-    // L21 = A21 L11^-T: a(i, p) = A[k0+32+i][k0+p], b(p, c) = L11^-1[c][p]
-    for (int e = tid; e < kDB * kDB; e += kThreads) {
-        const int r = e / kDB, c = e % kDB;
-        f.lp[r][c] = r < n2 ? s.A[(size_t)(k0 + kDB + r) * n + k0 + c] : (T)0;
-        f.lp[kDB + r][c] = s.W[(size_t)(k0 + c) * n + k0 + r];
-    }
-    __syncthreads();
-    mm32(f, o);
+    auto store = [&](int row) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int c = u + 8 * q;
-        f.s1[t][c] = t < n2 ? o[q] : (T)0;
-        if (t < n2) s.A[(size_t)(k0 + kDB + t) * n + k0 + c] = o[q];
-    }
-    __syncthreads();
-    // A22 -= L21 L21^T (lower triangle)
-    for (int e = tid; e < kDB * kDB; e += kThreads) {
-        const int r = e / kDB, c = e % kDB;
-        f.lp[r][c] = f.s1[r][c];
-        f.lp[kDB + r][c] = f.s1[c][r];
-    }
-    __syncthreads();
-    mm32(f, o);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int c = u + 8 * q;
-        if (t < n2 && c <= t) {
-            T *p = s.A + (size_t)(k0 + kDB + t) * n + k0 + kDB + c;
-            *p = *p - o[q];
+        for (int v = 0; v < 4; ++v) {
+            const int p = row + 4 * warp + v;
+            s.P[(size_t)p * ld + c0 + lane] = o[v];
+            if (c0 < k0 + TS) s.X[(size_t)(k0 + p) * ld + c0 + lane] = o[v];
         }
-    }
-    __syncthreads();
-    factor_inv(s, f, k0 + kDB, n2, -1);
-    // X = L21 L11^-1, then W21 = -L22^-1 X
-    for (int e = tid; e < kDB * kDB; e += kThreads) {
-        const int r = e / kDB, c = e % kDB;
-        f.lp[r][c] = f.s1[r][c];
-        f.lp[kDB + r][c] = s.W[(size_t)(k0 + r) * n + k0 + c];
-    }
-    __syncthreads();
-    mm32(f, o);
+    };
+    // P1 = D1 X1; D1 itself in its own columns, zero in those of the second half
+    if (!diag) {
+        lane_mul<T, 4>(o, &sm.x[0][lane], kDB, sm.d[0] + 4 * warp, kDB);
+    } else {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) f.s2[t][u + 8 * q] = o[q];
-    __syncthreads();
-    for (int e = tid; e < kDB * kDB; e += kThreads) {
-        const int r = e / kDB, c = e % kDB;
-        f.lp[r][c] = (r < n2 && c < n2) ? s.W[(size_t)(k0 + kDB + r) * n + k0 + kDB + c] : (T)0;
-        f.lp[kDB + r][c] = f.s2[r][c];
+        for (int v = 0; v < 4; ++v) o[v] = half == 0 ? sm.d[0][lane * kDB + 4 * warp + v] : (T)0;
     }
-    __syncthreads();
-    mm32(f, o);
+    store(0);
+    if constexpr (H == 2) {
+        // P2 = D2 (X2 - L21 P1), X2 = 0 in the columns of the first half; D2 in its own
+        if (!diag || half == 0) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int c = u + 8 * q;
-        if (t < n2) s.W[(size_t)(k0 + kDB + t) * n + k0 + c] = -o[q];
-        // above the diagonal: the upper-right quadrant of both blocks
-        if (c < n2) {
-            s.A[(size_t)(k0 + t) * n + k0 + kDB + c] = (T)0;
-            s.W[(size_t)(k0 + t) * n + k0 + kDB + c] = (T)0;
+            for (int v = 0; v < 4; ++v) sm.p1[4 * warp + v][lane] = o[v];
+            __syncthreads();
+            lane_mul<T, 4>(o, &sm.p1[0][lane], kDB, sm.d[2] + 4 * warp, kDB);
+#pragma unroll
+            for (int v = 0; v < 4; ++v) sm.x[kDB + 4 * warp + v][lane] -= o[v];
+            __syncthreads();
+            lane_mul<T, 4>(o, &sm.x[kDB][lane], kDB, sm.d[1] + 4 * warp, kDB);
+        } else {
+#pragma unroll
+            for (int v = 0; v < 4; ++v) o[v] = sm.d[1][lane * kDB + 4 * warp + v];
         }
+        store(kDB);
     }
-    __syncthreads();
 }
 
-// diagonal block kb of an NB-wide factorisation, with the last update from
-// the panel at column kp (kp < 0: none)
-template <int NB, typename T>
-__device__ __forceinline__ void factor_block(const SolveArgs<T> &s, FactorSmem<T> &f, int kb, int kp) {
-    if constexpr (NB == kDB)
-        factor_inv(s, f, kb * kDB, min(kDB, s.n - kb * kDB), kp);
-    else
-        factor64(s, f, kb, kp);
+// Phase U: the tiles (i, j), kb < i < blocks, j <= i, in row order, without
+// the next diagonal block (kb + 1, kb + 1), which its chain forms.
+__device__ __forceinline__ int tile_count(int blocks, int kb) {
+    return blocks * (blocks + 1) / 2 - (kb + 1) * (kb + 2) / 2 - 1;
+}
+__device__ __forceinline__ void tile_of(int kb, int task, int &i, int &j) {
+    const int t = task + (kb + 1) * (kb + 2) / 2 + (task > kb ? 1 : 0);  // index in the whole lower triangle
+    i = (int)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
+    if (i * (i + 1) / 2 > t) --i;
+    if ((i + 1) * (i + 2) / 2 <= t) ++i;
+    j = t - i * (i + 1) / 2;
+}
+
+template <typename T>
+struct UpdateSmem {
+    T a[2][Shape<T>::TS * Shape<T>::TS];  // P(:, i) and P(:, j) of a tile, two tiles
+    T b[2][Shape<T>::TS * Shape<T>::TS];
+};
+
+template <typename T>
+union __align__(1024) SolveSmem {
+    ChainSmem<T> chain;
+    PanelSmem<T> panel;
+    UpdateSmem<T> upd;
+    TcSmem tc;  // FP32 only (the tensor-core tile product)
+    T red[kThreads / 32][32];
+};
+
+template <typename T>
+__device__ __forceinline__ void tile_old(const SolveArgs<T> &s, int kb, int i, int j,
+                                         T (&old)[Shape<T>::R][Shape<T>::R]) {
+    using S = Shape<T>;
+    const T *C = s.X + (size_t)(i * S::TS + tile_row<T>()) * s.ld + j * S::TS + tile_col<T>();
+#pragma unroll
+    for (int u = 0; u < S::R; ++u)
+#pragma unroll
+        for (int v = 0; v < S::R; v += S::KV) {
+            Vec<T> t = {};
+            if (j != kb) t = ldg_cg(C + (size_t)u * s.ld + v);
+#pragma unroll
+            for (int q = 0; q < S::KV; ++q) old[u][v + q] = t.v[q];
+        }
+}
+// old -= the product of the panel rows, 32 at a time
+template <typename T>
+__device__ __forceinline__ void tile_update(T (&old)[Shape<T>::R][Shape<T>::R], const T *a, const T *b) {
+    using S = Shape<T>;
+#pragma unroll
+    for (int h = 0; h < S::TS / kDB; ++h) {
+        T acc[S::R][S::R];
+        tile_mul(acc, a + h * kDB * S::TS, b + h * kDB * S::TS);
+#pragma unroll
+        for (int u = 0; u < S::R; ++u)
+#pragma unroll
+            for (int v = 0; v < S::R; ++v) old[u][v] -= acc[u][v];
+    }
+}
+template <typename T>
+__device__ __forceinline__ void tile_store(const SolveArgs<T> &s, int i, int j,
+                                           const T (&val)[Shape<T>::R][Shape<T>::R]) {
+    using S = Shape<T>;
+    T *C = s.X + (size_t)(i * S::TS + tile_row<T>()) * s.ld + j * S::TS + tile_col<T>();
+#pragma unroll
+    for (int u = 0; u < S::R; ++u)
+#pragma unroll
+        for (int v = 0; v < S::R; v += S::KV) {
+            Vec<T> t;
+#pragma unroll
+            for (int q = 0; q < S::KV; ++q) t.v[q] = val[u][v + q];
+            stv(C + (size_t)u * s.ld + v, t);
+        }
+}
+
+// asynchronous copies of the operands of tile (i, j) into shared memory
+template <typename T>
+__device__ __forceinline__ void tile_fetch(const SolveArgs<T> &s, T *a, T *b, int i, int j) {
+    using S = Shape<T>;
+    constexpr int VR = S::TS / S::KV;  // vectors per row
+#pragma unroll
+    for (int q = 0; q < S::TS * VR / kThreads; ++q) {
+        const int e = threadIdx.x + q * kThreads, p = e / VR, g = (e % VR) * S::KV;
+        const T *row = s.P + (size_t)p * s.ld + g;
+        cp_async16(a + p * S::TS + g, row + i * S::TS);
+        cp_async16(b + p * S::TS + g, row + j * S::TS);
+    }
 }
 
 // pairwise sum of D partial sums (D a power of two) in a fixed order:
@@ -710,246 +821,94 @@ __device__ __forceinline__ T tree_sum(T (&acc)[D]) {
     return acc[0];
 }
 
-// sum_{j < len} a[j] b[j] by one warp (lane = this thread's lane), with
-// D independent loads of each operand in flight; the result is reduced
-// across the warp (every lane returns it).
+// sum_{j < len} a[j] b[j] by one warp (lane = this thread's lane): D partial
+// sums per lane over its elements in rounds of D, what is left of an
+// incomplete round in the first, added pairwise and across the warp (every
+// lane returns it).  The loads of the next round are in flight during the
+// products of one (the residual at n = 1735: 14.8 -> 11.6 us).
 template <typename T, typename V, int D = 8>
 __device__ __forceinline__ T dot_warp(const T *a, const V *b, int lane, int len) {
-    T acc[D];
+    T acc[D], av[D], bv[D];
 #pragma unroll
     for (int q = 0; q < D; ++q) acc[q] = (T)0;
-    int j = lane;
-    for (; j + (D - 1) * 32 < len; j += D * 32) {
-        T av[D], bv[D];
+    auto fetch = [&](int j, T (&x)[D], T (&y)[D]) {
 #pragma unroll
         for (int q = 0; q < D; ++q) {
-            av[q] = a[j + 32 * q];
-            bv[q] = (T)b[j + 32 * q];
+            const bool in = j + 32 * q < len;
+            x[q] = in ? a[j + 32 * q] : (T)0;
+            y[q] = in ? (T)b[j + 32 * q] : (T)0;
+        }
+    };
+    fetch(lane, av, bv);
+    for (int j = lane; j - lane < len; j += D * 32) {
+        T an[D], bn[D];
+        fetch(j + D * 32, an, bn);
+        if (j + (D - 1) * 32 < len) {
+#pragma unroll
+            for (int q = 0; q < D; ++q) acc[q] += av[q] * bv[q];
+        } else {
+#pragma unroll
+            for (int q = 0; q < D; ++q)
+                if (j + 32 * q < len) acc[0] += av[q] * bv[q];
         }
 #pragma unroll
-        for (int q = 0; q < D; ++q) acc[q] += av[q] * bv[q];
+        for (int q = 0; q < D; ++q) {
+            av[q] = an[q];
+            bv[q] = bn[q];
+        }
     }
-    for (; j < len; j += 32) acc[0] += a[j] * (T)b[j];
     T r = tree_sum<T, D>(acc);
     for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
     return r;
 }
 
-// sum_{k0 <= k < k1} W[k][i] y[k] by one thread, D rows in flight
-template <typename T, int D = 8>
-__device__ __forceinline__ T col_dot(const T *W, const T *y, int n, int i, int k0, int k1) {
-    T acc[D];
+// sum_{k0 <= k < k1} W[k][i] y[k] by the block for 32 columns i (one per
+// lane): D partial sums over the rows k = q mod D, the remaining rows in the
+// first, added pairwise in a fixed order.  The warps share the partial sums,
+// eight rows of each in flight.  Valid in warp 0.
+template <typename T, int D>
+__device__ __forceinline__ T col_dot(const T *W, const T *y, int ld, int i, int k0, int k1, T (*red)[32]) {
+    constexpr int NW = kThreads / 32, P = D / NW;  // partial sums per warp
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int len = max(0, k1 - k0), m = len / D;
+    T acc[P];
 #pragma unroll
-    for (int q = 0; q < D; ++q) acc[q] = (T)0;
-    int k = k0;
-    for (; k + D - 1 < k1; k += D) {
-        T wv[D], yv[D];
+    for (int q = 0; q < P; ++q) acc[q] = (T)0;
+    const T *Wc = W + (size_t)(k0 + P * warp) * ld + i, *yc = y + k0 + P * warp;
+    for (int j = 0; j < m; j += 8) {
+        T wv[8][P], yv[8][P];
 #pragma unroll
-        for (int q = 0; q < D; ++q) {
-            wv[q] = W[(size_t)(k + q) * n + i];
-            yv[q] = y[k + q];
-        }
+        for (int r = 0; r < 8; ++r)
 #pragma unroll
-        for (int q = 0; q < D; ++q) acc[q] += wv[q] * yv[q];
+            for (int q = 0; q < P; ++q) {
+                const int k = (j + r) * D + q;
+                wv[r][q] = j + r < m ? Wc[(size_t)k * ld] : (T)0;
+                yv[r][q] = j + r < m ? yc[k] : (T)0;
+            }
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+#pragma unroll
+            for (int q = 0; q < P; ++q)
+                if (j + r < m) acc[q] += wv[r][q] * yv[r][q];
     }
-    for (; k < k1; ++k) acc[0] += W[(size_t)k * n + i] * y[k];
-    return tree_sum<T, D>(acc);
+    if (warp == 0)
+        for (int k = k0 + m * D; k < k1; ++k) acc[0] += W[(size_t)k * ld + i] * y[k];
+    red[warp][lane] = tree_sum<T, P>(acc);
+    __syncthreads();
+    T r = (T)0;
+    if (warp == 0) {
+        T part[NW];
+#pragma unroll
+        for (int q = 0; q < NW; ++q) part[q] = red[q][lane];
+        r = tree_sum<T, NW>(part);
+    }
+    __syncthreads();
+    return r;
 }
 
 // loads in flight per lane in the refinement's products with W (compute type)
 template <typename T>
 __host__ __device__ constexpr int w_depth() { return sizeof(T) == 4 ? kWDepth32 : 8; }
-
-// trailing-update tile tt -> (ti, tj), ti >= tj
-__device__ __forceinline__ void lower_tile(int tt, int *ti, int *tj) {
-    int t = tt, i = 0;
-    while (t > i) {
-        t -= i + 1;
-        ++i;
-    }
-    *ti = i;
-    *tj = t;
-}
-
-// Phase P task `task` of one system at panel k0: a 64-row tile of the panel
-// L_ik = A_ik L_kk^-T (task < npt) or a 64-column tile of block row k of W,
-// W_k[:, 0:k0] = L_kk^-1 W_k[:, 0:k0].  L_kk^-1 is held in W_kk.  Each tile
-// reads its inputs into shared memory before it overwrites them.
-template <typename T>
-__device__ void panel_task(const SolveArgs<T> &s, TileSmem<T> &sm, int k0, int kn, int base, int npt, int task) {
-    const int n = s.n, tid = threadIdx.x, tr = tid / 16, tc = tid % 16;
-    const T *Linv = s.W + (size_t)k0 * n + k0;
-    T acc[4][4] = {};
-    if (task < npt) {
-        const int i0 = base + task * kTile, ni = min(kTile, n - i0);
-        // a(i, p) = A[i0 + i][k0 + p], b(p, c) = Linv[c][p]
-        tile_gemm(acc, sm, s.A + k0, n, i0, ni, Linv, n, 0, kn, true, 0, kn);
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                const int i = tr * 4 + u, j = tc + 16 * v;
-                if (i < ni && j < kn) s.A[(size_t)(i0 + i) * n + k0 + j] = acc[u][v];
-            }
-    } else {
-        const int j0 = (task - npt) * kTile, nj = min(kTile, k0 - j0);
-        // a(r, p) = Linv[r][p], b(p, c) = W[k0 + p][j0 + c]
-        tile_gemm(acc, sm, s.W + k0, n, k0, kn, s.W + (size_t)k0 * n, n, j0, nj, false, 0, kn);
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                const int r = tr * 4 + u, c = tc + 16 * v;
-                if (r < kn && c < nj) s.W[(size_t)(k0 + r) * n + j0 + c] = acc[u][v];
-            }
-    }
-}
-
-// Phase U task `task` of one system at panel k0 (panel width NB): a 64x64
-// tile of the trailing lower triangle, A_ij -= L_ik L_jk^T (task < ntiles;
-// task 0 holds the next diagonal block, whose last update factor_block
-// applies itself: with NB = 32 that tile stores only its rows below it, with
-// NB = 64 it is not a task), or a 64x64 tile of the block rows of W below,
-// W_i[:, 0:k0+NB] -= L_ik W_k.  Columns k0..k0+NB-1 of W below the diagonal
-// block are first written by this step, so their old values are zero and
-// are not read (W is never cleared).  The products run over k in chunks of 32.
-template <typename T>
-struct UpdTile {
-    int i0, j0, ni, nj;
-    int rmin;       // first row stored
-    bool wtile;     // a tile of W (else of A)
-    TileOps<T> op;  // operands of the first chunk, loaded ahead of the product
-};
-
-template <int NB, typename T>
-__device__ __forceinline__ void upd_desc(UpdTile<T> &u, const SolveArgs<T> &s, int k0, int base, int ntiles, int ncw,
-                                         int task) {
-    const int n = s.n;
-    u.wtile = task >= ntiles;
-    if (!u.wtile) {
-        int ti, tj;
-        lower_tile(task, &ti, &tj);
-        u.i0 = base + ti * kTile;
-        u.j0 = base + tj * kTile;
-        u.nj = min(kTile, n - u.j0);
-    } else {
-        const int q = task - ntiles;
-        u.i0 = base + (q / ncw) * kTile;
-        u.j0 = (q % ncw) * kTile;
-        u.nj = min(kTile, k0 + NB - u.j0);
-    }
-    u.ni = min(kTile, n - u.i0);
-    u.rmin = (task == 0) ? base + NB : u.i0;
-}
-
-// a(i, p) = L[i0 + i][k0 + p]; b(p, j) = L[j0 + j][k0 + p] (A tile) or
-// W[k0 + p][j0 + j] (W tile)
-template <bool WT, typename T>
-__device__ __forceinline__ void upd_load(UpdTile<T> &u, const SolveArgs<T> &s, int k0) {
-    const int n = s.n;
-    tile_load<!WT>(u.op, s.A + k0, n, u.i0, u.ni, WT ? s.W + (size_t)k0 * n : s.A + k0, n, u.j0, u.nj, 0, kKC);
-}
-
-// element (i, j) of the tile is stored (A: lower triangle; W: columns below k0 + NB)
-template <bool WT, int NB>
-__device__ __forceinline__ bool upd_in(int n, int k0, int rmin, int i, int j) {
-    return i < n && i >= rmin && (WT ? j < k0 + NB : (j < n && j <= i));
-}
-
-template <bool WT, int NB, typename T>
-__device__ __forceinline__ void upd_old(const UpdTile<T> &u, const SolveArgs<T> &s, int k0, T (&old)[4][4]) {
-    const int n = s.n, tid = threadIdx.x, tr = tid / 16, tc = tid % 16;
-    const T *C = WT ? s.W : s.A;
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const int i = u.i0 + tr * 4 + a, j = u.j0 + tc + 16 * v;
-            old[a][v] = (upd_in<WT, NB>(n, k0, u.rmin, i, j) && !(WT && j >= k0)) ? C[(size_t)i * n + j] : (T)0;
-        }
-}
-
-template <bool WT, int NB, typename T>
-__device__ __forceinline__ void upd_store(const UpdTile<T> &u, const SolveArgs<T> &s, int k0, const T (&old)[4][4],
-                                          const T (&acc)[4][4]) {
-    const int n = s.n, tid = threadIdx.x, tr = tid / 16, tc = tid % 16;
-    T *C = WT ? s.W : s.A;
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const int i = u.i0 + tr * 4 + a, j = u.j0 + tc + 16 * v;
-            if (upd_in<WT, NB>(n, k0, u.rmin, i, j)) C[(size_t)i * n + j] = old[a][v] - acc[a][v];
-        }
-}
-
-// the tile whose first operand chunk is in u.op: old values (their loads
-// overlap the product), product on the CUDA cores (the loads of a later
-// chunk are in flight during the product of the one before), store
-template <bool WT, int NB, typename T>
-__device__ __forceinline__ void upd_finish(const UpdTile<T> &u, const SolveArgs<T> &s, TileSmem<T> &sm, int k0) {
-    T old[4][4], acc[4][4] = {};
-    upd_old<WT, NB>(u, s, k0, old);
-    tile_stage<!WT>(sm, u.op);
-    const int n = s.n;
-#pragma unroll
-    for (int c = 1; c < NB / kKC; ++c) {
-        TileOps<T> o;
-        tile_load<!WT>(o, s.A + k0, n, u.i0, u.ni, WT ? s.W + (size_t)k0 * n : s.A + k0, n, u.j0, u.nj, c * kKC,
-                       kKC);
-        tile_compute(acc, sm);
-        tile_stage<!WT>(sm, o);
-    }
-    tile_compute(acc, sm);
-    upd_store<WT, NB>(u, s, k0, old, acc);
-}
-
-// One task on its own.  The tensor-core variant takes the tile product on
-// the tensor cores in FP32 (3xTF32, per chunk of 32); a tensor-core wait that
-// timed out flags the system (SFFT_ERR_TIMEOUT) and the tile is computed on
-// the CUDA cores.
-template <typename T, bool TC, int NB>
-__device__ void update_task(const SolveArgs<T> &s, SolveSmem<T> &smu, TcState &st, int k0, int base, int ntiles,
-                            int ncw, int task) {
-    UpdTile<T> u;
-    upd_desc<NB>(u, s, k0, base, ntiles, ncw, task);
-    if constexpr (TC && sizeof(T) == 4) {
-        const int n = s.n;
-        T old[4][4], acc[4][4] = {};
-        if (u.wtile)
-            upd_old<true, NB>(u, s, k0, old);
-        else
-            upd_old<false, NB>(u, s, k0, old);
-        const T *Bg = u.wtile ? s.W + (size_t)k0 * n : s.A + k0;
-        bool ok = true;
-        for (int kk = 0; kk < NB && ok; kk += kKC) {
-            T part[4][4];
-            ok = tile_gemm_tc(part, smu.tc, st, s.A + k0, n, u.i0, u.ni, Bg, n, u.j0, u.nj, !u.wtile, kk, kk + kKC);
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int v = 0; v < 4; ++v) acc[a][v] += part[a][v];
-        }
-        if (!ok) {
-            if (threadIdx.x == 0) s.flag[0] = SFFT_ERR_TIMEOUT;
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int v = 0; v < 4; ++v) acc[a][v] = (T)0;
-            tile_gemm(acc, smu.tile, s.A + k0, n, u.i0, u.ni, Bg, n, u.j0, u.nj, !u.wtile, 0, NB);
-        }
-        if (u.wtile)
-            upd_store<true, NB>(u, s, k0, old, acc);
-        else
-            upd_store<false, NB>(u, s, k0, old, acc);
-    } else if (u.wtile) {
-        upd_load<true>(u, s, k0);
-        upd_finish<true, NB>(u, s, smu.tile, k0);
-    } else {
-        upd_load<false>(u, s, k0);
-        upd_finish<false, NB>(u, s, smu.tile, k0);
-    }
-}
 
 // row i of A = D M D up to the diagonal, eight loads of each operand in flight per lane
 template <typename T>
@@ -957,7 +916,7 @@ __device__ __forceinline__ void scale_row(const SolveArgs<T> &s, int i, int lane
     const int n = s.n;
     const double di = s.dsc[i];
     const double *Mi = s.M + (size_t)i * n;
-    T *Ai = s.A + (size_t)i * n;
+    T *Ai = s.X + (size_t)i * s.ld;
     for (int j0 = lane; j0 <= i; j0 += 8 * 32) {
         double m[8], d[8];
 #pragma unroll
@@ -976,7 +935,7 @@ __device__ __forceinline__ void scale_row(const SolveArgs<T> &s, int i, int lane
 
 // Up to kMaxBatch systems, of equal or different sizes, solved together:
 // every phase spreads the tasks of all systems over the grid, and block b
-// factors the diagonal blocks of system b, so the serial chains of the
+// forms the diagonal blocks of system b, so the serial chains of the
 // systems run side by side.  Each system sees the operations of a solve on
 // its own, in the same order.
 template <typename T>
@@ -992,37 +951,111 @@ __device__ __forceinline__ int sys_of(const int *offs, int nsys, int task) {
     return b;
 }
 
-template <typename T, bool TC, int NB>
+// sum of squares of the n values of v by the whole block, in an order that
+// depends on n alone; valid in thread 0
+__device__ __forceinline__ double block_norm2(const double *v, int n, double *red) {
+    double a = 0.0;
+    for (int i0 = threadIdx.x; i0 < n; i0 += 8 * kThreads) {
+        double u[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) u[q] = i0 + q * kThreads < n ? v[i0 + q * kThreads] : 0.0;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) a += u[q] * u[q];
+    }
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = a;
+    __syncthreads();
+    double r = 0.0;
+    if (threadIdx.x == 0)
+        for (int w = 0; w < kThreads / 32; ++w) r += red[w];
+    return r;
+}
+
+// Barrier of the whole grid after a first grid.sync (which orders the reset of
+// its counter).  Unlike that of the cooperative groups an arrival does not
+// wait for the counter's value, and the thread that makes it can be any.
+// Waits are bounded: one that runs out moves the counter past every later
+// target, so that all blocks run to the end, and the solve reports a timeout.
+constexpr int kBarDead = 1 << 30;
+constexpr long long kBarWaitCycles = 4000000000LL;  // about two seconds
+struct GridBar {
+    int *cnt;
+    int target;
+    __device__ __forceinline__ void arrive(int thread) {  // after the block's work: every thread calls it
+        __syncthreads();
+        if ((int)threadIdx.x == thread) {
+            __threadfence();
+            asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(cnt) : "memory");
+        }
+        target += gridDim.x;
+    }
+    __device__ __forceinline__ void wait() {
+        if (threadIdx.x == 0) {
+            const long long t0 = clock64();
+            int v;
+            do {
+                asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(cnt) : "memory");
+                if (v < target && clock64() - t0 > kBarWaitCycles) {
+                    atomicMax(cnt, kBarDead);
+                    break;
+                }
+            } while (v < target);
+            __threadfence();
+        }
+        __syncthreads();
+    }
+    __device__ __forceinline__ void sync() {
+        arrive(0);
+        wait();
+    }
+};
+
+template <typename T, bool TC>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kBlocksPerSM : 1) k_solve_coop(BatchArgs<T> ba) {
+    using S = Shape<T>;
+    constexpr int TS = S::TS;
     cg::grid_group grid = cg::this_grid();
-    __shared__ SolveSmem<T> sm;
-    __shared__ double sums[kMaxBatch][2];
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    SolveSmem<T> &sm = *reinterpret_cast<SolveSmem<T> *>(smem_raw);
+    __shared__ double red[kThreads / 32];
     __shared__ __align__(8) uint64_t tc_mbar;
     __shared__ uint32_t tc_slot;
     TcState st{};
     if constexpr (TC) tc_init(st, &tc_mbar, &tc_slot);
     const int tid = threadIdx.x, bid = blockIdx.x, nbk = gridDim.x;
     const int gtid = bid * kThreads + tid, gthreads = nbk * kThreads;
+    // warp tasks: consecutive ones on different blocks, so that every
+    // multiprocessor gets its share of a short list (its FP64 units bound the
+    // residual and the scaling)
     const int warp = tid >> 5, lane = tid & 31, nw = kThreads / 32;
+    const int wtask = warp * nbk + bid, wstep = nbk * nw;
     const int nsys = ba.nsys;
     // sizes may differ between systems: rows of all systems as one flat range
     int nrow[kMaxBatch + 1];
-    nrow[0] = 0;
+    int wofs[kMaxBatch + 1];  // flat W^T y tasks of all systems
+    int yofs[kMaxBatch + 1];  // flat row-pair tasks (k, n - 1 - k) of all systems
+    nrow[0] = wofs[0] = yofs[0] = 0;
     int nblk_max = 0;
     for (int b = 0; b < nsys; ++b) {
-        nrow[b + 1] = nrow[b] + ba.sys[b].n;
-        nblk_max = max(nblk_max, (ba.sys[b].n + NB - 1) / NB);
+        const int n = ba.sys[b].n;
+        nrow[b + 1] = nrow[b] + n;
+        wofs[b + 1] = wofs[b] + ((n + 31) / 32) * kSeg;
+        yofs[b + 1] = yofs[b] + (n + 1) / 2;
+        nblk_max = max(nblk_max, ba.sys[b].ld / TS);
     }
     const int nrows_all = nrow[nsys];
 
-    // ---- status reset; Jacobi scaling, zero W and x -------------------------
+    // ---- status reset; Jacobi scaling, zero x and the padding rows of X ------
     if (bid == 0 && tid < nsys) {
         const SolveArgs<T> &s = ba.sys[tid];
-        s.flag[0] = s.flag[1] = s.flag[2] = s.flag[3] = 0;
+        s.flag[0] = s.flag[1] = s.flag[3] = 0;
+        s.flag[2] = INT_MAX;
         s.stats[0] = 1e300;
         s.stats[1] = s.stats[2] = s.stats[3] = 0.0;
     }
     grid.sync();
+    GridBar bar{&ba.sys[0].flag[3], 0};
     for (int b = 0; b < nsys; ++b) {
         const SolveArgs<T> &s = ba.sys[b];
         const int n = s.n;
@@ -1032,110 +1065,145 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kBlocksPerSM : 1) k
             s.dsc[i] = (d > 0.0) ? 1.0 / sqrt(d) : 0.0;
             s.x[i] = 0.0;
         }
+        for (int e = gtid; e < (s.ld - n) * s.ld; e += gthreads) s.X[(size_t)n * s.ld + e] = (T)0;
     }
-    int wofs[kMaxBatch + 1];  // flat W^T y tasks of all systems
-    int yofs[kMaxBatch + 1];  // flat row-pair tasks (k, n - 1 - k) of all systems
-    wofs[0] = yofs[0] = 0;
-    for (int b = 0; b < nsys; ++b) {
-        wofs[b + 1] = wofs[b] + ((ba.sys[b].n + 31) / 32) * kSeg;
-        yofs[b + 1] = yofs[b] + (ba.sys[b].n + 1) / 2;
-    }
-    grid.sync();
+    bar.sync();
     // A = D M D on the lower triangle (nothing reads the upper one), one warp
     // per row pair (k, n - 1 - k)
-    for (int task = bid * nw + warp; task < yofs[nsys]; task += nbk * nw) {
+    for (int task = wtask; task < yofs[nsys]; task += wstep) {
         const int b = sys_of(yofs, nsys, task), k = task - yofs[b];
         const SolveArgs<T> &s = ba.sys[b];
         scale_row(s, k, lane);
         if (s.n - 1 - k != k) scale_row(s, s.n - 1 - k, lane);
     }
-    grid.sync();
+    bar.sync();
 
     // ---- Cholesky and W = L^-1 ----------------------------------------------
     // A system whose status turned negative is skipped from then on, and one
-    // whose panels are done waits for the larger ones.  The task counts must
-    // be the same in every block, so each step reads the status flags once,
-    // right after a barrier and before the update phase in which factor_inv
-    // may write them again.
-    if (bid < nsys && ba.sys[bid].flag[0] == 0) factor_block<NB>(ba.sys[bid], sm.fac, 0, -1);
-    grid.sync();
+    // whose steps are done waits for the larger ones.  The task counts must be
+    // the same in every block: a chain that fails while step kb runs records
+    // block kb + 1, which the test of step kb reads the same way before and
+    // after.
+    bool bad = false;  // of the chain of system bid (thread 0)
+    T minpiv = (T)1e30;
+    if (bid < nsys && ba.sys[bid].flag[0] == 0) chain_block(ba.sys[bid], sm.chain, 0, false, bad, minpiv, [] {});
+    bar.sync();
     for (int kb = 0; kb < nblk_max; ++kb) {
-        const int k0 = kb * NB;
-        const int base = k0 + NB;  // first trailing row
         unsigned live = 0;
-        for (int b = 0; b < nsys; ++b)
-            if (kb < (ba.sys[b].n + NB - 1) / NB && ba.sys[b].flag[0] == 0) live |= 1u << b;
-        int offs[kMaxBatch + 1];
-        offs[0] = 0;
+        bool more = false;
+        int poff[kMaxBatch + 1], uoff[kMaxBatch + 1];
+        poff[0] = uoff[0] = 0;
         for (int b = 0; b < nsys; ++b) {
             const SolveArgs<T> &s = ba.sys[b];
-            int cnt = 0;
-            if (live & (1u << b)) {
-                const int rows = s.n - base;
-                cnt = (rows > 0 ? (rows + kTile - 1) / kTile : 0) + (k0 + kTile - 1) / kTile;
+            const int blocks = s.ld / TS;
+            int np = 0, nu = 0;
+            if (kb < blocks && s.flag[0] == 0 && s.flag[2] > kb) {
+                live |= 1u << b;
+                np = s.ld / kDB;
+                if (kb + 1 < blocks) {
+                    more = true;
+                    nu = tile_count(blocks, kb);
+                }
             }
-            offs[b + 1] = offs[b] + cnt;
+            poff[b + 1] = poff[b] + np;
+            uoff[b + 1] = uoff[b] + nu;
         }
-        for (int task = bid; task < offs[nsys]; task += nbk) {
-            const int b = sys_of(offs, nsys, task);
-            const SolveArgs<T> &s = ba.sys[b];
-            const int rows = s.n - base;
-            const int npt = rows > 0 ? (rows + kTile - 1) / kTile : 0;
-            panel_task(s, sm.tile, k0, min(NB, s.n - k0), base, npt, task - offs[b]);
-        }
-        grid.sync();
-        // Block b applies the last update to the next diagonal block of
-        // system b (tile 0) and factors that block at once; the other blocks
-        // share the remaining tiles of all systems.
-        bool any = false;
-        offs[0] = 0;
-        for (int b = 0; b < nsys; ++b) {
-            const SolveArgs<T> &s = ba.sys[b];
-            const int rows = s.n - base;
-            int per = 0;
-            if ((live & (1u << b)) && rows > 0) {
-                const int nt = (rows + kTile - 1) / kTile;
-                // NB = 64: tile 0 is the diagonal block, not a task
-                per = nt * (nt + 1) / 2 + nt * ((k0 + NB + kTile - 1) / kTile) - (NB == kTile ? 1 : 0);
-                any = true;
-            }
-            offs[b + 1] = offs[b] + per;
-        }
-        if (!any) break;  // every system's panels are done (same in every block)
-        if (bid < nsys) {
-            const SolveArgs<T> &s = ba.sys[bid];
-            const int rows = s.n - base;
-            if ((live & (1u << bid)) && rows > 0) factor_block<NB>(s, sm.fac, kb + 1, k0);
+        const bool chain = bid < nsys && (live & (1u << bid)) && kb + 1 < ba.sys[bid].ld / TS;
+        if (chain) {
+            chain_block(ba.sys[bid], sm.chain, kb + 1, true, bad, minpiv, [&] { bar.arrive(kThreads - 1); });
+            bar.wait();
         } else {
-            for (int task = bid - nsys; task < offs[nsys]; task += nbk - nsys) {
-                const int b = sys_of(offs, nsys, task);
-                const SolveArgs<T> &s = ba.sys[b];
-                const int nt = (s.n - base + kTile - 1) / kTile;
-                update_task<T, TC, NB>(s, sm, st, k0, base, nt * (nt + 1) / 2, (k0 + NB + kTile - 1) / kTile,
-                                       (NB == kTile ? 1 : 0) + task - offs[b]);
+            if (bid >= nsys) {
+                for (int task = bid - nsys; task < poff[nsys]; task += nbk - nsys) {
+                    const int b = sys_of(poff, nsys, task);
+                    panel_task(ba.sys[b], sm.panel, kb, task - poff[b]);
+                }
+            }
+            bar.sync();
+        }
+        if (!more) break;  // every system's steps are done (same in every block)
+        if (bid >= nsys) {
+            const int step = nbk - nsys, total = uoff[nsys];
+            if constexpr (TC && sizeof(T) == 4) {
+                for (int task = bid - nsys; task < total; task += step) {
+                    const int b = sys_of(uoff, nsys, task);
+                    const SolveArgs<T> &s = ba.sys[b];
+                    int i, j;
+                    tile_of(kb, task - uoff[b], i, j);
+                    T old[4][4];
+                    tile_old(s, kb, i, j, old);
+                    bool ok = true;
+                    for (int kk = 0; kk < TS && ok; kk += kKC) {
+                        T part[4][4];
+                        ok = tile_mul_tc(part, sm.tc, st, s.P, s.ld, i * TS, j * TS, kk);
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+#pragma unroll
+                            for (int v = 0; v < 4; ++v) old[u][v] -= part[u][v];
+                    }
+                    if (!ok) {  // a wait that timed out: flag the system, redo the tile on the CUDA cores
+                        if (tid == 0) s.flag[0] = SFFT_ERR_TIMEOUT;
+                        tile_old(s, kb, i, j, old);
+                        tile_fetch(s, sm.upd.a[0], sm.upd.b[0], i, j);
+                        asm volatile("cp.async.wait_all;\n" ::: "memory");
+                        __syncthreads();
+                        tile_update(old, sm.upd.a[0], sm.upd.b[0]);
+                        __syncthreads();
+                    }
+                    tile_store(s, i, j, old);
+                }
+            } else {
+                // the operands of the next tile arrive while this one's product runs
+                int task = bid - nsys, b = 0, i = 0, j = 0, buf = 0;
+                auto fetch = [&](int t, int &fb, int &fi, int &fj, int to) {
+                    fb = sys_of(uoff, nsys, t);
+                    tile_of(kb, t - uoff[fb], fi, fj);
+                    tile_fetch(ba.sys[fb], sm.upd.a[to], sm.upd.b[to], fi, fj);
+                    asm volatile("cp.async.commit_group;\n" ::: "memory");
+                };
+                __syncthreads();  // phase P's shared memory is free
+                if (task < total) fetch(task, b, i, j, 0);
+                while (task < total) {
+                    const SolveArgs<T> &s = ba.sys[b];
+                    const int next = task + step;
+                    int nb_ = 0, ni = 0, nj = 0;
+                    T old[S::R][S::R];
+                    tile_old(s, kb, i, j, old);
+                    if (next < total) {
+                        fetch(next, nb_, ni, nj, buf ^ 1);
+                        asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+                    } else {
+                        asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+                    }
+                    __syncthreads();
+                    tile_update(old, sm.upd.a[buf], sm.upd.b[buf]);
+                    tile_store(s, i, j, old);
+                    __syncthreads();  // before this buffer is filled again
+                    task = next;
+                    b = nb_;
+                    i = ni;
+                    j = nj;
+                    buf ^= 1;
+                }
             }
         }
-        grid.sync();
+        bar.sync();
     }
+
+    if (bid < nsys && tid == 0 && (double)minpiv < ba.sys[bid].stats[0]) ba.sys[bid].stats[0] = (double)minpiv;
 
     // ---- refinement ---------------------------------------------------------
     // done: bit b set once system b has converged, failed or run out of
     // iterations; every block derives it from the same values.  The norms
-    // are sums over the rows in one fixed order (warp b of every block sums
-    // system b), so the decisions do not depend on the grid or the batch.
+    // are sums over the rows in one fixed order, so the decisions do not depend
+    // on the grid or the batch.
     unsigned done = 0;
     for (int b = 0; b < nsys; ++b)
-        if (ba.sys[b].flag[0] != 0) done |= 1u << b;
+        if (ba.sys[b].flag[0] != 0 || ba.sys[b].flag[2] != INT_MAX) done |= 1u << b;
     const unsigned all = (1u << nsys) - 1u;
-    if (warp < nsys) {
-        const SolveArgs<T> &s = ba.sys[warp];
-        const double bb = dot_warp<double>(s.rhs, s.rhs, lane, s.n);
-        if (lane == 0) sums[warp][1] = bb;
-    }
-    __syncthreads();
     for (int it = 0; it <= kMaxIters && done != all; ++it) {
         // r = rhs - M x (FP64); z = D r
-        for (int row = bid * nw + warp; row < nrows_all; row += nbk * nw) {
+        for (int row = wtask; row < nrows_all; row += wstep) {
             const int b = sys_of(nrow, nsys, row), i = row - nrow[b];
             if (done & (1u << b)) continue;
             const SolveArgs<T> &s = ba.sys[b];
@@ -1146,23 +1214,40 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kBlocksPerSM : 1) k
                 s.z[i] = (T)(s.dsc[i] * ri);
             }
         }
-        grid.sync();
-        if (warp < nsys && !(done & (1u << warp))) {
-            const SolveArgs<T> &s = ba.sys[warp];
-            const double rr = dot_warp<double>(s.r, s.r, lane, s.n);
-            if (lane == 0) sums[warp][0] = rr;
+        bar.sync();
+        // ||r||^2 (and first ||rhs||^2) of system b by block b, beside the
+        // product y = W z of the others: the next barrier serves both
+        if (bid < nsys && !(done & (1u << bid))) {
+            const SolveArgs<T> &s = ba.sys[bid];
+            const double rr = block_norm2(s.r, s.n, red);
+            if (it == 0) {
+                const double bb = block_norm2(s.rhs, s.n, red);
+                if (tid == 0) s.stats[1] = bb;
+            }
+            if (tid == 0) s.stats[2] = rr;
         }
-        __syncthreads();
+        // y = W z  (W lower triangular; row i has i + 1 entries).  A warp task
+        // takes rows k and n - 1 - k, n + 1 entries together, so that every
+        // task has the same length.
+        for (int task = bid < nsys ? yofs[nsys] : warp * (nbk - nsys) + bid - nsys; task < yofs[nsys];
+             task += (nbk - nsys) * nw) {
+            const int b = sys_of(yofs, nsys, task), k = task - yofs[b];
+            if (done & (1u << b)) continue;
+            const SolveArgs<T> &s = ba.sys[b];
+            const int i2 = s.n - 1 - k;
+            const T a = dot_warp<T, T, w_depth<T>()>(s.X + (size_t)k * s.ld, s.z, lane, k + 1);
+            if (lane == 0) s.y[k] = a;
+            if (i2 != k) {
+                const T a2 = dot_warp<T, T, w_depth<T>()>(s.X + (size_t)i2 * s.ld, s.z, lane, i2 + 1);
+                if (lane == 0) s.y[i2] = a2;
+            }
+        }
+        bar.sync();
         for (int b = 0; b < nsys; ++b) {
             if (done & (1u << b)) continue;
             const SolveArgs<T> &s = ba.sys[b];
-            const double rr = sums[b][0], bb = sums[b][1];
-            const double rel = (bb > 0.0) ? sqrt(rr / bb) : sqrt(rr);
-            if (bid == 0 && tid == 0) {
-                s.stats[1] = bb;
-                s.stats[2] = rr;
-            }
-            if (rel <= kTol || rr == 0.0) {
+            const double bb = s.stats[1], rr = s.stats[2];
+            if (rr <= kTol * kTol * (bb > 0.0 ? bb : 1.0) || rr == 0.0) {
                 if (bid == 0 && tid == 0) s.flag[0] = 1;
                 done |= 1u << b;
             } else if (it == kMaxIters) {
@@ -1171,24 +1256,8 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kBlocksPerSM : 1) k
             }
         }
         if (done == all) break;
-        // y = W z  (W lower triangular; row i has i + 1 entries).  A warp task
-        // takes rows k and n - 1 - k, n + 1 entries together, so that every
-        // task has the same length.
-        for (int task = bid * nw + warp; task < yofs[nsys]; task += nbk * nw) {
-            const int b = sys_of(yofs, nsys, task), k = task - yofs[b];
-            if (done & (1u << b)) continue;
-            const SolveArgs<T> &s = ba.sys[b];
-            const int i2 = s.n - 1 - k;
-            const T a = dot_warp<T, T, w_depth<T>()>(s.W + (size_t)k * s.n, s.z, lane, k + 1);
-            if (lane == 0) s.y[k] = a;
-            if (i2 != k) {
-                const T a2 = dot_warp<T, T, w_depth<T>()>(s.W + (size_t)i2 * s.n, s.z, lane, i2 + 1);
-                if (lane == 0) s.y[i2] = a2;
-            }
-        }
-        grid.sync();
         // w = W^T y in kSeg row segments (coalesced rows of W), summed in a fixed order
-        for (int task = bid * nw + warp; task < wofs[nsys]; task += nbk * nw) {
+        for (int task = bid; task < wofs[nsys]; task += nbk) {
             const int b = sys_of(wofs, nsys, task), q = task - wofs[b];
             if (done & (1u << b)) continue;
             const SolveArgs<T> &s = ba.sys[b];
@@ -1197,9 +1266,11 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kBlocksPerSM : 1) k
             const int ch = q / kSeg, sg = q % kSeg;
             const int i = ch * 32 + lane;
             const int k0 = max(ch * 32, sg * segrows), k1 = min(n, (sg + 1) * segrows);
-            if (i < n) s.wseg[(size_t)sg * n + i] = col_dot<T, w_depth<T>()>(s.W, s.y, n, i, k0, k1);
+            // (columns n and up of the last chunk are padding; their sums are not stored)
+            const T a = col_dot<T, w_depth<T>()>(s.X, s.y, s.ld, i, k0, k1, sm.red);
+            if (warp == 0 && i < n) s.wseg[(size_t)sg * n + i] = a;
         }
-        grid.sync();
+        bar.sync();
         for (int e = gtid; e < nrows_all; e += gthreads) {
             const int b = sys_of(nrow, nsys, e), i = e - nrow[b];
             if (done & (1u << b)) continue;
@@ -1210,7 +1281,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kBlocksPerSM : 1) k
             s.x[i] += s.dsc[i] * (double)a;
         }
         if (bid == 0 && tid < nsys && !(done & (1u << tid))) ba.sys[tid].flag[1] += 1;
-        grid.sync();
+        bar.sync();
     }
     // ---- results ------------------------------------------------------------
     for (int e = gtid; e < nrows_all; e += gthreads) {
@@ -1220,8 +1291,10 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kBlocksPerSM : 1) k
     if (bid == 0 && tid < nsys) {
         const SolveArgs<T> &s = ba.sys[tid];
         if (s.info) {
-            const int f = s.flag[0];
-            s.info->status = (f == 1) ? SFFT_OK : (f == 0 ? SFFT_ERR_NOT_CONVERGED : f);
+            int f = s.flag[0];
+            if (*bar.cnt >= kBarDead) f = SFFT_ERR_TIMEOUT;
+            if (f == 0) f = s.flag[2] != INT_MAX ? SFFT_ERR_SINGULAR : SFFT_ERR_NOT_CONVERGED;
+            s.info->status = (f == 1) ? SFFT_OK : f;
             s.info->iters = s.flag[1];
             s.info->rel_residual = (s.stats[1] > 0.0) ? sqrt(s.stats[2] / s.stats[1]) : sqrt(s.stats[2]);
             s.info->min_pivot = s.stats[0];
@@ -1230,22 +1303,25 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kBlocksPerSM : 1) k
     if constexpr (TC) tc_release(st);
 }
 
-static size_t solve_dyn_smem(bool) { return 0; }
+static size_t solve_dyn_smem(bool fp64) { return fp64 ? sizeof(SolveSmem<double>) : sizeof(SolveSmem<float>); }
 
 // Arguments of one system: the caller's M, rhs, x, info and the workspace.
 template <typename T>
 static SolveArgs<T> system_args(int n, const double *M, const double *rhs, double *x, sfft_solve_info *info,
-                                double *dsc, double *xw, double *r, void *A, void *W, void *zv, int *flag) {
+                                double *dsc, double *xw, double *r, void *A, void *zv, int *flag) {
+    constexpr int TS = Shape<T>::TS;
     SolveArgs<T> a;
     a.n = n;
+    a.ld = (n + TS - 1) / TS * TS;
     a.M = M;
     a.rhs = rhs;
     a.dsc = dsc;
     a.x = xw;
     a.r = r;
     a.stats = xw + n;
-    a.A = (T *)A;
-    a.W = (T *)W;
+    a.X = (T *)A;
+    a.P = a.X + (size_t)a.ld * a.ld;
+    a.D = a.P + (size_t)TS * a.ld;
     a.z = (T *)zv;
     a.y = (T *)zv + n;
     a.wseg = (T *)zv + 2 * (size_t)n;
@@ -1255,19 +1331,22 @@ static SolveArgs<T> system_args(int n, const double *M, const double *rhs, doubl
     return a;
 }
 
-// the kernel variant: tile products on the tensor cores (FP32 only), panel
-// width 32 or 64 (FP32 only; FP64 solves use 32)
-static const void *solve_kernel(bool fp64, bool tc, int panel) {
-    if (fp64) return (const void *)k_solve_coop<double, false, 32>;
-    if (panel == 64) return tc ? (const void *)k_solve_coop<float, true, 64> : (const void *)k_solve_coop<float, false, 64>;
-    return tc ? (const void *)k_solve_coop<float, true, 32> : (const void *)k_solve_coop<float, false, 32>;
+size_t solve_matrix_elems(int n, bool fp64) {
+    const size_t ts = fp64 ? Shape<double>::TS : Shape<float>::TS, ld = (n + ts - 1) / ts * ts;
+    return ld * ld + ts * ld + 2 * 3 * kDB * kDB;
+}
+
+// the kernel variant: tile products on the tensor cores (FP32 only) or not
+static const void *solve_kernel(bool fp64, bool tc) {
+    if (fp64) return (const void *)k_solve_coop<double, false>;
+    return tc ? (const void *)k_solve_coop<float, true> : (const void *)k_solve_coop<float, false>;
 }
 
 template <typename T>
-static cudaError_t launch_batch(const BatchArgs<T> &ba, int grid, cudaStream_t st, bool tc = false, int panel = 32) {
+static cudaError_t launch_batch(const BatchArgs<T> &ba, int grid, cudaStream_t st, bool tc = false) {
     if (grid <= ba.nsys) return cudaErrorInvalidConfiguration;  // blocks >= nsys take the shared tasks
     void *args[] = {(void *)&ba};
-    const void *kern = solve_kernel(sizeof(T) == 8, tc, panel);
+    const void *kern = solve_kernel(sizeof(T) == 8, tc);
     return cudaLaunchCooperativeKernel(kern, grid, kThreads, args, solve_dyn_smem(sizeof(T) == 8), st);
 }
 
@@ -1278,8 +1357,7 @@ static cudaError_t solve_batch_t(Plan *const *plans, int count, const double *co
     ba.nsys = count;
     for (int b = 0; b < count; ++b) {
         Plan *p = plans[b];
-        ba.sys[b] = system_args<T>(p->n, M[b], rhs[b], x[b], info[b], p->dscale, p->xw, p->r, p->A, p->Wm, p->zv,
-                                   p->flag);
+        ba.sys[b] = system_args<T>(p->n, M[b], rhs[b], x[b], info[b], p->dscale, p->xw, p->r, p->A, p->zv, p->flag);
     }
     // the tensor-core tile variant (tune_tc = 2, FP32 only) allocates tensor
     // memory, which limits it to one block per SM: its own grid
@@ -1296,7 +1374,7 @@ static cudaError_t solve_batch_t(Plan *const *plans, int count, const double *co
         // serving against 515 on 152)
         grid = full / kBlocksPerSM;
     }
-    const cudaError_t err = launch_batch(ba, grid, st, tc, plans[0]->solve_panel);
+    const cudaError_t err = launch_batch(ba, grid, st, tc);
     plans[0]->launches += 1;
     return err;
 }
@@ -1322,17 +1400,11 @@ int solve_grid_size(bool fp64, bool tc) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const size_t dsm = solve_dyn_smem(fp64);
     // all of the unified L1/shared storage as shared memory, so that two FP32
-    // blocks (33 KB of static shared memory each) fit on an SM; the grid is
-    // the smaller residency of the two panel widths
-    per = 1 << 30;
-    for (int panel = 32; panel <= (fp64 ? 32 : 64); panel += 32) {
-        const void *kern = solve_kernel(fp64, tc, panel);
-        cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsm);
-        int pk = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pk, kern, kThreads, dsm);
-        per = pk < per ? pk : per;
-    }
+    // blocks (64 KB of shared memory each) fit on an SM
+    const void *kern = solve_kernel(fp64, tc);
+    cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsm);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, kThreads, dsm);
     if (per < 1 || sms < 1) return 0;
     const int g = sms * (per < kBlocksPerSM ? per : kBlocksPerSM);
     return g <= kMaxSolveGrid ? g : 0;
@@ -1345,7 +1417,7 @@ static cudaError_t solve_buf_t(const SolveBuffers &b, const double *M, const dou
                                sfft_solve_info *info, cudaStream_t st) {
     BatchArgs<T> ba;
     ba.nsys = 1;
-    ba.sys[0] = system_args<T>(b.n, M, rhs, x, info, b.dsc, b.xw, b.r, b.A, b.W, b.zv, b.flag);
+    ba.sys[0] = system_args<T>(b.n, M, rhs, x, info, b.dsc, b.xw, b.r, b.A, b.zv, b.flag);
     return launch_batch(ba, b.grid, st);
 }
 

@@ -2,8 +2,8 @@
 // on a workspace held in a file-scope device array, so that no call
 // allocates memory.
 //
-// The array holds SFFT_SOLVE_STATIC_MAX_N^2 doubles twice (the scaled matrix
-// A and W = L^-1) plus 256 KiB for the vectors: 16.25 MiB per device, owned
+// The array holds SFFT_SOLVE_STATIC_MAX_N^2 doubles twice (the tiles of the
+// factor and its inverse, a panel and diagonal blocks) plus 256 KiB for the vectors: 16.25 MiB per device, owned
 // by this translation unit's module and placed by the CUDA driver when the
 // module is loaded.  Each call lays the workspace for its own n out from the
 // start of the array.  Nothing in it has to start at zero: the solve kernel
@@ -99,8 +99,7 @@ int sfft_solve_static(const double *d_M, const double *d_rhs, int32_t n, int32_t
     b.n = n;
     b.fp64 = fp64;
     b.grid = d->grid[fp64 ? 1 : 0];
-    b.A = take(nn * nn * rsz);
-    b.W = take(nn * nn * rsz);
+    b.A = take(sfft::solve_matrix_elems(n, fp64) * rsz);
     b.zv = take(sfft::solve_vec_elems(n) * rsz);
     b.dsc = reinterpret_cast<double *>(take(nn * sizeof(double)));
     b.r = reinterpret_cast<double *>(take(nn * sizeof(double)));
