@@ -35,7 +35,7 @@
 // What bounds it (n = 1735, 27 steps): one system alone by the step's latency
 // (the chain, or P, one to three rounds of tiles and two grid barriers);
 // eight systems by the tiles' FP32 products and their shared-memory reads.
-// One system 907 -> 545 us, eight of 507 to 1735 unknowns 1510 -> 947 us against
+// One system 907 -> 515 us, eight of 507 to 1735 unknowns 1510 -> 913 us against
 // 32-wide steps with two whole-grid barriers, the chain inside phase U.
 //   * refinement: residual GEMV in FP64 and two GEMVs with W.
 // Every control decision after a barrier uses values written before it, so
@@ -72,7 +72,8 @@ struct Shape {
     static constexpr int TS = sizeof(T) == 4 ? kTile : kDB;
     static constexpr int R = TS / 16;
     static constexpr int KV = 16 / sizeof(T);
-    static constexpr int LDD = kDB + KV;         // pitch of a 32 x 32 block held by the chain
+    static constexpr int LDD = kDB + KV;  // pitch of a 32 x 32 block in shared memory
+    static constexpr int LDT = TS + KV;   // pitch of a TS x TS tile held by the chain
     static constexpr int kDiag = TS == kDB ? 1 : 3;  // blocks of a diagonal block: D1, D2, L21
 };
 
@@ -153,23 +154,59 @@ __device__ __forceinline__ void tile_mul(T (&acc)[Shape<T>::R][Shape<T>::R], con
     }
 }
 
-// acc(v) = sum_p a[p * astep] b[p * bstep + v], p < 32 in order: a points at
-// this lane's row, b at this warp's NC columns
-template <typename T, int NC>
-__device__ __forceinline__ void lane_mul(T (&acc)[NC], const T *a, int astep, const T *b, int bstep) {
-    constexpr int KV = Shape<T>::KV;
-#pragma unroll
-    for (int v = 0; v < NC; ++v) acc[v] = (T)0;
+// 32 x 32 product by a team of threads (t: number in it): out(i, j) = or -=
+// sum_p a[p][i] b[p][j], p < 32 in order; out is kept as out[j][i].  Four rows
+// and CU columns per thread: 64 threads of 4 x 4 wait for shared memory (1500
+// cycles), 256 of 4 x 1 for its throughput (1260; a 16-byte read costs four
+// cycles even where lanes share it); 128 of 4 x 2 lie between.  FP64 is bound
+// by its units, which all threads share.  Not inlined: the chain calls it ten
+// times a step and finds its code in the cache.
+template <typename T, bool SUB, int TEAM>
+__device__ __noinline__ void unit(const T *a, int pa, const T *b, int pb, T *out, int po, int t) {
+    using S = Shape<T>;
+    constexpr int KV = S::KV, CU = kDB * kDB / 4 / TEAM;
+    a += 4 * (t & 7);
+    b += CU * (t >> 3);
+    T acc[4][CU] = {};
 #pragma unroll 8
     for (int p = 0; p < kDB; ++p) {
-        const T av = a[p * astep];
+        T av[4], bv[CU];
 #pragma unroll
-        for (int v = 0; v < NC; v += KV) {
-            const Vec<T> w = ldv(b + p * bstep + v);
+        for (int u = 0; u < 4; u += KV) {
+            const Vec<T> w = ldv(a + p * pa + u);
 #pragma unroll
-            for (int i = 0; i < KV; ++i) acc[v + i] += av * w.v[i];
+            for (int i = 0; i < KV; ++i) av[u + i] = w.v[i];
         }
+        if constexpr (CU == 1) {
+            bv[0] = b[p * pb];
+        } else if constexpr (CU == 2) {
+            const cpx<T> w = *reinterpret_cast<const cpx<T> *>(b + p * pb);
+            bv[0] = w.re;
+            bv[1] = w.im;
+        } else {
+#pragma unroll
+            for (int v = 0; v < CU; v += KV) {
+                const Vec<T> w = ldv(b + p * pb + v);
+#pragma unroll
+                for (int i = 0; i < KV; ++i) bv[v + i] = w.v[i];
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int v = 0; v < CU; ++v) acc[u][v] += av[u] * bv[v];
     }
+    out += CU * (t >> 3) * po + 4 * (t & 7);
+#pragma unroll
+    for (int v = 0; v < CU; ++v)
+#pragma unroll
+        for (int u = 0; u < 4; u += KV) {
+            Vec<T> w, o;
+            if (SUB) o = ldv(out + v * po + u);
+#pragma unroll
+            for (int i = 0; i < KV; ++i) w.v[i] = SUB ? o.v[i] - acc[u + i][v] : acc[u + i][v];
+            stv(out + v * po + u, w);
+        }
 }
 
 // ---- the FP32 tile GEMM on the tensor cores (tcgen05, sm_100 family) --------
@@ -397,9 +434,15 @@ __device__ __forceinline__ void bar_arrive(int id, int threads) {
 // to dt[c * ldd + r], zeros above the diagonal included.  Rows nb and up are
 // the identity's (the caller sets them); a pivot that is not positive sets
 // bad; minpiv takes the smallest of the rest.  Bound by the chain of pivots.
-// (5.2 k cycles; a whole block taking four columns a step, with a barrier and
-// an exchange each, took 12 k.)
-constexpr int kExStep = kDB * 4 + 4;
+// (About 4.5 k cycles; a whole block taking four columns a step, with a
+// barrier and an exchange each, took 12 k.)
+// The steps are a loop of short code (the columns move down by four registers
+// a step; 28 columns are updated in each of the first four steps and 12 in
+// each of the last four, dead ones among them): unrolled, the code ran once a
+// call and waited for its instructions.  In FP64 the updates take 64 cycles an
+// instruction, so there the loop is unrolled and the dead columns left out.
+constexpr int kExRows = kDB + 12;  // rows of ex: those of dead columns are read, not used
+constexpr int kExStep = kExRows * 4 + 4;
 template <typename T>
 __device__ __forceinline__ void get4(const T *p, T (&o)[4]) {
 #pragma unroll
@@ -430,82 +473,107 @@ __device__ __forceinline__ void lrow(const T (&r)[4], T i0, T i1, T i2, T i3, T 
     l[3] = (r[3] - l[0] * l30 - l[1] * l31 - l[2] * l32) * i3;
 }
 
-template <typename T>
-__device__ __noinline__ void factor_rows(const T *s, int lds, T *ex, int nb, bool &bad, T &minpiv) {
+template <typename T, int N>
+__device__ __forceinline__ void factor_steps(T (&a)[N], int jb0, T *ex, int nb, bool &bad, T &low) {
     constexpr unsigned kAll = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    T a[kDB], low = (T)1e30;
-#pragma unroll
-    for (int c = 0; c < kDB; ++c) a[c] = s[lane * lds + c];
-#pragma unroll
-    for (int jb = 0; jb < kDB; jb += 4) {
+    constexpr int U = sizeof(T) == 4 ? 1 : 4;
+#pragma unroll U
+    for (int jb = jb0; jb < jb0 + 16; jb += 4) {
         T pv[4][4];  // rows jb..jb+3 of the pivot block
 #pragma unroll
         for (int r = 0; r < 4; ++r)
 #pragma unroll
-            for (int c = 0; c <= r; ++c) pv[r][c] = __shfl_sync(kAll, a[jb + c], jb + r);
+            for (int c = 0; c <= r; ++c) pv[r][c] = __shfl_sync(kAll, a[c], jb + r);
         const T d0 = pv[0][0];
-        const T i0 = inv_sqrt(d0 > (T)0 ? d0 : (T)1);
+        const T i0 = inv_sqrt(d0);
         const T l10 = pv[1][0] * i0, l20 = pv[2][0] * i0, l30 = pv[3][0] * i0;
         const T d1 = pv[1][1] - l10 * l10;
-        const T i1 = inv_sqrt(d1 > (T)0 ? d1 : (T)1);
+        const T i1 = inv_sqrt(d1);
         const T l21 = (pv[2][1] - l20 * l10) * i1, l31 = (pv[3][1] - l30 * l10) * i1;
         const T d2 = pv[2][2] - l20 * l20 - l21 * l21;
-        const T i2 = inv_sqrt(d2 > (T)0 ? d2 : (T)1);
+        const T i2 = inv_sqrt(d2);
         const T l32 = (pv[3][2] - l30 * l20 - l31 * l21) * i2;
         const T d3 = pv[3][3] - l30 * l30 - l31 * l31 - l32 * l32;
-        const T i3 = inv_sqrt(d3 > (T)0 ? d3 : (T)1);
-        const T r[4] = {a[jb], a[jb + 1], a[jb + 2], a[jb + 3]};
+        const T i3 = inv_sqrt(d3);
+        const T r[4] = {a[0], a[1], a[2], a[3]};
         T lt[4];
         lrow(r, i0, i1, i2, i3, l10, l20, l21, l30, l31, l32, lt);
         T *e = ex + (jb >> 2) * kExStep;
         put4(e + lane * 4, lt);
         if (lane == 0) {
             const T iv[4] = {i0, i1, i2, i3};
-            put4(e + kDB * 4, iv);
+            put4(e + kExRows * 4, iv);
         }
         __syncwarp();
         bar_arrive(1 + (jb >> 2), 64);
+        e += (jb + 4) * 4;
+#pragma unroll
+        for (int c = 4; c < N; ++c) {
+            if (sizeof(T) == 8 && c >= N - (jb - jb0)) continue;
+            T lc[4];
+            get4(e + (c - 4) * 4, lc);
+            a[c - 4] = a[c] - (lt[0] * lc[0] + lt[1] * lc[1] + lt[2] * lc[2] + lt[3] * lc[3]);
+        }
         const T dp[4] = {d0, d1, d2, d3};
 #pragma unroll
         for (int p = 0; p < 4; ++p) {
             if (!(dp[p] > (T)0)) bad = true;
             if (jb + p < nb && dp[p] < low) low = dp[p];
         }
+    }
+}
+// (s: the block by columns, pitch lds)
+template <typename T>
+__device__ __noinline__ void factor_rows(const T *s, int lds, T *ex, int nb, bool &bad, T &minpiv) {
+    const int lane = threadIdx.x & 31;
+    T a[kDB], low = (T)1e30;
 #pragma unroll
-        for (int c = jb + 4; c < kDB; ++c) {
+    for (int c = 0; c < kDB; ++c) a[c] = s[c * lds + lane];
+    bool neg = bad;
+    factor_steps(a, 0, ex, nb, neg, low);
+    T a2[kDB / 2];
+#pragma unroll
+    for (int c = 0; c < kDB / 2; ++c) a2[c] = a[c];
+    factor_steps(a2, 16, ex, nb, neg, low);
+    bad = neg;
+    if (!neg && low < minpiv) minpiv = low;
+}
+template <typename T, int N>
+__device__ __forceinline__ void invert_steps(T (&y)[N], int jb0, const T *ex, T *dt) {
+    constexpr int U = sizeof(T) == 4 ? 1 : 4;
+#pragma unroll U
+    for (int jb = jb0; jb < jb0 + 16; jb += 4) {
+        const T *e = ex + (jb >> 2) * kExStep;
+        bar_sync(1 + (jb >> 2), 64);
+        T iv[4], l1[4], l2[4], l3[4], x[4];
+        get4(e + kExRows * 4, iv);
+        e += jb * 4;
+        get4(e + 4, l1);
+        get4(e + 8, l2);
+        get4(e + 12, l3);
+        const T r[4] = {y[0], y[1], y[2], y[3]};
+        lrow(r, iv[0], iv[1], iv[2], iv[3], l1[0], l2[0], l2[1], l3[0], l3[1], l3[2], x);
+        put4(dt + jb, x);
+#pragma unroll
+        for (int c = 4; c < N; ++c) {
+            if (sizeof(T) == 8 && c >= N - (jb - jb0)) continue;
             T lc[4];
             get4(e + c * 4, lc);
-            a[c] -= lt[0] * lc[0] + lt[1] * lc[1] + lt[2] * lc[2] + lt[3] * lc[3];
+            y[c - 4] = y[c] - (lc[0] * x[0] + lc[1] * x[1] + lc[2] * x[2] + lc[3] * x[3]);
         }
     }
-    if (!bad && low < minpiv) minpiv = low;
 }
 template <typename T>
 __device__ __noinline__ void invert_rows(const T *ex, T *dt, int ldd) {
     const int lane = threadIdx.x & 31;
-    T y[kDB];
+    T y[kDB], y2[kDB / 2];
 #pragma unroll
     for (int c = 0; c < kDB; ++c) y[c] = c == lane ? (T)1 : (T)0;
+    invert_steps(y, 0, ex, dt + lane * ldd);
 #pragma unroll
-    for (int jb = 0; jb < kDB; jb += 4) {
-        const T *e = ex + (jb >> 2) * kExStep;
-        bar_sync(1 + (jb >> 2), 64);
-        T iv[4], l1[4], l2[4], l3[4], x[4];
-        get4(e + kDB * 4, iv);
-        get4(e + (jb + 1) * 4, l1);
-        get4(e + (jb + 2) * 4, l2);
-        get4(e + (jb + 3) * 4, l3);
-        const T r[4] = {y[jb], y[jb + 1], y[jb + 2], y[jb + 3]};
-        lrow(r, iv[0], iv[1], iv[2], iv[3], l1[0], l2[0], l2[1], l3[0], l3[1], l3[2], x);
-        put4(dt + lane * ldd + jb, x);
-#pragma unroll
-        for (int c = jb + 4; c < kDB; ++c) {
-            T lc[4];
-            get4(e + c * 4, lc);
-            y[c] -= lc[0] * x[0] + lc[1] * x[1] + lc[2] * x[2] + lc[3] * x[3];
-        }
-    }
+    for (int c = 0; c < kDB / 2; ++c) y2[c] = y[c];
+    invert_steps(y2, 16, ex, dt + lane * ldd);
 }
 
 // Shared memory of the block that forms the diagonal blocks of its system.
@@ -515,126 +583,110 @@ template <typename T>
 struct ChainSmem {
     using S = Shape<T>;
     T d[S::kDiag][kDB * S::LDD];
-    T d1[kDB * S::LDD];  // the new D1 while the old one is in use
-    T xt[S::TS * S::TS];  // X(k+1, k) by columns
-    T lt[S::TS * S::TS];  // L_{k+1,k} by columns
+    T d1[kDB * S::LDD];    // the new D1 while the old one is in use
+    T xt[S::TS * S::LDT];  // X(k+1, k) by columns
+    T lt[S::TS * S::LDT];  // L_{k+1,k} by columns
+    T s[S::TS * S::LDT];   // X(k+1, k+1) by columns
     T ex[8 * kExStep];
-    T s[S::TS * (S::TS + 1)];  // X(k+1, k+1) by rows
 };
 
-// 32 rows (from row r0; a lane each) and this warp's NC columns from c0 of the
-// products that give L_{k+1,k}, each followed by sync()
-template <typename T, int NC, typename F>
-__device__ __forceinline__ void chain_panel(ChainSmem<T> &c, int r0, int c0, F sync) {
+// The 32 rows a..a+31 of a panel from those of X = [X1 X2] (by columns, pitch
+// px): L1 = X1 D1^T; X2 -= L1 L21^T; L2 = X2 D2^T into l1 and l2 (by columns,
+// pitch pl), each followed by sync()
+template <typename T, int TEAM, typename F>
+__device__ __forceinline__ void panel_rows(T *x, int px, const T (*d)[kDB * Shape<T>::LDD], T *l1, T *l2, int pl,
+                                           int t, F sync) {
     using S = Shape<T>;
-    constexpr int TS = S::TS, LDD = S::LDD;
-    const int i = r0 + (threadIdx.x & 31);
-    T o[NC];
-    lane_mul<T, NC>(o, c.xt + i, TS, c.d[0] + c0, LDD);  // L1(i, p) = sum_q X1(i, q) D1(p, q)
-#pragma unroll
-    for (int v = 0; v < NC; ++v) c.lt[(c0 + v) * TS + i] = o[v];
+    unit<T, false, TEAM>(x, px, d[0], S::LDD, l1, pl, t);
     sync();
-    if constexpr (TS == 2 * kDB) {
-        T *x2 = c.xt + kDB * TS;
-        lane_mul<T, NC>(o, c.lt + i, TS, c.d[2] + c0, LDD);  // X2 -= L1 L21^T
-#pragma unroll
-        for (int v = 0; v < NC; ++v) x2[(c0 + v) * TS + i] -= o[v];
+    if constexpr (S::kDiag == 3) {
+        unit<T, true, TEAM>(l1, pl, d[2], S::LDD, x + kDB * px, px, t);
         sync();
-        lane_mul<T, NC>(o, x2 + i, TS, c.d[1] + c0, LDD);  // L2 = X2 D2^T
-#pragma unroll
-        for (int v = 0; v < NC; ++v) c.lt[(kDB + c0 + v) * TS + i] = o[v];
+        unit<T, false, TEAM>(x + kDB * px, px, d[1], S::LDD, l2, pl, t);
         sync();
-    }
-}
-// the same rows and columns (from j0) of the diagonal block's last update
-template <typename T, int NC>
-__device__ __forceinline__ void chain_update(ChainSmem<T> &c, int r0, int j0) {
-    using S = Shape<T>;
-    constexpr int TS = S::TS, LDS = TS + 1;
-    const int i = r0 + (threadIdx.x & 31);
-    T *s = c.s + i * LDS + j0;
-#pragma unroll
-    for (int h = 0; h < TS / kDB; ++h) {
-        const T *l = c.lt + h * kDB * TS;
-        T o[NC];
-        lane_mul<T, NC>(o, l + i, TS, l + j0, TS);
-#pragma unroll
-        for (int v = 0; v < NC; ++v) s[v] -= o[v];
     }
 }
 
 // Forms diagonal block kb: with `update` its last update from step kb - 1
 // (whose blocks are in c.d) first; then its own blocks into c.d and
-// s.D[kb & 1].  arrive() is called once both tiles have been read.  The first
-// 32 rows go first; warps 4..7 update the other rows while warps 0 and 1
-// factor.
+// s.D[kb & 1].  arrive() is called once both tiles have been read.  For TS =
+// 64 warps 0, 1, 4 and 5 take the first 32 rows and the first two factor them,
+// while warps 2, 3, 6 and 7 (on the other schedulers) update the rest.
+constexpr int kBarTeam = 10, kBarFirst = 11;  // named barriers of the chain
 template <typename T, typename F>
 __device__ __forceinline__ void chain_block(const SolveArgs<T> &s, ChainSmem<T> &c, int kb, bool update, bool &bad,
                                             T &minpiv, F arrive) {
     using S = Shape<T>;
-    constexpr int TS = S::TS, KV = S::KV, LDD = S::LDD, LDS = TS + 1, NV = TS * TS / KV / kThreads, VR = TS / KV;
+    constexpr int TS = S::TS, KV = S::KV, LDD = S::LDD, LDT = S::LDT, NV = TS * TS / KV / kThreads, RG = TS / 8;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int k0 = kb * TS, nb = min(TS, s.n - k0), ld = s.ld;
+    // tiles by columns: a warp reads 64 bytes of 8 rows
     Vec<T> sv[NV], xv[NV];
-    if (update) {
+    auto row = [&](int q) { return ((warp + 8 * q) % RG) * 8 + (lane & 7); };
+    auto col = [&](int q) { return (((warp + 8 * q) / RG) * 4 + (lane >> 3)) * KV; };
 #pragma unroll
-        for (int q = 0; q < NV; ++q) {
-            const int e = tid + q * kThreads, i = e % TS, g = e / TS;
-            xv[q] = ldg_cg(s.X + (size_t)(k0 + i) * ld + k0 - TS + g * KV);
-        }
+    for (int q = 0; q < NV; ++q) {
+        const T *X = s.X + (size_t)(k0 + row(q)) * ld + k0 + col(q);
+        if (update) xv[q] = ldg_cg(X - TS);
+        sv[q] = ldg_cg(X);
     }
 #pragma unroll
     for (int q = 0; q < NV; ++q) {
-        const int e = tid + q * kThreads;
-        sv[q] = ldg_cg(s.X + (size_t)(k0 + e / VR) * ld + k0 + (e % VR) * KV);
-    }
-    if (update) {
+        const int r = row(q), j = col(q);
 #pragma unroll
-        for (int q = 0; q < NV; ++q) {
-            const int e = tid + q * kThreads, i = e % TS, g = e / TS;
-#pragma unroll
-            for (int v = 0; v < KV; ++v) c.xt[(g * KV + v) * TS + i] = xv[q].v[v];
+        for (int v = 0; v < KV; ++v) {
+            if (update) c.xt[(j + v) * LDT + r] = xv[q].v[v];
+            c.s[(j + v) * LDT + r] = r < nb ? sv[q].v[v] : (r == j + v ? (T)1 : (T)0);
         }
-    }
-#pragma unroll
-    for (int q = 0; q < NV; ++q) {
-        const int e = tid + q * kThreads, r = e / VR, j = (e % VR) * KV;
-#pragma unroll
-        for (int v = 0; v < KV; ++v) c.s[r * LDS + j + v] = r < nb ? sv[q].v[v] : (r == j + v ? (T)1 : (T)0);
     }
     __syncthreads();
     arrive();
-    if (update) {
-        chain_panel<T, 4>(c, 0, 4 * warp, [] { __syncthreads(); });
-        chain_update<T, 4>(c, 0, 4 * warp);
-        __syncthreads();
-    }
-    if (warp == 0) factor_rows<T>(c.s, LDS, c.ex, nb, bad, minpiv);
-    else if (warp == 1) invert_rows<T>(c.ex, c.d1, LDD);  // (the other warps still read the old D1)
-    if constexpr (TS == 2 * kDB) {
-        if (update && warp >= 4) {
-            chain_panel<T, 8>(c, kDB, 8 * (warp - 4), [] { bar_sync(kBarHelp, 128); });
-            chain_update<T, 8>(c, kDB, 8 * (warp - 4));
-            chain_update<T, 8>(c, kDB, kDB + 8 * (warp - 4));
+    if constexpr (TS == kDB) {
+        if (update) {
+            panel_rows<T, kThreads>(c.xt, LDT, c.d, c.lt, c.lt, LDT, tid, [] { __syncthreads(); });
+            unit<T, true, kThreads>(c.lt, LDT, c.lt, LDT, c.s, LDT, tid);
+            __syncthreads();
         }
+        if (warp == 0) factor_rows<T>(c.s, LDT, c.ex, nb, bad, minpiv);
+        else if (warp == 1) invert_rows<T>(c.ex, c.d[0], LDD);
+        __syncthreads();
+    } else {
+        T *l2 = c.lt + kDB * LDT;
+        const int t = (warp >> 2) * 64 + (tid & 63);  // number in the team
+        if (!(warp & 2)) {
+            if (update) {
+                panel_rows<T, 128>(c.xt, LDT, c.d, c.lt, l2, LDT, t, [] { bar_sync(kBarTeam, 128); });
+                bar_arrive(kBarFirst, 256);
+                unit<T, true, 128>(c.lt, LDT, c.lt, LDT, c.s, LDT, t);
+                unit<T, true, 128>(l2, LDT, l2, LDT, c.s, LDT, t);
+                bar_sync(kBarTeam, 128);
+            }
+            if (warp == 0) factor_rows<T>(c.s, LDT, c.ex, nb, bad, minpiv);
+            else if (warp == 1) invert_rows<T>(c.ex, c.d1, LDD);
+        } else if (update) {
+            bar_sync(kBarFirst, 256);  // the first rows' panel
+            panel_rows<T, 128>(c.xt + kDB, LDT, c.d, c.lt + kDB, l2 + kDB, LDT, t, [] { bar_sync(kBarHelp, 128); });
+#pragma unroll 1
+            for (int j0 = 0; j0 < TS; j0 += kDB) {  // S21, S22
+                T *out = c.s + j0 * LDT + kDB;
+                unit<T, true, 128>(c.lt + kDB, LDT, c.lt + j0, LDT, out, LDT, t);
+                unit<T, true, 128>(l2 + kDB, LDT, l2 + j0, LDT, out, LDT, t);
+            }
+        }
+        __syncthreads();
+        if (!(warp & 2)) {
+            T *s22 = c.s + kDB * LDT + kDB;
+            unit<T, false, 128>(c.s + kDB, LDT, c.d1, LDD, c.d[2], LDD, t);  // L21 = A21 D1^T
+            bar_sync(kBarTeam, 128);
+            unit<T, true, 128>(c.d[2], LDD, c.d[2], LDD, s22, LDT, t);  // A22 -= L21 L21^T
+            bar_sync(kBarTeam, 128);
+            if (warp == 0) factor_rows<T>(s22, LDT, c.ex, nb - kDB, bad, minpiv);
+            else if (warp == 1) invert_rows<T>(c.ex, c.d[1], LDD);
+        } else {
+            for (int e = t; e < kDB * LDD / KV; e += 128) stv(c.d[0] + e * KV, ldv(c.d1 + e * KV));
+        }
+        __syncthreads();
     }
-    __syncthreads();
-    for (int e = tid; e < kDB * LDD / KV; e += kThreads) stv(c.d[0] + e * KV, ldv(c.d1 + e * KV));
-    if constexpr (TS == 2 * kDB) {
-        T w[4];
-        lane_mul<T, 4>(w, c.s + (kDB + lane) * LDS, 1, c.d1 + 4 * warp, LDD);  // L21 = A21 D1^T
-#pragma unroll
-        for (int v = 0; v < 4; ++v) c.d[2][(4 * warp + v) * LDD + lane] = w[v];
-        __syncthreads();
-        lane_mul<T, 4>(w, c.d[2] + lane, LDD, c.d[2] + 4 * warp, LDD);  // A22 -= L21 L21^T
-#pragma unroll
-        for (int v = 0; v < 4; ++v) c.s[(kDB + lane) * LDS + kDB + 4 * warp + v] -= w[v];
-        __syncthreads();
-        if (warp == 0) factor_rows<T>(c.s + kDB * LDS + kDB, LDS, c.ex, nb - kDB, bad, minpiv);
-        else if (warp == 1) invert_rows<T>(c.ex, c.d[1], LDD);
-        __syncthreads();
-    }
-    if constexpr (TS == kDB) __syncthreads();
     T *D = s.D + (size_t)(kb & 1) * S::kDiag * kDB * kDB;
     for (int e = tid; e < S::kDiag * kDB * kDB / KV; e += kThreads) {
         const int q = e / (kDB / KV), g = e % (kDB / KV);
@@ -644,18 +696,18 @@ __device__ __forceinline__ void chain_block(const SolveArgs<T> &s, ChainSmem<T> 
     __syncthreads();
 }
 
-// Phase P task: 32 columns of the panel of step kb (column `lane` and rows
-// 4 warp + v per thread).
+// Phase P task: 32 columns of the panel of step kb.
 template <typename T>
 struct PanelSmem {
-    T d[Shape<T>::kDiag][kDB * kDB];
-    T x[Shape<T>::TS][kDB];  // X1, X2: the chunk's rows q of X(k, :), or its columns of X(:, k)
-    T p1[kDB][kDB];
+    using S = Shape<T>;
+    T d[S::kDiag][kDB * S::LDD];
+    T x[S::TS * S::LDD];  // [q][c]: the chunk's columns of X(k, :), or its rows of X(:, k)
+    T p[S::TS * S::LDD];  // [p][c]
 };
 template <typename T>
 __device__ __forceinline__ void panel_task(const SolveArgs<T> &s, PanelSmem<T> &sm, int kb, int task) {
     using S = Shape<T>;
-    constexpr int TS = S::TS, KV = S::KV, H = TS / kDB, VR = kDB / KV;
+    constexpr int TS = S::TS, KV = S::KV, LDD = S::LDD, VR = kDB / KV;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, ld = s.ld;
     const int k0 = kb * TS, c0 = task * kDB;
     const T *D = s.D + (size_t)(kb & 1) * S::kDiag * kDB * kDB;
@@ -663,63 +715,67 @@ __device__ __forceinline__ void panel_task(const SolveArgs<T> &s, PanelSmem<T> &
     Vec<T> dv[ND], xv[NX];
 #pragma unroll
     for (int q = 0; q < ND; ++q) dv[q] = ldg_cg(D + (size_t)(tid + q * kThreads) * KV);
-    const int half = (c0 - k0) / kDB;  // of the diagonal block (diag)
-    const bool diag = c0 >= k0 && c0 < k0 + TS;
+    const bool diag = c0 >= k0 && c0 < k0 + TS, upper = c0 < k0;
+    const int h0 = c0 - k0;  // (diag) first of the chunk's columns in the block
+    // after block k the rows of X(:, k), transposed: a warp reads 64 bytes of 8 rows
+    auto row = [&](int q) { return ((warp + 8 * q) & 3) * 8 + (lane & 7); };
+    auto col = [&](int q) { return (((warp + 8 * q) >> 2) * 4 + (lane >> 3)) * KV; };
+    if (!diag) {
 #pragma unroll
-    for (int q = 0; q < NX; ++q) {
-        const int e = tid + q * kThreads;
-        if (diag) xv[q] = {};
-        else
-            xv[q] = c0 < k0 ? ldg_cg(s.X + (size_t)(k0 + e / VR) * ld + c0 + (e % VR) * KV)
-                            : ldg_cg(s.X + (size_t)(c0 + lane) * ld + k0 + (e / kDB) * KV);
+        for (int q = 0; q < NX; ++q) {
+            const int e = tid + q * kThreads;
+            xv[q] = upper ? ldg_cg(s.X + (size_t)(k0 + e / VR) * ld + c0 + (e % VR) * KV)
+                          : ldg_cg(s.X + (size_t)(c0 + row(q)) * ld + k0 + col(q));
+        }
     }
     __syncthreads();  // the reads of the task before are done
 #pragma unroll
-    for (int q = 0; q < ND; ++q) stv(sm.d[0] + (tid + q * kThreads) * KV, dv[q]);
-#pragma unroll
-    for (int q = 0; q < NX; ++q) {
+    for (int q = 0; q < ND; ++q) {
         const int e = tid + q * kThreads;
-        if (c0 < k0 || diag) {
-            stv(&sm.x[0][0] + e * KV, xv[q]);
-        } else {
+        stv(sm.d[0] + (e / VR) * LDD + (e % VR) * KV, dv[q]);
+    }
+    if (!diag) {
 #pragma unroll
-            for (int v = 0; v < KV; ++v) sm.x[(e / kDB) * KV + v][lane] = xv[q].v[v];
+        for (int q = 0; q < NX; ++q) {
+            const int e = tid + q * kThreads;
+            if (upper) {
+                stv(sm.x + (e / VR) * LDD + (e % VR) * KV, xv[q]);
+            } else {
+#pragma unroll
+                for (int v = 0; v < KV; ++v) sm.x[(col(q) + v) * LDD + row(q)] = xv[q].v[v];
+            }
         }
     }
     __syncthreads();
-    T o[4];
-    auto store = [&](int row) {
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const int p = row + 4 * warp + v;
-            s.P[(size_t)p * ld + c0 + lane] = o[v];
-            if (c0 < k0 + TS) s.X[(size_t)(k0 + p) * ld + c0 + lane] = o[v];
+    // P1 = D1 X1, P2 = D2 (X2 - L21 P1); in the diagonal block's own columns
+    // [D1; -D2 L21 D1] and [0; D2]
+    if (diag) {
+        for (int e = tid; e < TS * kDB; e += kThreads) {
+            const int p = e / kDB, c = e % kDB;
+            if (p / kDB == h0 / kDB) sm.p[p * LDD + c] = sm.d[h0 / kDB][c * LDD + p % kDB];
+            else if (h0 > 0) sm.p[p * LDD + c] = (T)0;
+            else sm.x[p * LDD + c] = (T)0;  // X2
         }
-    };
-    // P1 = D1 X1; D1 itself in its own columns, zero in those of the second half
-    if (!diag) {
-        lane_mul<T, 4>(o, &sm.x[0][lane], kDB, sm.d[0] + 4 * warp, kDB);
-    } else {
-#pragma unroll
-        for (int v = 0; v < 4; ++v) o[v] = half == 0 ? sm.d[0][lane * kDB + 4 * warp + v] : (T)0;
+        __syncthreads();
     }
-    store(0);
-    if constexpr (H == 2) {
-        // P2 = D2 (X2 - L21 P1), X2 = 0 in the columns of the first half; D2 in its own
-        if (!diag || half == 0) {
-#pragma unroll
-            for (int v = 0; v < 4; ++v) sm.p1[4 * warp + v][lane] = o[v];
-            __syncthreads();
-            lane_mul<T, 4>(o, &sm.p1[0][lane], kDB, sm.d[2] + 4 * warp, kDB);
-#pragma unroll
-            for (int v = 0; v < 4; ++v) sm.x[kDB + 4 * warp + v][lane] -= o[v];
-            __syncthreads();
-            lane_mul<T, 4>(o, &sm.x[kDB][lane], kDB, sm.d[1] + 4 * warp, kDB);
-        } else {
-#pragma unroll
-            for (int v = 0; v < 4; ++v) o[v] = sm.d[1][lane * kDB + 4 * warp + v];
+    auto sync = [] { __syncthreads(); };
+    if (!diag) {
+        panel_rows<T, kThreads>(sm.x, LDD, sm.d, sm.p, sm.p + kDB * LDD, LDD, tid, sync);
+    } else if constexpr (S::kDiag == 3) {
+        if (h0 == 0) {
+            T *x2 = sm.x + kDB * LDD;
+            unit<T, true, kThreads>(sm.p, LDD, sm.d[2], LDD, x2, LDD, tid);
+            sync();
+            unit<T, false, kThreads>(x2, LDD, sm.d[1], LDD, sm.p + kDB * LDD, LDD, tid);
         }
-        store(kDB);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < NX; ++q) {
+        const int e = tid + q * kThreads, p = e / VR, g = (e % VR) * KV;
+        const Vec<T> v = ldv(sm.p + p * LDD + g);
+        stv(s.P + (size_t)p * ld + c0 + g, v);
+        if (upper || diag) stv(s.X + (size_t)(k0 + p) * ld + c0 + g, v);
     }
 }
 
@@ -985,7 +1041,6 @@ struct GridBar {
     __device__ __forceinline__ void arrive(int thread) {  // after the block's work: every thread calls it
         __syncthreads();
         if ((int)threadIdx.x == thread) {
-            __threadfence();
             asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(cnt) : "memory");
         }
         target += gridDim.x;
@@ -1001,7 +1056,6 @@ struct GridBar {
                     break;
                 }
             } while (v < target);
-            __threadfence();
         }
         __syncthreads();
     }
@@ -1010,6 +1064,12 @@ struct GridBar {
         wait();
     }
 };
+
+__device__ __forceinline__ int multiprocessor() {
+    int id;
+    asm volatile("mov.u32 %0, %smid;" : "=r"(id));
+    return id;
+}
 
 template <typename T, bool TC>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kBlocksPerSM : 1) k_solve_coop(BatchArgs<T> ba) {
@@ -1046,6 +1106,8 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kBlocksPerSM : 1) k
     }
     const int nrows_all = nrow[nsys];
 
+    __shared__ int rank_s;
+    int *workers = reinterpret_cast<int *>(ba.sys[0].stats + 4);
     // ---- status reset; Jacobi scaling, zero x and the padding rows of X ------
     if (bid == 0 && tid < nsys) {
         const SolveArgs<T> &s = ba.sys[tid];
@@ -1053,9 +1115,20 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kBlocksPerSM : 1) k
         s.flag[2] = INT_MAX;
         s.stats[0] = 1e300;
         s.stats[1] = s.stats[2] = s.stats[3] = 0.0;
+        if (tid == 0) *workers = 0;
     }
+    // A block that shares its multiprocessor with one that forms diagonal
+    // blocks takes no tasks of the factorisation: the chain would wait for its
+    // instructions.  The others draw their numbers.
+    if (bid < nsys && tid == 0) reinterpret_cast<int *>(ba.sys[bid].stats + 5)[0] = multiprocessor();
     grid.sync();
     GridBar bar{&ba.sys[0].flag[3], 0};
+    if (bid >= nsys && tid == 0) {
+        bool own = true;
+        for (int b = 0; b < nsys; ++b)
+            own = own && reinterpret_cast<const int *>(ba.sys[b].stats + 5)[0] != multiprocessor();
+        rank_s = own ? atomicAdd(workers, 1) : -1;
+    }
     for (int b = 0; b < nsys; ++b) {
         const SolveArgs<T> &s = ba.sys[b];
         const int n = s.n;
@@ -1084,6 +1157,9 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kBlocksPerSM : 1) k
     // the same in every block: a chain that fails while step kb runs records
     // block kb + 1, which the test of step kb reads the same way before and
     // after.
+    // (no worker left: a small grid set by hand; then all share the tasks)
+    const int nown = *workers, nwork = nown > 0 ? nown : nbk - nsys;
+    const int rank = bid < nsys ? -1 : (nown > 0 ? rank_s : bid - nsys);
     bool bad = false;  // of the chain of system bid (thread 0)
     T minpiv = (T)1e30;
     if (bid < nsys && ba.sys[bid].flag[0] == 0) chain_block(ba.sys[bid], sm.chain, 0, false, bad, minpiv, [] {});
@@ -1113,8 +1189,8 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kBlocksPerSM : 1) k
             chain_block(ba.sys[bid], sm.chain, kb + 1, true, bad, minpiv, [&] { bar.arrive(kThreads - 1); });
             bar.wait();
         } else {
-            if (bid >= nsys) {
-                for (int task = bid - nsys; task < poff[nsys]; task += nbk - nsys) {
+            if (rank >= 0) {
+                for (int task = rank; task < poff[nsys]; task += nwork) {
                     const int b = sys_of(poff, nsys, task);
                     panel_task(ba.sys[b], sm.panel, kb, task - poff[b]);
                 }
@@ -1122,10 +1198,10 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kBlocksPerSM : 1) k
             bar.sync();
         }
         if (!more) break;  // every system's steps are done (same in every block)
-        if (bid >= nsys) {
-            const int step = nbk - nsys, total = uoff[nsys];
+        if (rank >= 0) {
+            const int step = nwork, total = uoff[nsys];
             if constexpr (TC && sizeof(T) == 4) {
-                for (int task = bid - nsys; task < total; task += step) {
+                for (int task = rank; task < total; task += step) {
                     const int b = sys_of(uoff, nsys, task);
                     const SolveArgs<T> &s = ba.sys[b];
                     int i, j;
@@ -1154,7 +1230,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kBlocksPerSM : 1) k
                 }
             } else {
                 // the operands of the next tile arrive while this one's product runs
-                int task = bid - nsys, b = 0, i = 0, j = 0, buf = 0;
+                int task = rank, b = 0, i = 0, j = 0, buf = 0;
                 auto fetch = [&](int t, int &fb, int &fi, int &fj, int to) {
                     fb = sys_of(uoff, nsys, t);
                     tile_of(kb, t - uoff[fb], fi, fj);
@@ -1368,10 +1444,9 @@ static cudaError_t solve_batch_t(Plan *const *plans, int count, const double *co
     if (sg > count && sg <= full) {
         grid = sg;  // set by hand
     } else if (count == 1 && !tc && sizeof(T) == 4 && full >= 2 * kMaxSolveBatch) {
-        // one system alone: one block per SM (the step's serial chain, not the
-        // tile throughput, sets its time; 1.12 -> 1.02 ms at n = 1735); several:
-        // every resident block (batches of 8 on 304 blocks measured 561 pairs/s
-        // serving against 515 on 152)
+        // one system alone: one block per SM (the step's latency, not the
+        // tile throughput, sets its time: 582 us on 304 blocks, 515 on 152 at
+        // n = 1735); several: every resident block
         grid = full / kBlocksPerSM;
     }
     const cudaError_t err = launch_batch(ba, grid, st, tc);
