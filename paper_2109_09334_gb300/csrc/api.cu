@@ -167,6 +167,9 @@ void plan_free(Plan *p) {
                     p->bxy64, p->d_zdesc, p->d_rdesc, p->z0, p->cmat, p->unk, p->gam, p->bnd};
     for (void *b : bufs)
         if (b) cudaFree(b);
+    if (p->ev_fork) cudaEventDestroy(p->ev_fork);
+    if (p->ev_join) cudaEventDestroy(p->ev_join);
+    if (p->side) cudaStreamDestroy(p->side);
     free(p->h_int);
     free(p->host_pairs);
     delete p;
@@ -263,6 +266,13 @@ int plan_new(const sfft_config *cfg, cudaStream_t s, Plan **out) {
     p->fp64 = cfg->precision == SFFT_PREC_FP64;
     p->csz = p->fp64 ? sizeof(cpx<double>) : sizeof(cpx<float>);
     p->last_stream = s;
+    if (cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&p->ev_join, cudaEventDisableTiming) != cudaSuccess) {
+        cudaGetLastError();
+        plan_free(p);
+        return SFFT_ERR_CUDA;
+    }
     {
         const int rc = basis_build(p, s);
         if (rc != SFFT_OK) {
@@ -527,9 +537,23 @@ static int run_pair(Plan *p, const void *ref, const void *sci, const uint8_t *ma
     p->last_x = x;
     p->last_info = info;
     p->last_diff = diff;
-    cudaError_t e = build_system(p, ref, sci, mask, M, rhs, s);
-    if (e == cudaSuccess) e = solve_system(p, M, rhs, x, info, s);
-    if (e == cudaSuccess && mask) e = row_transform(p, ref, sci, nullptr, false, s);
+    cudaError_t e = build_system(p, ref, sci, mask, M, rhs, s, p->side);
+    if (e == cudaSuccess && mask) {
+        // the unmasked rows, for the subtraction, beside the lag sums' second
+        // stage and the solve
+        e = cudaStreamWaitEvent(p->side, p->ev_fork, 0);
+        if (e == cudaSuccess) {
+            e = row_transform(p, ref, sci, nullptr, false, p->side);
+            const cudaError_t r = cudaEventRecord(p->ev_join, p->side);
+            if (e == cudaSuccess) e = r;
+            const cudaError_t v = solve_system(p, M, rhs, x, info, s);
+            if (e == cudaSuccess) e = v;
+            const cudaError_t w = cudaStreamWaitEvent(s, p->ev_join, 0);
+            if (e == cudaSuccess) e = w;
+        }
+    } else if (e == cudaSuccess) {
+        e = solve_system(p, M, rhs, x, info, s);
+    }
     if (e == cudaSuccess) e = subtract_from_rows(p, x, diff, s);
     p->last_stream = s;
     return status_of(e);
@@ -637,7 +661,7 @@ int sfft_build_system(sfft_plan_t plan, const void *d_ref, const void *d_sci, co
     if (!images_aligned(d_ref, d_sci, d_mask)) return SFFT_ERR_INVALID;
     Plan *p = (Plan *)plan;
     p->last_stream = (cudaStream_t)stream;
-    return status_of(build_system(p, d_ref, d_sci, d_mask, d_M, d_rhs, (cudaStream_t)stream));
+    return status_of(build_system(p, d_ref, d_sci, d_mask, d_M, d_rhs, (cudaStream_t)stream, p->side));
 }
 
 int sfft_solve(sfft_plan_t plan, const double *d_M, const double *d_rhs, double *d_x, sfft_solve_info *d_info,
@@ -878,7 +902,6 @@ cudaError_t enqueue_pairs(const sfft_plan_t *plans, int32_t count, const void *c
         p->last_info = (d_infos && d_infos[i]) ? d_infos[i] : p->info_own;
         p->last_diff = d_diffs[i];
         p->last_stream = s;
-        e = build_system(p, p->last_ref, p->last_sci, p->last_mask, p->M_own, p->rhs_own, s);
     }
     // A launch lasts as long as its largest system: group the systems by
     // size, largest first (the order of the systems in a launch does not
@@ -887,25 +910,54 @@ cudaError_t enqueue_pairs(const sfft_plan_t *plans, int32_t count, const void *c
     for (int i = 0; i < count; ++i) order[i] = i;
     std::stable_sort(order.begin(), order.end(),
                      [&](int a, int b) { return ((Plan *)plans[a])->n > ((Plan *)plans[b])->n; });
-    for (int g = 0; g < count && e == cudaSuccess; g += group) {
+    // Builds and subtractions of different pairs run side by side on up to
+    // kLanes of the plans' own streams: the small kernels of a pair leave most
+    // multiprocessors idle, and the builds of one group of systems run during
+    // the solve of the group before.  Every lane is joined to s again whatever
+    // fails.  Sixteen sectors of 512 to 2048 pixels: 4.76 -> 3.31 ms on four lanes.
+    constexpr int kLanes = 4;
+    const int lanes = count < kLanes ? count : kLanes;
+    auto first = [&](cudaError_t k) {
+        if (e == cudaSuccess) e = k;
+    };
+    auto plan_at = [&](int q) { return (Plan *)plans[order[q]]; };
+    auto lane = [&](int q) { return ((Plan *)plans[q % lanes])->side; };
+    Plan *head = (Plan *)plans[0];
+    first(cudaEventRecord(head->ev_fork, s));
+    for (int l = 0; l < lanes; ++l) first(cudaStreamWaitEvent(lane(l), head->ev_fork, 0));
+    for (int q = 0; q < count; ++q) {
+        Plan *p = plan_at(q);
+        if (e == cudaSuccess)
+            first(build_system(p, p->last_ref, p->last_sci, p->last_mask, p->M_own, p->rhs_own, lane(q)));
+        first(cudaEventRecord(p->ev_join, lane(q)));  // the system is built
+    }
+    for (int g = 0; g < count; g += group) {
         const int cnt = count - g < group ? count - g : group;
         Plan *ps[kMaxSolveBatch];
         const double *M[kMaxSolveBatch], *rhs[kMaxSolveBatch];
         double *x[kMaxSolveBatch];
         sfft_solve_info *info[kMaxSolveBatch];
         for (int b = 0; b < cnt; ++b) {
-            ps[b] = (Plan *)plans[order[g + b]];
+            ps[b] = plan_at(g + b);
             M[b] = ps[b]->last_M;
             rhs[b] = ps[b]->last_rhs;
             x[b] = ps[b]->last_x;
             info[b] = ps[b]->last_info;
+            first(cudaStreamWaitEvent(s, ps[b]->ev_join, 0));
         }
-        e = solve_batch(ps, cnt, M, rhs, x, info, s);
+        if (e == cudaSuccess) first(solve_batch(ps, cnt, M, rhs, x, info, s));
+        first(cudaEventRecord(ps[0]->ev_fork, s));  // the group is solved
+        for (int b = 0; b < cnt; ++b) {
+            Plan *p = ps[b];
+            first(cudaStreamWaitEvent(lane(g + b), ps[0]->ev_fork, 0));
+            if (e == cudaSuccess && p->last_mask)
+                first(row_transform(p, p->last_ref, p->last_sci, nullptr, false, lane(g + b)));
+            if (e == cudaSuccess) first(subtract_from_rows(p, p->last_x, p->last_diff, lane(g + b)));
+        }
     }
-    for (int i = 0; i < count && e == cudaSuccess; ++i) {
-        Plan *p = (Plan *)plans[i];
-        if (p->last_mask) e = row_transform(p, p->last_ref, p->last_sci, nullptr, false, s);
-        if (e == cudaSuccess) e = subtract_from_rows(p, p->last_x, p->last_diff, s);
+    for (int l = 0; l < lanes; ++l) {
+        first(cudaEventRecord(plan_at(l)->ev_join, lane(l)));
+        first(cudaStreamWaitEvent(s, plan_at(l)->ev_join, 0));
     }
     return e;
 }

@@ -186,6 +186,9 @@ struct Plan {
     sfft_solve_info *last_info;
     void *last_diff;
     cudaStream_t last_stream;
+    // a stream of the plan's own beside the caller's, joined before any call returns
+    cudaStream_t side;
+    cudaEvent_t ev_fork, ev_join;
     PairDesc *host_pairs;  // [npairs]
 };
 
@@ -224,8 +227,10 @@ int basis_build(Plan *p, cudaStream_t s);  // p->n, sizes and cfg set; allocatio
 void basis_term_weights(const Plan *p, double xt0, double yt0, double *w);
 
 // launchers (return cudaError_t of the last launch)
+// side: a second stream for the kernels beside the transforms (the plan's, or
+// null: all on s); p->ev_fork is then recorded where F may be overwritten
 cudaError_t build_system(Plan *p, const void *ref, const void *sci, const uint8_t *mask, double *M,
-                         double *rhs, cudaStream_t s);
+                         double *rhs, cudaStream_t s, cudaStream_t side = nullptr);
 cudaError_t row_transform(Plan *p, const void *ref, const void *sci, const uint8_t *mask,
                           bool moments, cudaStream_t s);
 cudaError_t build_stage(Plan *p, int stage, double *M, double *rhs, cudaStream_t s);
