@@ -65,101 +65,175 @@ __global__ void k_kernel_table(int ylen, BasisView bv, const double *__restrict_
     }
 }
 
-// One block per column m: D~(., m) into Dt[m][x].  Thread t computes the Q
-// consecutive outputs x0 = Q t .. Q t + Q - 1.  For each kernel term (i, j)
-// the weighted column W(x) = xt^i F_j(x, m) is staged in shared memory (one
-// pad element after every Q, so the threads' strided accesses hit distinct
-// banks) and the L0 taps slide a Q-value window over it: one shared load and
-// Q complex multiply-adds per tap.  Q = 4 for FP32, 8 for FP64, so that
-// n0 = 4096 needs at most 1024 (FP32) or 512 (FP64) threads.
+// D~(x, m) into Dt[m][x]: one block per column m and segment of x.  For each
+// kernel term (i, j) the weighted column W(x) = xt^i F_j(x, m) is staged in
+// shared memory over the segment and w0 values on either side, wrapped at the
+// image edge (one pad element after every Q, so that the threads' strided
+// reads hit distinct banks); thread t slides a window of Q values over it for
+// its outputs Q t .. Q t + Q - 1: per tap a read of the kernel value, one of W,
+// and Q complex multiply-adds.  In FP32 these run in packed pairs (real and
+// imaginary part), with the kernel values kept as the pairs (-re, -re) and
+// (im, -im) that acc - k w = acc + (-re) (w.re, w.im) + (im, -im) (w.im, w.re)
+// takes: the roundings of four scalar ones.  Global memory is read and written
+// with consecutive x in consecutive threads; the sums' start S - B and their
+// result pass through shared memory.  Segments of 256 threads: several blocks
+// on a multiprocessor cover each other's loads.  A block for a whole column
+// (1024 threads, scalar multiply-adds) spent half of its time waiting:
+// 257 -> 219 us at 4096 x 4096, w = 8, 6 terms, FP32 (2322 columns of 2046, w =
+// 6: 124 -> 109 us).
 template <typename T>
 __host__ __device__ constexpr int sub_q() { return sizeof(T) == 4 ? 4 : 8; }
+constexpr int kSubThreads = 256;
+template <typename T>
+static int sub_threads(int n0) {
+    const int q = sub_q<T>(), most = sizeof(T) == 4 ? kSubThreads : 64;
+    return (n0 + q - 1) / q < most ? (n0 + q - 1) / q : most;
+}
+template <typename T>
+static size_t sub_smem(const Plan *p) {
+    const int q = sub_q<T>(), len = q * sub_threads<T>(p->n0) + 2 * p->cfg.w0;
+    return ((size_t)(sizeof(T) == 4 ? 2 : 1) * p->nk * p->L0 + 2 * (size_t)(len + len / q + q + 1)) * sizeof(cpx<T>);
+}
 
 // W0 >= 0: the kernel half-width is the compile-time W0 (the tap loop unrolls
 // completely, so the window shifts are register renames); W0 < 0: w0 at run time.
-template <typename T, bool P2, int W0>
-__global__ void __launch_bounds__(sizeof(T) == 4 ? 1024 : 512) k_sub_cols(int n0, int hc, int ncol, int offb, BasisView bv, FTab<T> ft,
-                                                                         int w0, int nbkg_off,
-                                                                         const cpx<T> *__restrict__ F,
-                                                                         const cpx<T> *__restrict__ kap,
-                                                                         const cpx<T> *__restrict__ yhat,
-                                                                         const double *__restrict__ x,
-                                                                         cpx<T> *__restrict__ Dt) {
+template <typename T, int W0>
+__global__ void __launch_bounds__(kSubThreads, sizeof(T) == 4 ? 4 : 1)
+    k_sub_cols(int n0, int hc, int ncol, int offb, BasisView bv, FTab<T> ft, int w0, int nbkg_off,
+               const cpx<T> *__restrict__ F, const cpx<T> *__restrict__ kap, const cpx<T> *__restrict__ yhat,
+               const double *__restrict__ x, cpx<T> *__restrict__ Dt) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr bool PK = sizeof(T) == 4;
+    constexpr int Q = sub_q<T>(), KS = PK ? 2 : 1;
     const int nk = bv.nk, nbt = bv.nb;
     if (W0 >= 0) w0 = W0;
     const int L0 = 2 * w0 + 1;
-    cpx<T> *kp = reinterpret_cast<cpx<T> *>(smem_raw);  // nk * L0
-    constexpr int Q = sub_q<T>();
-    cpx<T> *Wb = kp + nk * L0;  // two buffers of n0 + n0 / Q (padded), alternating by term
     auto padq = [](int v) { return v + v / Q; };
-    const int col = blockIdx.x, m = col % hc, tid = threadIdx.x, nthr = blockDim.x;
-    const int msk = n0 - 1;
-    // index mod n0 for -n0 <= v < 2 n0 (P2: n0 is a power of two)
-    auto wrapx = [&](int v) { return P2 ? (v & msk) : (v < 0 ? v + n0 : (v >= n0 ? v - n0 : v)); };
-    const int x0 = Q * tid;  // outputs x0 .. x0 + Q - 1 below n0
-    for (int e = tid; e < nk * L0; e += nthr) kp[e] = kap[(size_t)e * hc + m];
-    T xt[Q];
-#pragma unroll
-    for (int q = 0; q < Q; ++q) xt[q] = coord<T>(x0 + q, n0);
-    // S~ minus the background B~(x, m) = sum_s b_s bx_p(x) Y_q(m)
-    cpx<T> acc[Q];
-    {
-        const cpx<T> *Sc = F + ((size_t)(offb + bv.nfy) * ncol + col) * n0 + x0;
-#pragma unroll
-        for (int q = 0; q < Q; ++q) acc[q] = (P2 || x0 + q < n0) ? Sc[q] : mk((T)0, (T)0);
-        for (int s = 0; s < nbt; ++s) {
-            const int p = bv.sp(s), qq = bv.sq(s);
-            const cpx<T> yq = yhat[(size_t)qq * ncol + col];
-            const T bpq = (T)x[nbkg_off + s];
-#pragma unroll
-            for (int q = 0; q < Q; ++q) {
-                const T wx = ft.bx ? ((P2 || x0 + q < n0) ? ft.bx[(size_t)p * n0 + x0 + q] : (T)0) : ipow(xt[q], p);
-                acc[q] = csub(acc[q], scale(yq, bpq * wx));
-            }
+    const int tid = threadIdx.x, nthr = blockDim.x;
+    const int col = blockIdx.x, m = col % hc, xb = blockIdx.y * (Q * nthr);
+    const int len = min(Q * nthr, n0 - xb), ext = len + 2 * w0;  // outputs; staged values
+    cpx<T> *kp = reinterpret_cast<cpx<T> *>(smem_raw);  // nk * L0 (in FP32 two pairs each)
+    cpx<T> *Wb = kp + KS * nk * L0;  // two buffers, alternating by term
+    const int wlen = padq(Q * nthr + 2 * w0) + Q + 1;
+    for (int e = tid; e < nk * L0; e += nthr) {
+        const cpx<T> v = kap[(size_t)e * hc + m];
+        if constexpr (PK) {
+            kp[2 * e] = mk(-v.re, -v.re);
+            kp[2 * e + 1] = mk(v.im, -v.im);
+        } else {
+            kp[e] = v;
         }
     }
+    // S~ minus the background B~(x, m) = sum_p bx_p(x) sum_q b_pq Y_q(m)
+    const cpx<T> *Sc = F + ((size_t)(offb + bv.nfy) * ncol + col) * n0 + xb;
+    cpx<T> v[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) v[q] = tid + q * nthr < len ? Sc[tid + q * nthr] : mk((T)0, (T)0);
+    __shared__ cpx<T> bp[kMaxFun];
+    for (int p = tid; p < bv.nbx; p += nthr) {
+        cpx<T> b = mk((T)0, (T)0);
+        for (int s = 0; s < nbt; ++s)
+            if (bv.sp(s) == p) b = cadd(b, scale(yhat[(size_t)bv.sq(s) * ncol + col], (T)x[nbkg_off + s]));
+        bp[p] = b;
+    }
+    __syncthreads();
+    for (int p = 0; p < bv.nbx; ++p) {
+        const T *wx = ft.bx + (size_t)p * n0 + xb + tid;
+        const cpx<T> b = bp[p];
+#pragma unroll
+        for (int q = 0; q < Q; ++q)
+            if (tid + q * nthr < len) v[q] = csub(v[q], scale(b, wx[q * nthr]));
+    }
+#pragma unroll
+    for (int q = 0; q < Q; ++q) Wb[wlen + padq(tid + q * nthr)] = v[q];
+    __syncthreads();
+    cpx<T> acc[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) acc[q] = Wb[wlen + padq(Q * tid) + q];
     // terms grouped by their y-function j: F_j is loaded once per group.  The
     // weighted columns alternate between two buffers, so one barrier per term
     // separates a buffer's fill from its reads and from its refill two terms on.
-    const int wlen = n0 + (n0 + Q - 1) / Q;
+    constexpr int NF = Q + 1;  // staged values per thread (2 w0 <= nthr, or the rest below)
+    auto wrapx = [&](int e) {  // image column of staged value e
+        const int u = xb - w0 + e;
+        return u < 0 ? u + n0 : (u >= n0 ? u - n0 : u);
+    };
+    int xi[NF];
+#pragma unroll
+    for (int q = 0; q < NF; ++q) xi[q] = tid + q * nthr < ext ? wrapx(tid + q * nthr) : -1;
     int nterm = 0;
     for (int j = 0; j < bv.nfy; ++j) {
         const int ncj = bv.jcnt(j);
         if (ncj == 0) continue;
-        cpx<T> f[Q];
-        const cpx<T> *Fj = F + ((size_t)(offb + j) * ncol + col) * n0 + x0;
+        const cpx<T> *Fj = F + ((size_t)(offb + j) * ncol + col) * n0;
+        cpx<T> f[NF];
 #pragma unroll
-        for (int q = 0; q < Q; ++q) f[q] = (P2 || x0 + q < n0) ? Fj[q] : mk((T)0, (T)0);
+        for (int q = 0; q < NF; ++q) f[q] = xi[q] >= 0 ? Fj[xi[q]] : mk((T)0, (T)0);
         for (int k = 0; k < ncj; ++k) {
-            const int t = bv.jterm(j, k), i = bv.ti(t);
+            const int t = bv.jterm(j, k);
+            const T *wx = ft.fx + (size_t)bv.ti(t) * n0;
             cpx<T> *W = Wb + (size_t)(nterm++ & 1) * wlen;
 #pragma unroll
-            for (int q = 0; q < Q; ++q)
-                if (P2 || x0 + q < n0) {
-                    const T wx = ft.fx ? ft.fx[(size_t)i * n0 + x0 + q] : ipow(xt[q], i);
-                    W[padq(x0 + q)] = scale(f[q], wx);
-                }
+            for (int q = 0; q < NF; ++q)
+                if (xi[q] >= 0) W[padq(tid + q * nthr)] = scale(f[q], wx[xi[q]]);
+            for (int e = tid + NF * nthr; e < ext; e += nthr)  // (few threads, wide kernels)
+                W[padq(e)] = scale(Fj[wrapx(e)], wx[wrapx(e)]);
             __syncthreads();  // this buffer is filled; the other one's reads (two terms ago) are done
-            const cpx<T> *kt = kp + t * L0;
-            cpx<T> win[Q];
+            const cpx<T> *kt = kp + KS * t * L0;
+            const cpx<T> *Wt = W + padq(Q * tid);
+            if constexpr (PK) {
+                pair32 pa[Q], win[Q], swp[Q];  // sums; window values (re, im) and (im, re)
+                auto get = [&](int e, pair32 &v, pair32 &w) {
+                    const cpx<T> c = Wt[padq(e)];
+                    v = pack2(c.re, c.im);
+                    w = pack2(c.im, c.re);
+                };
 #pragma unroll
-            for (int q = 0; q < Q; ++q) win[q] = W[padq(wrapx(x0 - w0 + q))];
+                for (int q = 0; q < Q; ++q) {
+                    pa[q] = pack2(acc[q].re, acc[q].im);
+                    get(q, win[q], swp[q]);
+                }
 #pragma unroll
-            for (int a = (W0 >= 0 ? W0 : w0); a >= -(W0 >= 0 ? W0 : w0); --a) {
-                const cpx<T> kv = kt[a + w0];
+                for (int c = 0; c <= 2 * (W0 >= 0 ? W0 : w0); ++c) {  // tap a = w0 - c
+                    const float4 kv = *reinterpret_cast<const float4 *>(kt + 2 * (L0 - 1 - c));
+                    const pair32 kr = pack2(kv.x, kv.y), ki = pack2(kv.z, kv.w);
 #pragma unroll
-                for (int q = 0; q < Q; ++q) acc[q] = cfms(acc[q], kv, win[q]);
+                    for (int q = 0; q < Q; ++q) fma2(pa[q], kr, win[q]);
 #pragma unroll
-                for (int q = 0; q + 1 < Q; ++q) win[q] = win[q + 1];
-                win[Q - 1] = W[padq(wrapx(x0 + Q - a))];
+                    for (int q = 0; q < Q; ++q) fma2(pa[q], ki, swp[q]);
+#pragma unroll
+                    for (int q = 0; q + 1 < Q; ++q) {
+                        win[q] = win[q + 1];
+                        swp[q] = swp[q + 1];
+                    }
+                    get(Q + c, win[Q - 1], swp[Q - 1]);
+                }
+#pragma unroll
+                for (int q = 0; q < Q; ++q) acc[q] = unpack2(pa[q]);
+            } else {
+                cpx<T> win[Q];
+#pragma unroll
+                for (int q = 0; q < Q; ++q) win[q] = Wt[padq(q)];
+#pragma unroll
+                for (int c = 0; c <= 2 * (W0 >= 0 ? W0 : w0); ++c) {
+                    const cpx<T> kv = kt[L0 - 1 - c];
+#pragma unroll
+                    for (int q = 0; q < Q; ++q) acc[q] = cfms(acc[q], kv, win[q]);
+#pragma unroll
+                    for (int q = 0; q + 1 < Q; ++q) win[q] = win[q + 1];
+                    win[Q - 1] = Wt[padq(Q + c)];
+                }
             }
         }
     }
-    cpx<T> *out = Dt + (size_t)col * n0 + x0;
+    cpx<T> *W = Wb + (size_t)(nterm & 1) * wlen;  // (last read two terms ago)
+#pragma unroll
+    for (int q = 0; q < Q; ++q) W[padq(Q * tid) + q] = acc[q];
+    __syncthreads();
+    cpx<T> *out = Dt + (size_t)col * n0 + xb;
 #pragma unroll
     for (int q = 0; q < Q; ++q)
-        if (P2 || x0 + q < n0) out[q] = acc[q];
+        if (tid + q * nthr < len) out[tid + q * nthr] = W[padq(tid + q * nthr)];
 }
 
 // two consecutive complex values from global memory (16-byte aligned for
@@ -338,21 +412,20 @@ static cudaError_t sub_t(Plan *p, const double *x, void *diff, cudaStream_t s) {
     k_kernel_table<T><<<blocks, 256, 0, s>>>(p->ylen, p->bv, x, ksum, (const cpx<T> *)p->twy, (cpx<T> *)p->kap);
     if ((err = cudaGetLastError())) return err;
     {
-        const int nthr = (p->n0 + sub_q<T>() - 1) / sub_q<T>();
-        const size_t smem = ((size_t)p->nk * p->L0 + 2 * (size_t)(p->n0 + (p->n0 + sub_q<T>() - 1) / sub_q<T>())) *
-                            sizeof(cpx<T>);
+        const int nthr = sub_threads<T>(p->n0), seg = sub_q<T>() * nthr;
+        const size_t smem = sub_smem<T>(p);
         const int nbkg_off = p->n - p->nb;
-        auto kern = p->gen0 ? k_sub_cols<T, false, -1> : k_sub_cols<T, true, -1>;
+        auto kern = k_sub_cols<T, -1>;
         switch (p->cfg.w0) {  // the half-widths of the workloads, unrolled
-            case 4: kern = p->gen0 ? k_sub_cols<T, false, 4> : k_sub_cols<T, true, 4>; break;
-            case 5: kern = p->gen0 ? k_sub_cols<T, false, 5> : k_sub_cols<T, true, 5>; break;
-            case 6: kern = p->gen0 ? k_sub_cols<T, false, 6> : k_sub_cols<T, true, 6>; break;
-            case 7: kern = p->gen0 ? k_sub_cols<T, false, 7> : k_sub_cols<T, true, 7>; break;
-            case 8: kern = p->gen0 ? k_sub_cols<T, false, 8> : k_sub_cols<T, true, 8>; break;
+            case 4: kern = k_sub_cols<T, 4>; break;
+            case 5: kern = k_sub_cols<T, 5>; break;
+            case 6: kern = k_sub_cols<T, 6>; break;
+            case 7: kern = k_sub_cols<T, 7>; break;
+            case 8: kern = k_sub_cols<T, 8>; break;
             default: break;
         }
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        kern<<<p->ncol, nthr, smem, s>>>(p->n0, p->hc, p->ncol, p->offb, p->bv, ftab_of<T>(p), p->cfg.w0, nbkg_off,
+        kern<<<dim3(p->ncol, (p->n0 + seg - 1) / seg), nthr, smem, s>>>(p->n0, p->hc, p->ncol, p->offb, p->bv, ftab_of<T>(p), p->cfg.w0, nbkg_off,
                                         (const cpx<T> *)p->F, (const cpx<T> *)p->kap, (const cpx<T> *)p->yhat, x,
                                         (cpx<T> *)p->U);
         if ((err = cudaGetLastError())) return err;
