@@ -19,50 +19,61 @@
 
 namespace sfft {
 
-// ksum[t] = sum over (a,b) != 0 of a_t,ab  (FP64)
-__global__ void k_kernel_sums(BasisView bv, const double *__restrict__ x, double *__restrict__ ksum) {
-    const int t = blockIdx.x;
-    double s = 0.0;
-    const int L1 = 2 * bv.w1 + 1, L = (2 * bv.w0 + 1) * L1;
-    for (int off = threadIdx.x; off < L; off += blockDim.x) {
-        const int a = off / L1 - bv.w0, b = off % L1 - bv.w1;
-        if (a == 0 && b == 0) continue;
-        const int u = bv.unknown(t, a, b);
-        if (u >= 0) s += x[u];
-    }
-    __shared__ double red[32];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double v = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += red[w];
-        ksum[t] = v;
-    }
-}
-
-// kap[t][a + w0][m]
+// kap[t][a + w0][m] = sum_b k_t(a, b) exp(-2 pi i m b / ylen), one block per
+// (t, a) and 256 frequencies.  The row's coefficients are read and rounded to
+// the compute type once; in the centre row the (0, 0) value also loses the sum
+// of the term's other coefficients (FP64).  Bound by the twiddle reads, b words
+// apart across the lanes: one serves b and -b.  (A sum kernel before, and per
+// output 2 w1 + 1 reads of the FP64 coefficients, of twiddles and as many
+// moduli: 4.7 + 17.9 -> 8.2 us at 4096 x 4096, w = 8, 6 terms.)
 template <typename T>
-__global__ void k_kernel_table(int ylen, BasisView bv, const double *__restrict__ x, const double *__restrict__ ksum,
-                               const cpx<T> *__restrict__ tw1, cpx<T> *__restrict__ kap) {
-    const int w0 = bv.w0, w1 = bv.w1;
-    const int h1c = ylen / 2 + 1, L0 = 2 * w0 + 1;
-    const size_t total = (size_t)bv.nk * L0 * h1c;
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-        const int m = (int)(e % h1c);
-        const int ta = (int)(e / h1c);
-        const int t = ta / L0, a = ta % L0 - w0;
-        T re = (T)0, im = (T)0;
-        for (int b = -w1; b <= w1; ++b) {
-            const int u = bv.unknown(t, a, b);
-            double c = u >= 0 ? x[u] : 0.0;
-            if (a == 0 && b == 0) c -= ksum[t];
-            cpx<T> w = tw1[imod(m * b, ylen)];  // exp(-2 pi i m b / ylen)
-            re += (T)c * w.re;
-            im += (T)c * w.im;
+__global__ void __launch_bounds__(256) k_kernel_table(int ylen, BasisView bv, const double *__restrict__ x,
+                                                      const cpx<T> *__restrict__ tw1, cpx<T> *__restrict__ kap) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T *c = reinterpret_cast<T *>(smem_raw);  // [2 w1 + 1]
+    const int w0 = bv.w0, w1 = bv.w1, L0 = 2 * w0 + 1, L1 = 2 * w1 + 1;
+    const int h1c = ylen / 2 + 1, t = blockIdx.y / L0, a = (int)blockIdx.y % L0 - w0;
+    double ksum = 0.0;  // in thread 0 of a centre row
+    if (a == 0) {
+        double s = 0.0;
+        for (int off = threadIdx.x; off < L0 * L1; off += blockDim.x) {
+            const int oa = off / L1 - w0, ob = off % L1 - w1;
+            if (oa == 0 && ob == 0) continue;
+            const int u = bv.unknown(t, oa, ob);
+            if (u >= 0) s += x[u];
         }
-        kap[e] = mk(re, im);
+        __shared__ double red[32];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+        __syncthreads();
+        if (threadIdx.x == 0)
+            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) ksum += red[w];
     }
+    for (int b = threadIdx.x; b < L1; b += blockDim.x) {
+        if (a == 0 && b == w1) continue;
+        const int u = bv.unknown(t, a, b - w1);
+        c[b] = u >= 0 ? (T)x[u] : (T)0;
+    }
+    if (a == 0 && threadIdx.x == 0) {
+        const int u = bv.unknown(t, 0, 0);
+        c[w1] = (T)((u >= 0 ? x[u] : 0.0) - ksum);
+    }
+    __syncthreads();
+    const int m = blockIdx.x * blockDim.x + threadIdx.x;
+    if (m >= h1c) return;
+    T re = c[w1], im = (T)0;
+    int idx = m;  // m b mod ylen
+    for (int b = 1; b <= w1; ++b) {
+        const cpx<T> w = tw1[idx];  // exp(-2 pi i m b / ylen)
+        const T cp = c[w1 + b], cm = c[w1 - b];
+        re += cp * w.re;
+        im += cp * w.im;
+        re += cm * w.re;
+        im -= cm * w.im;
+        idx += m;
+        if (idx >= ylen) idx -= ylen;
+    }
+    kap[(size_t)blockIdx.y * h1c + m] = mk(re, im);
 }
 
 // D~(x, m) into Dt[m][x]: one block per column m and segment of x.  For each
@@ -403,13 +414,10 @@ static cudaError_t launch_rows_inv(Plan *p, void *diff, cudaStream_t s) {
 template <typename T>
 static cudaError_t sub_t(Plan *p, const double *x, void *diff, cudaStream_t s) {
     cudaError_t err;
-    double *ksum = p->xw + p->n + kSolveTail;  // after the solve's statistics and partial sums
-    p->launches += 4;
-    k_kernel_sums<<<p->nk, 256, 0, s>>>(p->bv, x, ksum);
-    const size_t tot = (size_t)p->nk * p->L0 * p->hc;
-    int blocks = (int)((tot + 255) / 256);
-    if (blocks > 8192) blocks = 8192;
-    k_kernel_table<T><<<blocks, 256, 0, s>>>(p->ylen, p->bv, x, ksum, (const cpx<T> *)p->twy, (cpx<T> *)p->kap);
+    p->launches += 3;
+    const size_t csmem = (size_t)p->L1 * sizeof(T);
+    k_kernel_table<T><<<dim3((p->hc + 255) / 256, p->nk * p->L0), 256, csmem, s>>>(
+        p->ylen, p->bv, x, (const cpx<T> *)p->twy, (cpx<T> *)p->kap);
     if ((err = cudaGetLastError())) return err;
     {
         const int nthr = sub_threads<T>(p->n0), seg = sub_q<T>() * nthr;
