@@ -213,15 +213,14 @@ def stage_bytes(spec, n):
     c = 8                                  # FP32 complex
     b = 4 if spec.dtype == "float32" else 8
     nk = (f.dk + 1) * (f.dk + 2) // 2
-    nimg = nk + 1
     # stage-1 rows of the Omega and Theta products (Lambda is evaluated in
-    # closed form for the polynomial basis, outside the gather)
+    # closed form for the polynomial basis, outside the lag sums)
     nrows = (nk * (nk + 1) // 2) * (4 * f.w0 + 1) + nk * (2 * f.w0 + 1)
     h1c = spec.n1 // 2 + 1
     return {
         "rows": 2 * P * b + (f.dk + 2) * H * c,
-        "cols": (f.dk + 2) * H * c + nimg * H * c,
-        "gather": nimg * H * c + nrows * h1c * c,
+        "cols": 0,  # no column spectra: the lag sums along x come from the row transforms
+        "gather": (f.dk + 2) * H * c + nrows * h1c * c,
         "lags": nrows * h1c * c + n * n * 8,
         "solve": 2 * n * n * 8,
         "subtract": (f.dk + 2) * H * c + 2 * H * c + P * b,
@@ -235,18 +234,17 @@ def stage_flops(spec, n):
     n0, n1 = spec.n0, spec.n1
     h1c = n1 // 2 + 1
     nk = (f.dk + 1) * (f.dk + 2) // 2
-    nimg = nk + 1
-    na = min(64, n0)
-    units = h1c * (n0 // na)
     n_om = nk * (nk + 1) // 2
     n_other = nk  # Theta; Lambda is in closed form for the polynomial basis (not in the gather)
-    # per pair and residue class: products, two 8-point DFTs, twiddles, compensated outer sums
-    per_unit = lambda lags: na * 6 + 2 * 60 * (na // 8) + 7 * 6 * (na // 8) + lags * 18
+    # lag sums along x: windows of 128 (core 128 - 4 w), a transform of every
+    # core and window sequence, the products of every bin
+    windows = h1c * -(-n0 // (128 - 4 * f.w0))
+    per_window = (2 * nk + 1) * 5 * 128 * 7 + (n_om + n_other) * 8 * 128
     nfft_rows = (f.dk + 3) // 2
     return {
         "rows": n0 * nfft_rows * 5 * n1 * math.log2(n1) + 60 * n0 * n1,
-        "cols": h1c * nimg * 5 * n0 * math.log2(n0),
-        "gather": units * (n_om * per_unit(4 * f.w0 + 1) + n_other * per_unit(2 * f.w0 + 1)),
+        "cols": 0.0,
+        "gather": windows * per_window,
         "lags": 0.0,
         "solve": n ** 3 / 3.0,
         "subtract": h1c * n0 * nk * (2 * f.w0 + 1) * 8 + (n0 // 2) * 5 * n1 * math.log2(n1),
@@ -524,7 +522,7 @@ def run_ours(args):
         result["stages_note"] = ("each stage replayed alone on one plan; 'solve' is one system per launch, "
                                  "the serving path solves `batch` per launch")
         result["serving_share"] = {k: round(v / tot, 3) for k, v in per_pair.items()}
-        kern = {"rows": "k_rows", "cols": "k_cols", "gather": "k_gather", "lags": "k_stage2",
+        kern = {"rows": "k_rows", "cols": "k_cols", "gather": "k_lagx", "lags": "k_stage2",
                 "solve": "k_solve_coop", "subtract": "k_sub_cols + k_rows_inv"}[top]
         sf = stage_flops(spec, plan.n)
         clk = clocks["sm_max_mhz"] or 2070.0
@@ -547,7 +545,7 @@ def run_ours(args):
                                   "flops_source": "this implementation's own operation count of the stage",
                                   "peak_source": f"FP32 CUDA-core peak 152 SM x 128 lanes x 2 x {clk:.0f} MHz"}
         result["stages_hbm_frac"] = {k: round(sb[k] / (stage_ms[k] / 1e3) / 1e9 / peak, 3)
-                                     for k in ("rows", "cols", "gather", "subtract") if stage_ms.get(k)}
+                                     for k in ("rows", "gather", "subtract") if stage_ms.get(k)}
         ba = pair_alg_bytes(spec)
         result["pair_roofline"] = {"alg_bytes_per_pair": ba, "achieved_GBs": ba / (ms_step / 1e3) / 1e9,
                                    "frac": ba / (ms_step / 1e3) / 1e9 / peak}
@@ -601,7 +599,7 @@ def run_ours(args):
                          "runs_pairs_per_s": [round(world * ke / r, 1) for r in runs]}
 
     # the solve of `batch` built systems in one launch (sfft_solve_batch), with
-    # 32- and 64-wide Cholesky panels: the serving path's solve step alone
+    # either panel width setting: the serving path's solve step alone
     if not args.no_solve_batch and world == 1:
         from paper_2109_09334_gb300 import SfftPlan as _Plan
         nb = args.batch
@@ -844,7 +842,7 @@ def measure_sectors(args, dev, world, rank):
         x0, y0 = (int(v) for v in rng.integers(0, 4096 - n + 1, size=2))
         f = sp.fit
         plan = SfftPlan(n, n, f.w0, f.w1, f.dk, f.db, f.const_phot_ratio, dtype="float32", precision=args.precision)
-        # systems solved several per launch: 64-wide Cholesky panels
+        # the panel width setting of batches
         plan.solve_panel = 64 if args.sector_solve == "batched" else 32
         Rt = torch.from_numpy(np.ascontiguousarray(R[x0:x0 + n, y0:y0 + n])).to(dev)
         St = torch.from_numpy(np.ascontiguousarray(S[x0:x0 + n, y0:y0 + n])).to(dev)

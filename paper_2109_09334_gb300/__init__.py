@@ -114,7 +114,7 @@ class SfftPlan:
 
     @property
     def solve_panel(self):
-        """Panel width of the FP32 solve's blocked Cholesky (32 or 64)."""
+        """Panel width setting of the FP32 solve (32 or 64): shared by the systems of a launch; the results do not depend on it."""
         return binding.sfft_plan_solve_panel(self.handle)
 
     @solve_panel.setter
