@@ -148,6 +148,16 @@ int sfft_plan_set_solve_panel(sfft_plan_t plan, int32_t width);
 int sfft_plan_solve_panel(sfft_plan_t plan, int32_t *width);
 
 /*
+ * Testing hook: the limit, in clock cycles, of each wait on the grid barrier
+ * inside the solve launches that this plan comes first in.  cycles < 0 sets the
+ * default, about two seconds, back.  A wait that runs out ends the launch:
+ * every block returns, the status of each of its systems is SFFT_ERR_TIMEOUT and
+ * the coefficients are zero.  With 0 the first block that has to wait at all
+ * gives up, so that this path can be exercised with no fault on the GPU.
+ */
+int sfft_plan_debug_solve_wait(sfft_plan_t plan, int64_t cycles);
+
+/*
  * Build the normal equations M theta = rhs of Eq. 18 (blocks Eq. 19-24) from
  * the reference R and science S, through the lag tables of App. B
  * (Eq. B5-B16): forward FFTs of the monomial-weighted images R^ij = xt^i yt^j R

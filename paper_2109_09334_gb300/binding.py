@@ -83,6 +83,7 @@ def library():
         lib.sfft_plan_workspace_bytes.argtypes = [vp, ctypes.POINTER(ctypes.c_uint64)]
         lib.sfft_plan_set_solve_panel.argtypes = [vp, ctypes.c_int32]
         lib.sfft_plan_solve_panel.argtypes = [vp, ctypes.POINTER(ctypes.c_int32)]
+        lib.sfft_plan_debug_solve_wait.argtypes = [vp, ctypes.c_int64]
         lib.sfft_build_system.argtypes = [vp, vp, vp, vp, vp, vp, vp]
         lib.sfft_solve.argtypes = [vp, vp, vp, vp, vp, vp]
         lib.sfft_solve_batch.argtypes = [vp, i32, vp, vp, vp, vp, vp]
@@ -205,6 +206,11 @@ def sfft_plan_solve_panel(plan):
     w = ctypes.c_int32()
     _check(library().sfft_plan_solve_panel(plan, ctypes.byref(w)), "sfft_plan_solve_panel")
     return w.value
+
+
+def sfft_plan_debug_solve_wait(plan, cycles):
+    """Testing hook: limit of each wait on the solve's grid barrier (< 0: the default)."""
+    _check(library().sfft_plan_debug_solve_wait(plan, int(cycles)), "sfft_plan_debug_solve_wait")
 
 
 def sfft_plan_workspace_bytes(plan):

@@ -241,6 +241,7 @@ int plan_new(const sfft_config *cfg, cudaStream_t s, Plan **out) {
     if (!p) return SFFT_ERR_OOM;
     memset((void *)p, 0, sizeof(Plan));
     p->solve_panel = 32;
+    p->solve_wait = kSolveWaitCycles;
     {
         int dev = 0;
         if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -618,6 +619,12 @@ int sfft_plan_set_solve_panel(sfft_plan_t plan, int32_t width) {
 int sfft_plan_solve_panel(sfft_plan_t plan, int32_t *width) {
     if (!plan || !width) return SFFT_ERR_INVALID;
     *width = ((Plan *)plan)->solve_panel;
+    return SFFT_OK;
+}
+
+int sfft_plan_debug_solve_wait(sfft_plan_t plan, int64_t cycles) {
+    if (!plan) return SFFT_ERR_INVALID;
+    ((Plan *)plan)->solve_wait = cycles < 0 ? kSolveWaitCycles : cycles;
     return SFFT_OK;
 }
 

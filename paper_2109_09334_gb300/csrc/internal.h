@@ -22,6 +22,8 @@ constexpr int kLagLen = 128;
 // (2 per block), then the subtraction's kernel sums.
 constexpr int kMaxSolveGrid = 512;
 constexpr int kSolveTail = 8 + 2 * kMaxSolveGrid;
+// Limit of a wait on the solve's grid barrier, in cycles (about two seconds).
+constexpr long long kSolveWaitCycles = 4000000000LL;
 // Systems solved together by one launch of the batched solve.
 constexpr int kMaxSolveBatch = 8;
 
@@ -128,6 +130,7 @@ struct Plan {
     // panel width setting (32, the default, or 64): must agree within a batch;
     // the factorisation takes 64-wide steps for both (solve.cu)
     int solve_panel;
+    long long solve_wait;  // limit of a wait on the solve's grid barrier (kSolveWaitCycles but in tests)
     int sms;  // multiprocessors of the device the plan was created on
     // basis (see BasisView); the tables are built at plan creation
     int bspline;           // 0 polynomial, 1 B-spline

@@ -997,6 +997,7 @@ __device__ __forceinline__ void scale_row(const SolveArgs<T> &s, int i, int lane
 template <typename T>
 struct BatchArgs {
     int nsys;
+    long long wait;  // limit of a wait on the grid barrier, in cycles
     SolveArgs<T> sys[kMaxBatch];
 };
 
@@ -1031,13 +1032,17 @@ __device__ __forceinline__ double block_norm2(const double *v, int n, double *re
 // Barrier of the whole grid after a first grid.sync (which orders the reset of
 // its counter).  Unlike that of the cooperative groups an arrival does not
 // wait for the counter's value, and the thread that makes it can be any.
-// Waits are bounded: one that runs out moves the counter past every later
-// target, so that all blocks run to the end, and the solve reports a timeout.
+// Waits are bounded.  One that runs out replaces a count below its target by
+// kBarDead, in one atomic step: a barrier is complete for every block or for
+// none, and no block passes a later one.  wait and sync then return false, to
+// all threads of the block alike, and the block must not go on (a late block
+// may still be writing what the others would read): it leaves for the end of
+// the kernel.  The limit (kSolveWaitCycles) is far above any step.
 constexpr int kBarDead = 1 << 30;
-constexpr long long kBarWaitCycles = 4000000000LL;  // about two seconds
 struct GridBar {
     int *cnt;
     int target;
+    long long limit;
     __device__ __forceinline__ void arrive(int thread) {  // after the block's work: every thread calls it
         __syncthreads();
         if ((int)threadIdx.x == thread) {
@@ -1045,23 +1050,21 @@ struct GridBar {
         }
         target += gridDim.x;
     }
-    __device__ __forceinline__ void wait() {
+    __device__ __forceinline__ bool wait() {
+        int v = 0;
         if (threadIdx.x == 0) {
             const long long t0 = clock64();
-            int v;
             do {
                 asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(cnt) : "memory");
-                if (v < target && clock64() - t0 > kBarWaitCycles) {
-                    atomicMax(cnt, kBarDead);
-                    break;
-                }
+                // (a count that moved meanwhile is read again: at most one turn per block)
+                if (v < target && clock64() - t0 > limit && atomicCAS(cnt, v, kBarDead) == v) v = kBarDead;
             } while (v < target);
         }
-        __syncthreads();
+        return !__syncthreads_or(v >= kBarDead);
     }
-    __device__ __forceinline__ void sync() {
+    __device__ __forceinline__ bool sync() {
         arrive(0);
-        wait();
+        return wait();
     }
 };
 
@@ -1071,18 +1074,14 @@ __device__ __forceinline__ int multiprocessor() {
     return id;
 }
 
+// Factorisation and refinement of all systems; false if a wait on the grid
+// barrier ran out (in every block alike).
 template <typename T, bool TC>
-__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kBlocksPerSM : 1) k_solve_coop(BatchArgs<T> ba) {
+__device__ __forceinline__ bool solve_systems(const BatchArgs<T> &ba, SolveSmem<T> &sm, TcState &st) {
     using S = Shape<T>;
     constexpr int TS = S::TS;
     cg::grid_group grid = cg::this_grid();
-    extern __shared__ __align__(1024) unsigned char smem_raw[];
-    SolveSmem<T> &sm = *reinterpret_cast<SolveSmem<T> *>(smem_raw);
     __shared__ double red[kThreads / 32];
-    __shared__ __align__(8) uint64_t tc_mbar;
-    __shared__ uint32_t tc_slot;
-    TcState st{};
-    if constexpr (TC) tc_init(st, &tc_mbar, &tc_slot);
     const int tid = threadIdx.x, bid = blockIdx.x, nbk = gridDim.x;
     const int gtid = bid * kThreads + tid, gthreads = nbk * kThreads;
     // warp tasks: consecutive ones on different blocks, so that every
@@ -1122,7 +1121,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kBlocksPerSM : 1) k
     // instructions.  The others draw their numbers.
     if (bid < nsys && tid == 0) reinterpret_cast<int *>(ba.sys[bid].stats + 5)[0] = multiprocessor();
     grid.sync();
-    GridBar bar{&ba.sys[0].flag[3], 0};
+    GridBar bar{&ba.sys[0].flag[3], 0, ba.wait};
     if (bid >= nsys && tid == 0) {
         bool own = true;
         for (int b = 0; b < nsys; ++b)
@@ -1140,7 +1139,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kBlocksPerSM : 1) k
         }
         for (int e = gtid; e < (s.ld - n) * s.ld; e += gthreads) s.X[(size_t)n * s.ld + e] = (T)0;
     }
-    bar.sync();
+    if (!bar.sync()) return false;
     // A = D M D on the lower triangle (nothing reads the upper one), one warp
     // per row pair (k, n - 1 - k)
     for (int task = wtask; task < yofs[nsys]; task += wstep) {
@@ -1149,7 +1148,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kBlocksPerSM : 1) k
         scale_row(s, k, lane);
         if (s.n - 1 - k != k) scale_row(s, s.n - 1 - k, lane);
     }
-    bar.sync();
+    if (!bar.sync()) return false;
 
     // ---- Cholesky and W = L^-1 ----------------------------------------------
     // A system whose status turned negative is skipped from then on, and one
@@ -1163,7 +1162,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kBlocksPerSM : 1) k
     bool bad = false;  // of the chain of system bid (thread 0)
     T minpiv = (T)1e30;
     if (bid < nsys && ba.sys[bid].flag[0] == 0) chain_block(ba.sys[bid], sm.chain, 0, false, bad, minpiv, [] {});
-    bar.sync();
+    if (!bar.sync()) return false;
     for (int kb = 0; kb < nblk_max; ++kb) {
         unsigned live = 0;
         bool more = false;
@@ -1187,7 +1186,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kBlocksPerSM : 1) k
         const bool chain = bid < nsys && (live & (1u << bid)) && kb + 1 < ba.sys[bid].ld / TS;
         if (chain) {
             chain_block(ba.sys[bid], sm.chain, kb + 1, true, bad, minpiv, [&] { bar.arrive(kThreads - 1); });
-            bar.wait();
+            if (!bar.wait()) return false;
         } else {
             if (rank >= 0) {
                 for (int task = rank; task < poff[nsys]; task += nwork) {
@@ -1195,7 +1194,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kBlocksPerSM : 1) k
                     panel_task(ba.sys[b], sm.panel, kb, task - poff[b]);
                 }
             }
-            bar.sync();
+            if (!bar.sync()) return false;
         }
         if (!more) break;  // every system's steps are done (same in every block)
         if (rank >= 0) {
@@ -1263,7 +1262,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kBlocksPerSM : 1) k
                 }
             }
         }
-        bar.sync();
+        if (!bar.sync()) return false;
     }
 
     if (bid < nsys && tid == 0 && (double)minpiv < ba.sys[bid].stats[0]) ba.sys[bid].stats[0] = (double)minpiv;
@@ -1290,7 +1289,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kBlocksPerSM : 1) k
                 s.z[i] = (T)(s.dsc[i] * ri);
             }
         }
-        bar.sync();
+        if (!bar.sync()) return false;
         // ||r||^2 (and first ||rhs||^2) of system b by block b, beside the
         // product y = W z of the others: the next barrier serves both
         if (bid < nsys && !(done & (1u << bid))) {
@@ -1318,7 +1317,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kBlocksPerSM : 1) k
                 if (lane == 0) s.y[i2] = a2;
             }
         }
-        bar.sync();
+        if (!bar.sync()) return false;
         for (int b = 0; b < nsys; ++b) {
             if (done & (1u << b)) continue;
             const SolveArgs<T> &s = ba.sys[b];
@@ -1346,7 +1345,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kBlocksPerSM : 1) k
             const T a = col_dot<T, w_depth<T>()>(s.X, s.y, s.ld, i, k0, k1, sm.red);
             if (warp == 0 && i < n) s.wseg[(size_t)sg * n + i] = a;
         }
-        bar.sync();
+        if (!bar.sync()) return false;
         for (int e = gtid; e < nrows_all; e += gthreads) {
             const int b = sys_of(nrow, nsys, e), i = e - nrow[b];
             if (done & (1u << b)) continue;
@@ -1357,18 +1356,31 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kBlocksPerSM : 1) k
             s.x[i] += s.dsc[i] * (double)a;
         }
         if (bid == 0 && tid < nsys && !(done & (1u << tid))) ba.sys[tid].flag[1] += 1;
-        bar.sync();
+        if (!bar.sync()) return false;
     }
-    // ---- results ------------------------------------------------------------
-    for (int e = gtid; e < nrows_all; e += gthreads) {
-        const int b = sys_of(nrow, nsys, e), i = e - nrow[b];
-        ba.sys[b].xout[i] = ba.sys[b].x[i];
+    return true;
+}
+
+template <typename T, bool TC>
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kBlocksPerSM : 1) k_solve_coop(BatchArgs<T> ba) {
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    SolveSmem<T> &sm = *reinterpret_cast<SolveSmem<T> *>(smem_raw);
+    __shared__ __align__(8) uint64_t tc_mbar;
+    __shared__ uint32_t tc_slot;
+    TcState st{};
+    if constexpr (TC) tc_init(st, &tc_mbar, &tc_slot);
+    const bool ok = solve_systems<T, TC>(ba, sm, st);
+    __syncthreads();  // (block 0: its first thread wrote the statuses)
+    // results (all zero where the barrier ran out)
+    for (int b = 0; b < ba.nsys; ++b) {
+        const SolveArgs<T> &s = ba.sys[b];
+        for (int i = blockIdx.x * kThreads + threadIdx.x; i < s.n; i += gridDim.x * kThreads)
+            s.xout[i] = ok ? s.x[i] : 0.0;
     }
-    if (bid == 0 && tid < nsys) {
-        const SolveArgs<T> &s = ba.sys[tid];
+    if (blockIdx.x == 0 && (int)threadIdx.x < ba.nsys) {
+        const SolveArgs<T> &s = ba.sys[threadIdx.x];
         if (s.info) {
-            int f = s.flag[0];
-            if (*bar.cnt >= kBarDead) f = SFFT_ERR_TIMEOUT;
+            int f = ok ? s.flag[0] : SFFT_ERR_TIMEOUT;
             if (f == 0) f = s.flag[2] != INT_MAX ? SFFT_ERR_SINGULAR : SFFT_ERR_NOT_CONVERGED;
             s.info->status = (f == 1) ? SFFT_OK : f;
             s.info->iters = s.flag[1];
@@ -1431,6 +1443,7 @@ static cudaError_t solve_batch_t(Plan *const *plans, int count, const double *co
                                  double *const *x, sfft_solve_info *const *info, cudaStream_t st) {
     BatchArgs<T> ba;
     ba.nsys = count;
+    ba.wait = plans[0]->solve_wait;
     for (int b = 0; b < count; ++b) {
         Plan *p = plans[b];
         ba.sys[b] = system_args<T>(p->n, M[b], rhs[b], x[b], info[b], p->dscale, p->xw, p->r, p->A, p->zv, p->flag);
@@ -1492,6 +1505,7 @@ static cudaError_t solve_buf_t(const SolveBuffers &b, const double *M, const dou
                                sfft_solve_info *info, cudaStream_t st) {
     BatchArgs<T> ba;
     ba.nsys = 1;
+    ba.wait = kSolveWaitCycles;
     ba.sys[0] = system_args<T>(b.n, M, rhs, x, info, b.dsc, b.xw, b.r, b.A, b.zv, b.flag);
     return launch_batch(ba, b.grid, st);
 }
