@@ -12,6 +12,8 @@
 // real FFT per row then gives D.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "fft.cuh"
 #include "fft16.cuh"
@@ -95,27 +97,44 @@ __global__ void __launch_bounds__(256) k_kernel_table(int ylen, BasisView bv, co
 template <typename T>
 __host__ __device__ constexpr int sub_q() { return sizeof(T) == 4 ? 4 : 8; }
 constexpr int kSubThreads = 256;
+// Launch shape.  Where the kernel values leave no room for both pairs each
+// (n_K L0 above some 12000 values), they are kept once and the pairs made at
+// every tap (223 instead of 176 us at 4093 x 256, w0 = 100, w1 = 0, 6 terms,
+// where both fit).  Where they leave none for the segments of 256 threads
+// either, these are halved: whatever fits beside a whole column fits so.
+struct SubShape {
+    int threads;
+    bool two;  // both pairs kept
+    size_t smem;
+};
 template <typename T>
-static int sub_threads(int n0) {
-    const int q = sub_q<T>(), most = sizeof(T) == 4 ? kSubThreads : 64;
-    return (n0 + q - 1) / q < most ? (n0 + q - 1) / q : most;
-}
-template <typename T>
-static size_t sub_smem(const Plan *p) {
-    const int q = sub_q<T>(), len = q * sub_threads<T>(p->n0) + 2 * p->cfg.w0;
-    return ((size_t)(sizeof(T) == 4 ? 2 : 1) * p->nk * p->L0 + 2 * (size_t)(len + len / q + q + 1)) * sizeof(cpx<T>);
+static SubShape sub_shape(const Plan *p) {
+    constexpr int q = sub_q<T>(), most = sizeof(T) == 4 ? kSubThreads : 64;
+    constexpr size_t room = 227 * 1024 - kMaxFun * sizeof(cpx<T>);  // (bp)
+    SubShape h;
+    h.threads = std::min((p->n0 + q - 1) / q, most);
+    auto size = [&](int copies) {
+        const int len = q * h.threads + 2 * p->cfg.w0;
+        return ((size_t)copies * p->nk * p->L0 + 2 * (size_t)(len + len / q + q + 1)) * sizeof(cpx<T>);
+    };
+    h.two = sizeof(T) == 4 && size(2) <= room;
+    if (!h.two)
+        while (h.threads > 1 && size(1) > room) h.threads = (h.threads + 1) / 2;
+    h.smem = size(h.two ? 2 : 1);
+    return h;
 }
 
 // W0 >= 0: the kernel half-width is the compile-time W0 (the tap loop unrolls
 // completely, so the window shifts are register renames); W0 < 0: w0 at run time.
-template <typename T, int W0>
+// TWO: both pairs of a kernel value in shared memory (FP32).
+template <typename T, int W0, bool TWO>
 __global__ void __launch_bounds__(kSubThreads, sizeof(T) == 4 ? 4 : 1)
     k_sub_cols(int n0, int hc, int ncol, int offb, BasisView bv, FTab<T> ft, int w0, int nbkg_off,
                const cpx<T> *__restrict__ F, const cpx<T> *__restrict__ kap, const cpx<T> *__restrict__ yhat,
                const double *__restrict__ x, cpx<T> *__restrict__ Dt) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr bool PK = sizeof(T) == 4;
-    constexpr int Q = sub_q<T>(), KS = PK ? 2 : 1;
+    constexpr int Q = sub_q<T>(), KS = TWO ? 2 : 1;
     const int nk = bv.nk, nbt = bv.nb;
     if (W0 >= 0) w0 = W0;
     const int L0 = 2 * w0 + 1;
@@ -123,12 +142,12 @@ __global__ void __launch_bounds__(kSubThreads, sizeof(T) == 4 ? 4 : 1)
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int col = blockIdx.x, m = col % hc, xb = blockIdx.y * (Q * nthr);
     const int len = min(Q * nthr, n0 - xb), ext = len + 2 * w0;  // outputs; staged values
-    cpx<T> *kp = reinterpret_cast<cpx<T> *>(smem_raw);  // nk * L0 (in FP32 two pairs each)
+    cpx<T> *kp = reinterpret_cast<cpx<T> *>(smem_raw);  // nk * L0 (TWO: two pairs each)
     cpx<T> *Wb = kp + KS * nk * L0;  // two buffers, alternating by term
     const int wlen = padq(Q * nthr + 2 * w0) + Q + 1;
     for (int e = tid; e < nk * L0; e += nthr) {
         const cpx<T> v = kap[(size_t)e * hc + m];
-        if constexpr (PK) {
+        if constexpr (TWO) {
             kp[2 * e] = mk(-v.re, -v.re);
             kp[2 * e + 1] = mk(v.im, -v.im);
         } else {
@@ -206,8 +225,14 @@ __global__ void __launch_bounds__(kSubThreads, sizeof(T) == 4 ? 4 : 1)
                 }
 #pragma unroll
                 for (int c = 0; c <= 2 * (W0 >= 0 ? W0 : w0); ++c) {  // tap a = w0 - c
-                    const float4 kv = *reinterpret_cast<const float4 *>(kt + 2 * (L0 - 1 - c));
-                    const pair32 kr = pack2(kv.x, kv.y), ki = pack2(kv.z, kv.w);
+                    pair32 kr, ki;
+                    if constexpr (TWO) {
+                        const float4 kv = *reinterpret_cast<const float4 *>(kt + 2 * (L0 - 1 - c));
+                        kr = pack2(kv.x, kv.y), ki = pack2(kv.z, kv.w);
+                    } else {
+                        const cpx<T> kv = kt[L0 - 1 - c];
+                        kr = pack2(-kv.re, -kv.re), ki = pack2(kv.im, -kv.im);
+                    }
 #pragma unroll
                     for (int q = 0; q < Q; ++q) fma2(pa[q], kr, win[q]);
 #pragma unroll
@@ -420,22 +445,25 @@ static cudaError_t sub_t(Plan *p, const double *x, void *diff, cudaStream_t s) {
         p->ylen, p->bv, x, (const cpx<T> *)p->twy, (cpx<T> *)p->kap);
     if ((err = cudaGetLastError())) return err;
     {
-        const int nthr = sub_threads<T>(p->n0), seg = sub_q<T>() * nthr;
-        const size_t smem = sub_smem<T>(p);
+        const SubShape h = sub_shape<T>(p);
+        const int seg = sub_q<T>() * h.threads;
         const int nbkg_off = p->n - p->nb;
-        auto kern = k_sub_cols<T, -1>;
-        switch (p->cfg.w0) {  // the half-widths of the workloads, unrolled
-            case 4: kern = k_sub_cols<T, 4>; break;
-            case 5: kern = k_sub_cols<T, 5>; break;
-            case 6: kern = k_sub_cols<T, 6>; break;
-            case 7: kern = k_sub_cols<T, 7>; break;
-            case 8: kern = k_sub_cols<T, 8>; break;
-            default: break;
+        constexpr bool two = sizeof(T) == 4;
+        auto kern = h.two ? k_sub_cols<T, -1, two> : k_sub_cols<T, -1, false>;
+        if (h.two || !two) {
+            switch (p->cfg.w0) {  // the half-widths of the workloads, unrolled
+                case 4: kern = k_sub_cols<T, 4, two>; break;
+                case 5: kern = k_sub_cols<T, 5, two>; break;
+                case 6: kern = k_sub_cols<T, 6, two>; break;
+                case 7: kern = k_sub_cols<T, 7, two>; break;
+                case 8: kern = k_sub_cols<T, 8, two>; break;
+                default: break;
+            }
         }
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        kern<<<dim3(p->ncol, (p->n0 + seg - 1) / seg), nthr, smem, s>>>(p->n0, p->hc, p->ncol, p->offb, p->bv, ftab_of<T>(p), p->cfg.w0, nbkg_off,
-                                        (const cpx<T> *)p->F, (const cpx<T> *)p->kap, (const cpx<T> *)p->yhat, x,
-                                        (cpx<T> *)p->U);
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h.smem);
+        kern<<<dim3(p->ncol, (p->n0 + seg - 1) / seg), h.threads, h.smem, s>>>(
+            p->n0, p->hc, p->ncol, p->offb, p->bv, ftab_of<T>(p), p->cfg.w0, nbkg_off, (const cpx<T> *)p->F,
+            (const cpx<T> *)p->kap, (const cpx<T> *)p->yhat, x, (cpx<T> *)p->U);
         if ((err = cudaGetLastError())) return err;
     }
     if (p->segy) return rows_inv_segments(p, diff, s);
