@@ -556,9 +556,12 @@ typedef enum {
  * solve's tensor-core tile products stay as set: a single system's time does
  * not predict batched solves, and the tensor-core products round
  * differently).  The shapes change how the work is split into blocks, not
- * the arithmetic, so results are unchanged.  They stay with the plan and are
- * remembered for later plans (and server slots, pool lanes) of the same image
- * size, types and D_K in this process.  Synchronises the stream.
+ * the arithmetic, so results are unchanged.  A shape of a kernel that the plan
+ * does not run (the column FFT where the lag sums along x come from short
+ * windows, the row FFTs where rows are transformed by segments) stays as it
+ * is.  The shapes stay with the plan and are remembered for later plans (and
+ * server slots, pool lanes) of the same image size, types and D_K that run the
+ * same transforms, in this process.  Synchronises the stream.
  */
 int sfft_plan_autotune(sfft_plan_t plan, const void *d_ref, const void *d_sci, void *d_diff,
                        sfft_stream_t stream);

@@ -186,9 +186,10 @@ void plan_free(Plan *p) {
     } while (0)
 
 // Launch shapes found by sfft_plan_autotune, kept for later plans of the same
-// image size, types and kernel degree (server slots, pool lanes).
+// image size, types and kernel degree whose transforms are the same kernels
+// (server slots, pool lanes).
 struct TuneEntry {
-    int n0, n1, dtype, precision, dk, basis, kdeg, kint;
+    int n0, n1, dtype, precision, dk, basis, kdeg, kint, segx, segy;
     int32_t shapes[SFFT_TUNING_LEN];
 };
 
@@ -212,27 +213,28 @@ static TuneEntry g_tune[kTuneCache];
 static int g_ntune = 0;
 static std::mutex g_tune_mu;
 
-static bool tune_key_eq(const TuneEntry &e, const sfft_config *c) {
+static bool tune_key_eq(const TuneEntry &e, const Plan *p) {
+    const sfft_config *c = &p->cfg;
     return e.n0 == c->n0 && e.n1 == c->n1 && e.dtype == c->dtype && e.precision == c->precision && e.dk == c->dk &&
-           e.basis == c->basis && e.kdeg == c->kdeg && e.kint == c->kint;
+           e.basis == c->basis && e.kdeg == c->kdeg && e.kint == c->kint && e.segx == p->segx && e.segy == p->segy;
 }
 
 static void tune_lookup(Plan *p) {
     std::lock_guard<std::mutex> lock(g_tune_mu);
     for (int k = 0; k < g_ntune; ++k)
-        if (tune_key_eq(g_tune[k], &p->cfg)) set_shapes(p, g_tune[k].shapes);
+        if (tune_key_eq(g_tune[k], p)) set_shapes(p, g_tune[k].shapes);
 }
 
 static void tune_store(const Plan *p) {
     std::lock_guard<std::mutex> lock(g_tune_mu);
     int k = 0;
-    while (k < g_ntune && !tune_key_eq(g_tune[k], &p->cfg)) ++k;
+    while (k < g_ntune && !tune_key_eq(g_tune[k], p)) ++k;
     if (k == g_ntune) {
         if (g_ntune == kTuneCache) k = 0;  // full: overwrite the oldest slot
         else ++g_ntune;
     }
     const sfft_config &c = p->cfg;
-    g_tune[k] = TuneEntry{c.n0, c.n1, c.dtype, c.precision, c.dk, c.basis, c.kdeg, c.kint, {}};
+    g_tune[k] = TuneEntry{c.n0, c.n1, c.dtype, c.precision, c.dk, c.basis, c.kdeg, c.kint, p->segx, p->segy, {}};
     get_shapes(p, g_tune[k].shapes);
 }
 
@@ -755,6 +757,7 @@ int sfft_plan_autotune(sfft_plan_t plan, const void *d_ref, const void *d_sci, v
     // sets it by hand).
     for (Knob &kb : knobs) {
         if (kb.stage == SFFT_STAGE_COLS && (p->gen0 || p->segx)) continue;  // no column FFT
+        if (kb.stage != SFFT_STAGE_COLS && p->segy) continue;  // rows by segments: one shape
         int best = 0;
         float best_ms = 1e30f;
         for (int c : kb.cand) {
