@@ -323,7 +323,10 @@ int sfft_run_pair(sfft_plan_t plan, const void *d_ref, const void *d_sci,
  *                    the solve panel width); a plan listed twice, or a
  *                    mismatch, is SFFT_ERR_INVALID.
  *   d_refs, d_scis, d_diffs : count device image pointers, each as in
- *                    sfft_run_pair (d_diffs[i] distinct from the inputs).
+ *                    sfft_run_pair (d_diffs[i] distinct from the inputs of
+ *                    pair i).  Every system is built before the first
+ *                    difference image is written, and these are written in
+ *                    the order of the pairs where they share memory.
  *   d_masks        : NULL, or count pointers, each NULL or a mask.
  *   d_xs, d_infos  : NULL, or count pointers, each NULL (plan-owned buffer)
  *                    or a device buffer as in sfft_run_pair.
