@@ -1444,7 +1444,10 @@ cudaError_t row_transform(Plan *p, const void *ref, const void *sci, const uint8
 // With a side stream the moments, the zero-lag sums and the closed-form Lambda
 // (few blocks or short, and independent of the transforms) run beside the
 // transforms and lag sums: 1024 x 1024 pair 291 -> 269 us, FP64 build of 1000 x
-// 1024 742 -> 663 us, FP64 pair of 256 x 256 410 -> 378 us.
+// 1024 742 -> 663 us, FP64 pair of 256 x 256 410 -> 378 us.  Not beside the direct lag
+// sums (k_xcorr): their few long blocks, placed while others ran, shared some
+// multiprocessors and left others idle (FP64, 17 B-spline terms, 300 x 280: 3175 us
+// in line, 4634 beside, 3142 after them; 300 x 256: 3030, 6657, 3008).
 cudaError_t build_system(Plan *p, const void *ref, const void *sci, const uint8_t *mask, double *M,
                          double *rhs, cudaStream_t s, cudaStream_t side) {
     if (side == nullptr) {
@@ -1461,6 +1464,7 @@ cudaError_t build_system(Plan *p, const void *ref, const void *sci, const uint8_
     if (b == cudaSuccess) b = launch_lambda(p, side);
     const cudaError_t r = cudaEventRecord(p->ev_join, side);
     if (e == cudaSuccess) e = cols_of(p, s);
+    if (e == cudaSuccess && p->gen0 && !p->segx) e = cudaStreamWaitEvent(s, p->ev_join, 0);
     if (e == cudaSuccess) e = gather_of(p, s);
     const cudaError_t f = cudaEventRecord(p->ev_fork, s);  // the row transforms are read
     if (e == cudaSuccess) e = stage2_of(p, s);
