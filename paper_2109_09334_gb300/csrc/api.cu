@@ -287,9 +287,19 @@ int plan_new(const sfft_config *cfg, cudaStream_t s, Plan **out) {
     // Overlap-save transforms: the lag sums along x for the polynomial basis
     // (B-spline plans need the column spectra for Lambda, and keep the row
     // transforms these were computed from), the rows where n1 is not a power
-    // of two.
-    p->segx = p->lam_closed && p->nk <= 6;
-    p->segy = p->segx && p->gen1;
+    // of two.  FP64 keeps the transforms whose operations are fewer on small
+    // sizes: the column FFT and gather where a window of 128 holds a large part
+    // of a column that is itself an FFT length and there are many columns
+    // (64 x 4096, 6 terms, w = 3: 780 us by windows, 560 so; 128 x 4096, w = 8: 1684
+    // and 1295; the other way round above 256 rows: 1024 x 4096 4470 and 5281),
+    // and Bluestein rows of at most 256 points where the segments, of 256 points
+    // whatever n1, have more columns and sequences (64 x 48, 6 terms: build and
+    // subtraction 267 + 185 us by segments, 159 + 158 so; 64 x 17, 3 terms: 163 + 134
+    // and 96 + 117; 64 x 160, 6 terms, the other way round: 334 + 226 and 366 + 357).
+    const bool fft = p->fp64 && !p->gen0 && !p->gen1 && p->n1 > 512 && p->n0 <= (p->nk == 3 ? 512 : 256);
+    p->segx = p->lam_closed && p->nk <= 6 && !fft;
+    const bool blu = p->fp64 && p->m1 <= (p->nk == 6 ? 256 : p->nk == 3 ? 128 : 0);
+    p->segy = p->segx && p->gen1 && !blu;
     p->ylen = p->segy ? kSegLen : p->n1;
     p->hc = p->ylen / 2 + 1;
     p->nsy = 1;

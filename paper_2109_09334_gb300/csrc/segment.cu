@@ -144,19 +144,34 @@ __global__ void __launch_bounds__(LagShape<NK>::kThreads, sizeof(T) == 4 ? (NK =
         stw[q] = tw128[q];
         stp[q] = tw128[(q >> 3) * (q & 7)];
     }
-    // this warp's sequence: s < NK core sequences, then NK + 1 window ones
-    constexpr int kWarpsPerSeq = SEG / 4;
-    const int sq = warp / kWarpsPerSeq;
-    const bool is_core = sq < NK;
-    const int t = is_core ? sq : sq - NK;  // kernel term (t = NK: S)
-    int ti = 0, tj = nfy;
-    if (t < NK) term_ij(t, &ti, &tj);
-    const int fsq = is_core ? tj : offb + tj;  // its row-transform sequence
-    const int g = lane & 7, sub = (warp % kWarpsPerSeq) * 4 + (lane >> 3);
+    // Sequence q < NK: core ones, then NK + 1 window ones; its power of xt and
+    // its row-transform sequence.
+    auto sequence = [&](int q, int &ti, int &fsq) {
+        const int t = q < NK ? q : q - NK;  // kernel term (t = NK: S)
+        int tj = nfy;
+        ti = 0;
+        if (t < NK) term_ij(t, &ti, &tj);
+        fsq = q < NK ? tj : offb + tj;
+    };
+    const int nseg = (n0 + core - 1) / core;
+    // this thread's sequence and segment: eight threads a transform, the
+    // segments of a sequence side by side.  In FP64, whose instructions take a
+    // warp 64 cycles whatever the number of its lanes at work, a column of fewer
+    // segments than a batch has packs its transforms (build
+    // of 64 x 2000, 6 terms, w = 8: 1187 -> 963 us)
+    const int per = sizeof(T) == 8 ? min(SEG, nseg) : SEG;
+    const int sq = (tid >> 3) / per, sub = (tid >> 3) % per, g = lane & 7;
+    const bool has = sq < NSEQ, is_core = sq < NK;
+    int ti = 0, fsq = 0;
+    if (has) sequence(sq, ti, fsq);
     cpx<T> *row = spec + (size_t)(sq * SEG + sub) * kLagRow;
     const bool centre = c % hc == 0;
-    if (centre) {  // means of the sequences (real at m = 0)
+    if (centre) {  // means of the sequences (real at m = 0), a warp each
+        constexpr int kWarpsPerSeq = SEG / 4;
         if (warp % kWarpsPerSeq == 0) {
+            const int q = warp / kWarpsPerSeq;
+            int ti, fsq;
+            sequence(q, ti, fsq);
             const cpx<T> *col = F + (size_t)fsq * seqstride + (size_t)c * n0;
             const T *wx = fx + (size_t)ti * n0;
             double a = 0.0;
@@ -165,16 +180,15 @@ __global__ void __launch_bounds__(LagShape<NK>::kThreads, sizeof(T) == 4 ? (NK =
                 a += (double)(ti > 0 ? v * wx[x] : v);
             }
             for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-            if (lane == 0) mean[sq] = (T)(a / n0);
+            if (lane == 0) mean[q] = (T)(a / n0);
         }
     }
     __syncthreads();
-    const T mu = centre ? mean[sq] : (T)0;
+    const T mu = centre && has ? mean[sq] : (T)0;
     const int k = tid & (kLagL - 1), role = tid / kLagL;  // product sums: bin and role
     cpx<T> acc[Sh::kOwn];
 #pragma unroll
     for (int p = 0; p < Sh::kOwn; ++p) acc[p] = mk((T)0, (T)0);
-    const int nseg = (n0 + core - 1) / core;
     const bool small = n0 < 2 * kLagL;  // windows may wrap more than once
     // asynchronous copies of a batch's windows (and the weights xt^i along
     // them) into shared memory, one window per warp and turn
@@ -214,7 +228,7 @@ __global__ void __launch_bounds__(LagShape<NK>::kThreads, sizeof(T) == 4 ? (NK =
         asm volatile("cp.async.wait_group 0;\n" ::);
         __syncthreads();  // this batch's windows are staged; the sums of the one before are done
         const int seg = s0 + sub;
-        if (seg < nseg) {
+        if (has && seg < nseg) {
             const int x0 = seg * core;
             cpx<T> v[16];
 #pragma unroll
