@@ -141,6 +141,27 @@ __global__ void k_twiddle(int n, cpx<T> *tw) {
     }
 }
 
+// v to the grid of T, a fraction (d + 1/2) / num of the step up before the cut
+template <typename T>
+__device__ T dithered(double v, int d, int num) {
+    if (num == 1 || v == 0.0 || v == 1.0 || v == -1.0) return (T)v;
+    int e;
+    frexp(v, &e);
+    const double step = ldexp(1.0, e - 24);
+    return (T)(floor(v / step + (d + 0.5) / num) * step);
+}
+template <typename T>
+__global__ void k_lag_tables(LagTab<T> *tab) {
+    const int q = threadIdx.x;
+    double sn, cs;
+    sincospi(-2.0 * (double)q / kLagLen, &sn, &cs);
+    for (int d = 0; d < LagTab<T>::kNum; ++d) {
+        tab->fwd[d][q].re = dithered<T>(cs, d, LagTab<T>::kNum);
+        tab->fwd[d][q].im = dithered<T>(sn, d, LagTab<T>::kNum);
+    }
+    tab->inv[q] = make_int2(__double2int_rn(cs * 268435456.0), __double2int_rn(-sn * 268435456.0));
+}
+
 static bool is_pow2(int v) { return v > 0 && (v & (v - 1)) == 0; }
 
 int plan_validate(const sfft_config *c) {
@@ -298,7 +319,16 @@ int plan_new(const sfft_config *cfg, cudaStream_t s, Plan **out) {
     // and 96 + 117; 64 x 160, 6 terms, the other way round: 334 + 226 and 366 + 357).
     const bool fft = p->fp64 && !p->gen0 && !p->gen1 && p->n1 > 512 && p->n0 <= (p->nk == 3 ? 512 : 256);
     p->segx = p->lam_closed && p->nk <= 6 && !fft;
-    const bool blu = p->fp64 && p->m1 <= (p->nk == 6 ? 256 : p->nk == 3 ? 128 : 0);
+    // FP32 fits of more than one term keep Bluestein rows up to 512 pixels for
+    // their accuracy: the core of a segment begins and ends with the sky, whose
+    // spectrum then fills every column (alone in column 0 otherwise), and with few
+    // segments to a row the lag sums are rounded at its size.  Error of the
+    // difference image that comes from the build, 1500 pixels in x, 6 terms, w = 8,
+    // by segments and by Bluestein: 9.2e-6 and 4.1e-6 at 240 pixels, 7.4e-6 and 5.2e-6
+    // at 300, 5.2e-6 and 4.9e-6 at 500; from 600 up it is the other way round (400 x
+    // 600: 4.5e-6 and 6.8e-6), Bluestein's own roundings growing with its length.
+    const int blu_most = !p->fp64 ? (p->nk == 1 ? 0 : 1024) : p->nk == 6 ? 256 : p->nk == 3 ? 128 : 0;
+    const bool blu = p->m1 <= blu_most;
     p->segy = p->segx && p->gen1 && !blu;
     p->ylen = p->segy ? kSegLen : p->n1;
     p->hc = p->ylen / 2 + 1;
@@ -394,7 +424,7 @@ int plan_new(const sfft_config *cfg, cudaStream_t s, Plan **out) {
         const size_t dt = std::max(half, (size_t)p->h1c * p->n0);
         SFFT_ALLOC(p->U, (p->gen0 || p->segx ? dt : (size_t)p->nimg * half) * csz);
     }
-    if (p->segx) SFFT_ALLOC(p->tw128, 128 * csz);
+    if (p->segx) SFFT_ALLOC(p->tw128, p->fp64 ? sizeof(LagTab<double>) : sizeof(LagTab<float>));
     if (p->segy) SFFT_ALLOC(p->twy, (size_t)p->ylen * csz);
     else p->twy = p->tw1;
     SFFT_ALLOC(p->kimg, (size_t)p->L0 * p->L1 * sizeof(double));
@@ -464,7 +494,7 @@ int plan_new(const sfft_config *cfg, cudaStream_t s, Plan **out) {
                                              (cpx<double> *)p->yhat);
         else
             k_poly_dft<double><<<by, 128, 0, s>>>(p->n1, p->h1c, p->nby, t64b, 0, 1, 0, tby, (cpx<double> *)p->yhat);
-        if (p->segx) k_twiddle<double><<<1, 128, 0, s>>>(128, (cpx<double> *)p->tw128);
+        if (p->segx) k_lag_tables<<<1, kLagLen, 0, s>>>((LagTab<double> *)p->tw128);
         if (p->segy) k_twiddle<double><<<1, 256, 0, s>>>(p->ylen, (cpx<double> *)p->twy);
     } else {
         k_round<float><<<(p->n0 + 255) / 256, 256, 0, s>>>(p->n0, t64a, (cpx<float> *)p->tw0);
@@ -479,7 +509,7 @@ int plan_new(const sfft_config *cfg, cudaStream_t s, Plan **out) {
                                              (cpx<float> *)p->yhat);
         else
             k_poly_dft<float><<<by, 128, 0, s>>>(p->n1, p->h1c, p->nby, t64b, 0, 1, 0, tby, (cpx<float> *)p->yhat);
-        if (p->segx) k_twiddle<float><<<1, 128, 0, s>>>(128, (cpx<float> *)p->tw128);
+        if (p->segx) k_lag_tables<<<1, kLagLen, 0, s>>>((LagTab<float> *)p->tw128);
         if (p->segy) k_twiddle<float><<<1, 256, 0, s>>>(p->ylen, (cpx<float> *)p->twy);
     }
     for (int ax = 0; ax < 2; ++ax) {  // Bluestein tables of the axes that are not powers of two

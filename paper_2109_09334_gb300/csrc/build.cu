@@ -1360,9 +1360,8 @@ static cudaError_t launch_gather(Plan *p, cudaStream_t s) {
 
 template <typename T>
 static cudaError_t launch_stage2(Plan *p, cudaStream_t s) {
-    const int xlen = p->segx ? kLagLen : p->n0;  // length of the transforms along x
-    k_stage2<T><<<p->nrows, 256, 0, s>>>(1.0 / ((double)xlen * (double)p->ylen), p->ylen, p->hc, p->ncol, p->cfg.w0, p->cfg.w1, p->bv,
-                                         p->npairs, p->pairs, (const cpx<T> *)p->Q, (const cpx<T> *)p->yhat,
+    k_stage2<T><<<p->nrows, 256, 0, s>>>(1.0 / ((double)lag_norm(p) * (double)p->ylen), p->ylen, p->hc, p->ncol, p->cfg.w0,
+                                         p->cfg.w1, p->bv, p->npairs, p->pairs, (const cpx<T> *)p->Q, (const cpx<T> *)p->yhat,
                                          (const cpx<T> *)p->twy, p->lag, p->lag_om, p->lag_la, p->lag_th);
     p->launches++;
     return cudaGetLastError();

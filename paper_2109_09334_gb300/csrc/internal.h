@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include "../../include/sfft.h"
+#include "common.cuh"
 
 namespace sfft {
 
@@ -26,6 +27,16 @@ constexpr int kSolveTail = 8 + 2 * kMaxSolveGrid;
 constexpr long long kSolveWaitCycles = 4000000000LL;
 // Systems solved together by one launch of the batched solve.
 constexpr int kMaxSolveBatch = 8;
+
+// Tables of the lag sums along x (segment.cu): twiddles exp(-2 pi i q / kLagLen),
+// in FP32 as kNum roundings of each whose mean is the value to a sixteenth of an
+// ulp, and (FP32) exp(2 pi i q / kLagLen) in units of 2^-28.
+template <typename T>
+struct LagTab {
+    static constexpr int kNum = sizeof(T) == 4 ? 8 : 1;
+    cpx<T> fwd[kNum][kLagLen];
+    int2 inv[kLagLen];
+};
 
 enum PairKind { PK_OMEGA = 0, PK_LAMBDA = 1, PK_THETA = 2, PK_OMEGA2 = 3 };
 
@@ -228,6 +239,9 @@ int basis_terms(const sfft_config *c, int *nk, int *nb);
 int basis_build(Plan *p, cudaStream_t s);  // p->n, sizes and cfg set; allocations owned by p
 // weights of the kernel terms at one normalised position (w: nk values)
 void basis_term_weights(const Plan *p, double xt0, double yt0, double *w);
+
+// The stage-1 table holds the lag sums along x times this.
+inline int lag_norm(const Plan *p) { return p->segy ? kLagLen : p->n0; }
 
 // launchers (return cudaError_t of the last launch)
 // side: a second stream for the kernels beside the transforms (the plan's, or

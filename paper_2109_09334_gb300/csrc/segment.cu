@@ -18,6 +18,7 @@
 //     transform table: column c = segment * 129 + m.
 #include <cuda_runtime.h>
 
+#include <type_traits>
 #include <utility>
 
 #include "common.cuh"
@@ -39,20 +40,33 @@ namespace sfft {
 // Then thread (k, role) adds the products of bin k over its segments to
 // register sums.  At the end Z_p(k), k < 128, of product p is inverted in two
 // steps, k = c + 16 r: Y_c(s) = sum_r Z(c + 16 r) e^(2 pi i r s / 8), and
-// Q(rho) = sum_c e^(2 pi i c rho / 128) Y_c(rho mod 8), the outer sum
-// compensated (its 16 terms carry independent roundings; in plain FP32 the
-// inverse alone would double the error of M).  In each bin the sum over
-// segments runs over terms of that bin's own size, so plain sums serve there.
+// Q(rho) = sum_c e^(2 pi i c rho / 128) Y_c(rho mod 8).
+//
+// Accuracy, FP32 (error of the difference image against 64 bits; the column FFT
+// and the direct lag sums that these took the place of are "before"):
+//   * Roundings of the inverse are white over the bins and so hide the weak high
+//     frequencies, where M's small eigenvalues are.  It is taken in integers (30
+//     bits of Z, 64-bit sums) and leaves one rounding, that of the stored Q.
+//   * Rounded twiddles and constants act like one filter in every column and
+//     segment, so their effect does not average out.  Columns take turns in eight
+//     roundings of each (LagTab) whose mean is right; what is left of the error
+//     alternates with the column and lands at lags of an eighth of the row.
+//     Without it the coefficients' error doubles (1024 x 1024, 3 terms, w = 6: 5.6e-6
+//     and 1.1e-5; before 5.6e-6).
+//   * In each bin the sum over segments runs over terms of that bin's own size:
+//     compensated sums changed no error by more than 2 %.
+// 4096 x 4096, w = 8: 8.8e-6 before, 7.9e-6 with an FP32 inverse and rounded twiddles,
+// 6.9e-6 (342 -> 357 us, most of it the integer inverse); 1501 x 1024, w = 5: 2.4e-6
+// before, 3.8e-6, 2.5e-6.
 //
 // The core's halos are zero and the window's hold the wrapped image, so the
 // segments need no special case at the image edge and any n0 serves.  The
 // windows of a batch come by asynchronous copies that run during the product
 // sums of the batch before.  Bound by instruction issue and shared-memory
-// traffic (58 % issue active, 26 warps per multiprocessor), not by HBM (the
+// traffic (@@ARITH@@), not by HBM (the
 // row transforms are read once).  Against the column FFT and gather it
-// replaced (w0 = 8, 6 terms, 4096 x 4096, FP32): 630 -> 350 us; against direct
-// lag sums (2046 columns of x, w0 = 6): 2250 -> 219 us; the image error of the
-// difference against 64 bits falls (fewer roundings per term).
+// replaced (w0 = 8, 6 terms, 4096 x 4096, FP32): 630 -> 357 us; against direct
+// lag sums (2046 columns of x, w0 = 6): 2250 -> 230 us.
 // Window 128: a longer one (256) has fewer halo samples but twice the
 // exchange per transform; the lags need 4 w0 < 128.
 //
@@ -116,6 +130,79 @@ __device__ __forceinline__ void lag_products(cpx<T> (&acc)[OWN], const cpx<T> *s
      ...);
 }
 
+// Forward dft8 and dft16 (fft.cuh, fft16.cuh) with given cos(pi / 4), cos(pi /
+// 8) and sin(pi / 8)
+template <typename T>
+struct LagConst {
+    T c4, c8, s8;
+};
+template <typename T>
+__device__ __forceinline__ void dft8c(cpx<T> (&v)[8], const LagConst<T> &k) {
+    cpx<T> a[4], b[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        a[i] = v[i] + v[i + 4];
+        b[i] = v[i] - v[i + 4];
+    }
+    b[1] = cmul(b[1], mk(k.c4, -k.c4));
+    b[2] = mul_i(b[2], -1);
+    b[3] = cmul(b[3], mk(-k.c4, -k.c4));
+    dft4(a[0], a[1], a[2], a[3], -1);
+    dft4(b[0], b[1], b[2], b[3], -1);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        v[2 * i] = a[i];
+        v[2 * i + 1] = b[i];
+    }
+}
+template <typename T>
+__device__ __forceinline__ void dft16c(cpx<T> (&v)[16], const LagConst<T> &k) {
+#pragma unroll
+    for (int r = 0; r < 4; ++r) dft4(v[r], v[r + 4], v[r + 8], v[r + 12], -1);
+    v[5] = cmul(v[5], mk(k.c8, -k.s8));
+    v[9] = cmul(v[9], mk(k.c4, -k.c4));
+    v[13] = cmul(v[13], mk(k.s8, -k.c8));
+    v[6] = cmul(v[6], mk(k.c4, -k.c4));
+    v[10] = mul_i(v[10], -1);
+    v[14] = cmul(v[14], mk(-k.c4, -k.c4));
+    v[7] = cmul(v[7], mk(k.s8, -k.c8));
+    v[11] = cmul(v[11], mk(-k.c4, -k.c4));
+    v[15] = cmul(v[15], mk(-k.c8, k.s8));
+#pragma unroll
+    for (int r = 0; r < 4; ++r) dft4(v[4 * r], v[4 * r + 1], v[4 * r + 2], v[4 * r + 3], -1);
+}
+
+// 8-point inverse DFT of integers up to 2^30 in magnitude, exact but for the
+// products with cos(pi / 4) (30 bits); outputs up to 2^33.5, in the order 0, 2,
+// 4, 6, 1, 3, 5, 7
+using i64 = long long;
+__device__ __forceinline__ void idft4(i64 (&re)[8], i64 (&im)[8], int o) {
+    const i64 ar = re[o] + re[o + 2], ai = im[o] + im[o + 2], br = re[o] - re[o + 2], bi = im[o] - im[o + 2];
+    const i64 cr = re[o + 1] + re[o + 3], ci = im[o + 1] + im[o + 3];
+    const i64 er = re[o + 1] - re[o + 3], ei = im[o + 1] - im[o + 3];
+    re[o] = ar + cr, im[o] = ai + ci;
+    re[o + 1] = br - ei, im[o + 1] = bi + er;
+    re[o + 2] = ar - cr, im[o + 2] = ai - ci;
+    re[o + 3] = br + ei, im[o + 3] = bi - er;
+}
+__device__ __forceinline__ void idft8(i64 (&re)[8], i64 (&im)[8]) {
+    auto cos4 = [](i64 v) { return (v * 759250125LL + (1LL << 29)) >> 30; };  // 2^30 cos(pi / 4)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const i64 ar = re[k], ai = im[k], br = re[k + 4], bi = im[k + 4];
+        re[k] = ar + br, im[k] = ai + bi;
+        re[k + 4] = ar - br, im[k + 4] = ai - bi;
+    }
+    i64 r = re[5], i = im[5];
+    re[5] = cos4(r - i), im[5] = cos4(i + r);
+    r = re[6], i = im[6];
+    re[6] = -i, im[6] = r;
+    r = re[7], i = im[7];
+    re[7] = cos4(-r - i), im[7] = cos4(r - i);
+    idft4(re, im, 0);
+    idft4(re, im, 4);
+}
+
 template <int BYTES>
 __device__ __forceinline__ void cp_async(void *smem, const void *gmem) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"((unsigned)__cvta_generic_to_shared(smem)),
@@ -125,7 +212,7 @@ __device__ __forceinline__ void cp_async(void *smem, const void *gmem) {
 template <typename T, int NK>
 __global__ void __launch_bounds__(LagShape<NK>::kThreads, sizeof(T) == 4 ? (NK == 3 ? 4 : 2) : 1)
     k_lagx(int n0, int hc, int ncol, int w0, int offb, int nfy, const cpx<T> *__restrict__ F,
-           const T *__restrict__ fx, const cpx<T> *__restrict__ tw128, cpx<T> *__restrict__ Q) {
+           const T *__restrict__ fx, const LagTab<T> *__restrict__ tab, int norm, cpx<T> *__restrict__ Q) {
     using Sh = LagShape<NK>;
     constexpr int NP = Sh::kPairs, NSEQ = Sh::kSeq, SEG = Sh::kSeg;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -133,17 +220,15 @@ __global__ void __launch_bounds__(LagShape<NK>::kThreads, sizeof(T) == 4 ? (NK =
     cpx<T> *raw = spec + (size_t)NSEQ * SEG * kLagRow;       // [row-transform sequences][SEG][kLagWin]
     const int nraw = offb + nfy + 1;
     T *wraw = reinterpret_cast<T *>(raw + (size_t)nraw * SEG * kLagWin);  // [nfy - 1][SEG][kLagWin]: xt^i, i >= 1
-    __shared__ cpx<T> stw[kLagL];                         // exp(-2 pi i q / 128)
     __shared__ cpx<T> stp[kLagL];                         // exp(-2 pi i j g / 128) at 8 j + g (no bank conflicts)
     __shared__ T mean[NSEQ];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int c = blockIdx.x;
     const int h = 2 * w0, core = kLagL - 2 * h;
     const size_t seqstride = (size_t)ncol * n0;
-    for (int q = tid; q < kLagL; q += Sh::kThreads) {
-        stw[q] = tw128[q];
-        stp[q] = tw128[(q >> 3) * (q & 7)];
-    }
+    const int dither = (c % hc) % LagTab<T>::kNum;
+    for (int q = tid; q < kLagL; q += Sh::kThreads) stp[q] = tab->fwd[dither][(q >> 3) * (q & 7)];
+    const LagConst<T> lc{tab->fwd[dither][16].re, tab->fwd[dither][8].re, -tab->fwd[dither][8].im};
     // Sequence q < NK: core ones, then NK + 1 window ones; its power of xt and
     // its row-transform sequence.
     auto sequence = [&](int q, int &ti, int &fsq) {
@@ -256,7 +341,7 @@ __global__ void __launch_bounds__(LagShape<NK>::kThreads, sizeof(T) == 4 ? (NK =
                         if (g + 8 * i >= hi) v[i] = mk((T)0, (T)0);
                 }
             }
-            dft16(v, -1);
+            dft16c(v, lc);
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
                 const cpx<T> y = v[slot16(j)];
@@ -272,7 +357,7 @@ __global__ void __launch_bounds__(LagShape<NK>::kThreads, sizeof(T) == 4 ? (NK =
             __syncwarp(0xffu << (lane & 24));
 #pragma unroll
             for (int b = 0; b < 2; ++b) {
-                dft8(u[b], -1);
+                dft8c(u[b], lc);
 #pragma unroll
                 for (int q = 0; q < 8; ++q) row[16 * q + 8 * b + g] = u[b][q];
             }
@@ -314,28 +399,63 @@ __global__ void __launch_bounds__(LagShape<NK>::kThreads, sizeof(T) == 4 ? (NK =
         }
     }
     // Y_c(s) at row s, and the outer twiddles e^(2 pi i c rho / 128), in rows
-    // that lanes of consecutive rho read without bank conflicts
+    // that lanes of consecutive rho read without bank conflicts.  In FP32 both
+    // are integers: Z in units of 2^-30 of its product's largest value (up to a
+    // power of two), Y of 2^-27, the twiddles of 2^-28.
+    constexpr bool kInt = sizeof(T) == 4;
     constexpr int kYRow = 17, kYLen = 8 * kYRow;
-    cpx<T> *Y = Z + NP * kLagL;   // [NP][8][kYRow]
-    cpx<T> *tq = Y + NP * kYLen;  // [16][2 h + 1]
+    using E = typename std::conditional<kInt, int2, cpx<T>>::type;
+    E *Y = reinterpret_cast<E *>(Z + NP * kLagL);  // [NP][8][kYRow]
+    E *tq = Y + NP * kYLen;                        // [16][2 h + 1]
     const int nl = 2 * h + 1;
+    __shared__ unsigned zmax[NP];  // bits of the largest magnitude (of a NaN where there is one)
+    if constexpr (kInt) {
+        for (int p = warp; p < NP; p += Sh::kThreads / 32) {
+            unsigned m = 0;
+#pragma unroll
+            for (int i = 0; i < kLagL / 32; ++i) {
+                const cpx<T> z = Z[p * kLagL + lane + 32 * i];
+                m = max(m, max(__float_as_uint(fabsf(z.re)), __float_as_uint(fabsf(z.im))));
+            }
+            m = __reduce_max_sync(0xffffffffu, m);
+            if (lane == 0) zmax[p] = max(m, 32u << 23);
+        }
+        __syncthreads();
+    }
     for (int e = tid; e < NP * 16; e += Sh::kThreads) {
         const cpx<T> *z = Z + (e >> 4) * kLagL + (e & 15);
-        cpx<T> v[8];
+        E *y = Y + (e >> 4) * kYLen + (e & 15);
+        if constexpr (kInt) {
+            const float up = __uint_as_float((283u - (zmax[e >> 4] >> 23)) << 23);  // the largest to 2^29 .. 2^30
+            i64 re[8], im[8];
 #pragma unroll
-        for (int r = 0; r < 8; ++r) v[r] = z[16 * r];
-        dft8(v, 1);
-        cpx<T> *y = Y + (e >> 4) * kYLen + (e & 15);
+            for (int r = 0; r < 8; ++r) {
+                const cpx<T> v = z[16 * r];
+                re[r] = __float2int_rn(v.re * up);
+                im[r] = __float2int_rn(v.im * up);
+            }
+            idft8(re, im);
+            auto part = [](i64 v) { return (int)((v + 4) >> 3); };
 #pragma unroll
-        for (int r = 0; r < 8; ++r) y[kYRow * r] = v[r];
+            for (int r = 0; r < 8; ++r)
+                y[kYRow * r] = make_int2(part(re[(r & 1) * 4 + r / 2]), part(im[(r & 1) * 4 + r / 2]));
+        } else {
+            cpx<T> v[8];
+#pragma unroll
+            for (int r = 0; r < 8; ++r) v[r] = z[16 * r];
+            dft8(v, 1);
+#pragma unroll
+            for (int r = 0; r < 8; ++r) y[kYRow * r] = v[r];
+        }
     }
     for (int e = tid; e < 16 * nl; e += Sh::kThreads) {
-        const int cc = e / nl, rho = e - cc * nl - h;
-        tq[e] = conj(stw[(cc * rho) & (kLagL - 1)]);
+        const int cc = e / nl, rho = e - cc * nl - h, q = (cc * rho) & (kLagL - 1);
+        if constexpr (kInt) tq[e] = tab->inv[q];
+        else tq[e] = conj(tab->fwd[0][q]);
     }
     __syncthreads();
-    // 128 times the lag sums, in the row order of the stage-1 table: the
-    // Omega products (a, q) first, then the Theta products
+    // norm times the lag sums, in the row order of the stage-1 table: the Omega
+    // products (a, q) first, then the Theta products
     const int nom = NK * (NK + 1) / 2 * nl, nq = nom + NK * (2 * w0 + 1);
     for (int e = tid; e < nq; e += Sh::kThreads) {
         int p, rho;
@@ -354,12 +474,33 @@ __global__ void __launch_bounds__(LagShape<NK>::kThreads, sizeof(T) == 4 ? (NK =
             // products before (a, NK): sum over a' <= a of (NK + 1 - a'), minus 1
             p = (a + 1) * (NK + 1) - a * (a + 1) / 2 - 1;
         }
-        const cpx<T> *y = Y + p * kYLen + kYRow * (rho & 7), *w = tq + rho + h;
-        CAcc<T> s;
-        s.zero();
+        const E *y = Y + p * kYLen + kYRow * (rho & 7), *w = tq + rho + h;
+        cpx<T> out;
+        if constexpr (kInt) {
+            i64 re = 0, im = 0;
 #pragma unroll 4
-        for (int cc = 0; cc < 16; cc += 2) s.add(cmul(w[cc * nl], y[cc]) + cmul(w[(cc + 1) * nl], y[cc + 1]));
-        Q[(size_t)e * ncol + c] = mk((T)s.re.value(), (T)s.im.value());
+            for (int cc = 0; cc < 16; ++cc) {
+                const int2 a = w[cc * nl], b = y[cc];
+                re += (i64)a.x * b.x - (i64)a.y * b.y;
+                im += (i64)a.x * b.y + (i64)a.y * b.x;
+            }
+            // norm times the sums, from their bits 20 and up (the rest is below Y's
+            // roundings) in one rounding; NaN where Z is not finite
+            const unsigned m = zmax[p];
+            const float unit = (m < 0x7f800000u ? __uint_as_float(((m >> 23) - 29u) << 23) * 0x1p-12f
+                                                : __uint_as_float(0x7fffffffu)) * norm;
+            auto value = [&](i64 v) {
+                return fmaf((float)(int)(v >> 42), unit * 0x1p22f, (float)(int)((v >> 20) & 0x3fffff) * unit);
+            };
+            out = mk(value(re), value(im));
+        } else {
+            CAcc<T> s;
+            s.zero();
+#pragma unroll 4
+            for (int cc = 0; cc < 16; cc += 2) s.add(cmul(w[cc * nl], y[cc]) + cmul(w[(cc + 1) * nl], y[cc + 1]));
+            out = scale(mk((T)s.re.value(), (T)s.im.value()), (T)norm / kLagL);
+        }
+        Q[(size_t)e * ncol + c] = out;
     }
 }
 
@@ -374,7 +515,7 @@ static cudaError_t lagx_nk(Plan *p, cudaStream_t s) {
     auto kern = k_lagx<T, NK>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     kern<<<p->ncol, Sh::kThreads, smem, s>>>(p->n0, p->hc, p->ncol, p->cfg.w0, p->offb, p->nfy,
-                                             (const cpx<T> *)p->F, ftab_of<T>(p).fx, (const cpx<T> *)p->tw128,
+                                             (const cpx<T> *)p->F, ftab_of<T>(p).fx, (const LagTab<T> *)p->tw128, lag_norm(p),
                                              (cpx<T> *)p->Q);
     p->launches++;
     return cudaGetLastError();

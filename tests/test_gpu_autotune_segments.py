@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 
 def test_shapes_of_kernels_not_run_stay():
     from paper_2109_09334_gb300 import SfftPlan, binding as B
-    n0, n1 = 96, 300
+    n0, n1 = 96, 600
     R, S = (torch.from_numpy(random_field(n0, n1, k)).float().cuda() for k in (1, 2))
     seg, blu = SfftPlan(n0, n1, 3, 3, 1, 1, 1), None
     was = B.sfft_plan_tuning(seg.handle)
