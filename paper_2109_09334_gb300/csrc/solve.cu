@@ -1034,13 +1034,17 @@ __device__ __forceinline__ double block_norm2(const double *v, int n, double *re
 // wait for the counter's value, and the thread that makes it can be any.
 // Waits are bounded.  One that runs out replaces a count below its target by
 // kBarDead, in one atomic step: a barrier is complete for every block or for
-// none, and no block passes a later one.  wait and sync then return false, to
-// all threads of the block alike, and the block must not go on (a late block
-// may still be writing what the others would read): it leaves for the end of
-// the kernel.  The limit (kSolveWaitCycles) is far above any step.
+// none, and no later one completes.  A late block may then still be writing what
+// the others read, so alive() is false from then on, to all threads of a block
+// alike, and the block leaves the kernel before every step whose loops and
+// branches follow values in memory; what runs in between works on meaningless
+// values, within its bounds.  (These checks: 471 -> 478 us for one system of 1732
+// unknowns; at every barrier, 482.)  The limit (kSolveWaitCycles) is far above any
+// step.
 constexpr int kBarDead = 1 << 30;
 struct GridBar {
     int *cnt;
+    volatile int *dead;  // in shared memory
     int target;
     long long limit;
     __device__ __forceinline__ void arrive(int thread) {  // after the block's work: every thread calls it
@@ -1050,22 +1054,24 @@ struct GridBar {
         }
         target += gridDim.x;
     }
-    __device__ __forceinline__ bool wait() {
-        int v = 0;
+    __device__ __forceinline__ void wait() {
         if (threadIdx.x == 0) {
             const long long t0 = clock64();
+            int v;
             do {
                 asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(cnt) : "memory");
                 // (a count that moved meanwhile is read again: at most one turn per block)
                 if (v < target && clock64() - t0 > limit && atomicCAS(cnt, v, kBarDead) == v) v = kBarDead;
             } while (v < target);
+            if (v >= kBarDead) *dead = 1;
         }
-        return !__syncthreads_or(v >= kBarDead);
+        __syncthreads();
     }
-    __device__ __forceinline__ bool sync() {
+    __device__ __forceinline__ void sync() {
         arrive(0);
-        return wait();
+        wait();
     }
+    __device__ __forceinline__ bool alive() { return *dead == 0; }  // after a wait, before the next arrive
 };
 
 __device__ __forceinline__ int multiprocessor() {
@@ -1074,14 +1080,40 @@ __device__ __forceinline__ int multiprocessor() {
     return id;
 }
 
-// Factorisation and refinement of all systems; false if a wait on the grid
-// barrier ran out (in every block alike).
+// The end of a launch whose barrier ran out: zero coefficients, the status, tensor
+// memory released.  Every thread of the block calls it and does not return.
 template <typename T, bool TC>
-__device__ __forceinline__ bool solve_systems(const BatchArgs<T> &ba, SolveSmem<T> &sm, TcState &st) {
+__device__ __noinline__ void leave(const BatchArgs<T> *ba, TcState st) {
+    for (int b = 0; b < ba->nsys; ++b) {
+        const SolveArgs<T> &s = ba->sys[b];
+        for (int i = blockIdx.x * kThreads + threadIdx.x; i < s.n; i += gridDim.x * kThreads) s.xout[i] = 0.0;
+    }
+    if (blockIdx.x == 0 && (int)threadIdx.x < ba->nsys) {
+        const SolveArgs<T> &s = ba->sys[threadIdx.x];
+        if (s.info) {
+            s.info->status = SFFT_ERR_TIMEOUT;
+            s.info->iters = s.flag[1];
+            s.info->rel_residual = (s.stats[1] > 0.0) ? sqrt(s.stats[2] / s.stats[1]) : sqrt(s.stats[2]);
+            s.info->min_pivot = s.stats[0];
+        }
+    }
+    if constexpr (TC) tc_release(st);
+    asm volatile("exit;");
+}
+
+template <typename T, bool TC>
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kBlocksPerSM : 1)
+    k_solve_coop(const __grid_constant__ BatchArgs<T> ba) {
     using S = Shape<T>;
     constexpr int TS = S::TS;
     cg::grid_group grid = cg::this_grid();
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    SolveSmem<T> &sm = *reinterpret_cast<SolveSmem<T> *>(smem_raw);
     __shared__ double red[kThreads / 32];
+    __shared__ __align__(8) uint64_t tc_mbar;
+    __shared__ uint32_t tc_slot;
+    TcState st{};
+    if constexpr (TC) tc_init(st, &tc_mbar, &tc_slot);
     const int tid = threadIdx.x, bid = blockIdx.x, nbk = gridDim.x;
     const int gtid = bid * kThreads + tid, gthreads = nbk * kThreads;
     // warp tasks: consecutive ones on different blocks, so that every
@@ -1121,7 +1153,9 @@ __device__ __forceinline__ bool solve_systems(const BatchArgs<T> &ba, SolveSmem<
     // instructions.  The others draw their numbers.
     if (bid < nsys && tid == 0) reinterpret_cast<int *>(ba.sys[bid].stats + 5)[0] = multiprocessor();
     grid.sync();
-    GridBar bar{&ba.sys[0].flag[3], 0, ba.wait};
+    __shared__ int dead_s;
+    if (tid == 0) dead_s = 0;
+    GridBar bar{&ba.sys[0].flag[3], &dead_s, 0, ba.wait};
     if (bid >= nsys && tid == 0) {
         bool own = true;
         for (int b = 0; b < nsys; ++b)
@@ -1139,7 +1173,7 @@ __device__ __forceinline__ bool solve_systems(const BatchArgs<T> &ba, SolveSmem<
         }
         for (int e = gtid; e < (s.ld - n) * s.ld; e += gthreads) s.X[(size_t)n * s.ld + e] = (T)0;
     }
-    if (!bar.sync()) return false;
+    bar.sync();
     // A = D M D on the lower triangle (nothing reads the upper one), one warp
     // per row pair (k, n - 1 - k)
     for (int task = wtask; task < yofs[nsys]; task += wstep) {
@@ -1148,7 +1182,7 @@ __device__ __forceinline__ bool solve_systems(const BatchArgs<T> &ba, SolveSmem<
         scale_row(s, k, lane);
         if (s.n - 1 - k != k) scale_row(s, s.n - 1 - k, lane);
     }
-    if (!bar.sync()) return false;
+    bar.sync();
 
     // ---- Cholesky and W = L^-1 ----------------------------------------------
     // A system whose status turned negative is skipped from then on, and one
@@ -1161,8 +1195,10 @@ __device__ __forceinline__ bool solve_systems(const BatchArgs<T> &ba, SolveSmem<
     const int rank = bid < nsys ? -1 : (nown > 0 ? rank_s : bid - nsys);
     bool bad = false;  // of the chain of system bid (thread 0)
     T minpiv = (T)1e30;
-    if (bid < nsys && ba.sys[bid].flag[0] == 0) chain_block(ba.sys[bid], sm.chain, 0, false, bad, minpiv, [] {});
-    if (!bar.sync()) return false;
+    const bool first = bid < nsys && ba.sys[bid].flag[0] == 0;
+    if (!bar.alive()) leave<T, TC>(&ba, st);
+    if (first) chain_block(ba.sys[bid], sm.chain, 0, false, bad, minpiv, [] {});
+    bar.sync();
     for (int kb = 0; kb < nblk_max; ++kb) {
         unsigned live = 0;
         bool more = false;
@@ -1183,10 +1219,11 @@ __device__ __forceinline__ bool solve_systems(const BatchArgs<T> &ba, SolveSmem<
             poff[b + 1] = poff[b] + np;
             uoff[b + 1] = uoff[b] + nu;
         }
+        if (!bar.alive()) leave<T, TC>(&ba, st);
         const bool chain = bid < nsys && (live & (1u << bid)) && kb + 1 < ba.sys[bid].ld / TS;
         if (chain) {
             chain_block(ba.sys[bid], sm.chain, kb + 1, true, bad, minpiv, [&] { bar.arrive(kThreads - 1); });
-            if (!bar.wait()) return false;
+            bar.wait();
         } else {
             if (rank >= 0) {
                 for (int task = rank; task < poff[nsys]; task += nwork) {
@@ -1194,7 +1231,7 @@ __device__ __forceinline__ bool solve_systems(const BatchArgs<T> &ba, SolveSmem<
                     panel_task(ba.sys[b], sm.panel, kb, task - poff[b]);
                 }
             }
-            if (!bar.sync()) return false;
+            bar.sync();
         }
         if (!more) break;  // every system's steps are done (same in every block)
         if (rank >= 0) {
@@ -1262,7 +1299,7 @@ __device__ __forceinline__ bool solve_systems(const BatchArgs<T> &ba, SolveSmem<
                 }
             }
         }
-        if (!bar.sync()) return false;
+        bar.sync();
     }
 
     if (bid < nsys && tid == 0 && (double)minpiv < ba.sys[bid].stats[0]) ba.sys[bid].stats[0] = (double)minpiv;
@@ -1275,6 +1312,7 @@ __device__ __forceinline__ bool solve_systems(const BatchArgs<T> &ba, SolveSmem<
     unsigned done = 0;
     for (int b = 0; b < nsys; ++b)
         if (ba.sys[b].flag[0] != 0 || ba.sys[b].flag[2] != INT_MAX) done |= 1u << b;
+    if (!bar.alive()) leave<T, TC>(&ba, st);
     const unsigned all = (1u << nsys) - 1u;
     for (int it = 0; it <= kMaxIters && done != all; ++it) {
         // r = rhs - M x (FP64); z = D r
@@ -1289,7 +1327,7 @@ __device__ __forceinline__ bool solve_systems(const BatchArgs<T> &ba, SolveSmem<
                 s.z[i] = (T)(s.dsc[i] * ri);
             }
         }
-        if (!bar.sync()) return false;
+        bar.sync();
         // ||r||^2 (and first ||rhs||^2) of system b by block b, beside the
         // product y = W z of the others: the next barrier serves both
         if (bid < nsys && !(done & (1u << bid))) {
@@ -1317,7 +1355,7 @@ __device__ __forceinline__ bool solve_systems(const BatchArgs<T> &ba, SolveSmem<
                 if (lane == 0) s.y[i2] = a2;
             }
         }
-        if (!bar.sync()) return false;
+        bar.sync();
         for (int b = 0; b < nsys; ++b) {
             if (done & (1u << b)) continue;
             const SolveArgs<T> &s = ba.sys[b];
@@ -1330,6 +1368,7 @@ __device__ __forceinline__ bool solve_systems(const BatchArgs<T> &ba, SolveSmem<
                 done |= 1u << b;
             }
         }
+        if (!bar.alive()) leave<T, TC>(&ba, st);
         if (done == all) break;
         // w = W^T y in kSeg row segments (coalesced rows of W), summed in a fixed order
         for (int task = bid; task < wofs[nsys]; task += nbk) {
@@ -1345,7 +1384,7 @@ __device__ __forceinline__ bool solve_systems(const BatchArgs<T> &ba, SolveSmem<
             const T a = col_dot<T, w_depth<T>()>(s.X, s.y, s.ld, i, k0, k1, sm.red);
             if (warp == 0 && i < n) s.wseg[(size_t)sg * n + i] = a;
         }
-        if (!bar.sync()) return false;
+        bar.sync();
         for (int e = gtid; e < nrows_all; e += gthreads) {
             const int b = sys_of(nrow, nsys, e), i = e - nrow[b];
             if (done & (1u << b)) continue;
@@ -1356,31 +1395,18 @@ __device__ __forceinline__ bool solve_systems(const BatchArgs<T> &ba, SolveSmem<
             s.x[i] += s.dsc[i] * (double)a;
         }
         if (bid == 0 && tid < nsys && !(done & (1u << tid))) ba.sys[tid].flag[1] += 1;
-        if (!bar.sync()) return false;
+        bar.sync();
     }
-    return true;
-}
-
-template <typename T, bool TC>
-__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kBlocksPerSM : 1) k_solve_coop(BatchArgs<T> ba) {
-    extern __shared__ __align__(1024) unsigned char smem_raw[];
-    SolveSmem<T> &sm = *reinterpret_cast<SolveSmem<T> *>(smem_raw);
-    __shared__ __align__(8) uint64_t tc_mbar;
-    __shared__ uint32_t tc_slot;
-    TcState st{};
-    if constexpr (TC) tc_init(st, &tc_mbar, &tc_slot);
-    const bool ok = solve_systems<T, TC>(ba, sm, st);
+    // ---- results ------------------------------------------------------------
+    for (int e = gtid; e < nrows_all; e += gthreads) {
+        const int b = sys_of(nrow, nsys, e), i = e - nrow[b];
+        ba.sys[b].xout[i] = ba.sys[b].x[i];
+    }
     __syncthreads();  // (block 0: its first thread wrote the statuses)
-    // results (all zero where the barrier ran out)
-    for (int b = 0; b < ba.nsys; ++b) {
-        const SolveArgs<T> &s = ba.sys[b];
-        for (int i = blockIdx.x * kThreads + threadIdx.x; i < s.n; i += gridDim.x * kThreads)
-            s.xout[i] = ok ? s.x[i] : 0.0;
-    }
-    if (blockIdx.x == 0 && (int)threadIdx.x < ba.nsys) {
-        const SolveArgs<T> &s = ba.sys[threadIdx.x];
+    if (bid == 0 && tid < nsys) {
+        const SolveArgs<T> &s = ba.sys[tid];
         if (s.info) {
-            int f = ok ? s.flag[0] : SFFT_ERR_TIMEOUT;
+            int f = s.flag[0];
             if (f == 0) f = s.flag[2] != INT_MAX ? SFFT_ERR_SINGULAR : SFFT_ERR_NOT_CONVERGED;
             s.info->status = (f == 1) ? SFFT_OK : f;
             s.info->iters = s.flag[1];
