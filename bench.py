@@ -97,7 +97,7 @@ def workload_config(spec, precision):
                         f"w={f.w0}, D_K={f.dk}, D_B={f.db}, const_phot_ratio={f.const_phot_ratio}",
             "image": [spec.n0, spec.n1], "w": f.w0, "dk": f.dk, "db": f.db,
             "const_phot_ratio": f.const_phot_ratio, "precision": precision,
-            "l2": "not flushed: each step touches ~1.3 GB (inputs 134 MB + workspace), > 129 MB L2; "
+            "l2": "not flushed: each step touches ~0.6 GB (inputs 134 MB + workspace), > 129 MB L2; "
                   "two input pairs alternate"}
 
 

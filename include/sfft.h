@@ -542,8 +542,10 @@ int sfft_pool_usage(sfft_pool_t pool, uint64_t *bytes, int32_t *lanes);
 /* Stages of one pair, as re-enqueued by sfft_replay_stage. */
 typedef enum {
     SFFT_STAGE_ROWS = 0,     /* masked row FFTs of yt^j R and S, per-row moments */
-    SFFT_STAGE_COLS = 1,     /* moment sums and column FFTs of xt^i (row transforms) */
-    SFFT_STAGE_GATHER = 2,   /* spectrum products and pruned inverse DFT along x */
+    SFFT_STAGE_COLS = 1,     /* moment sums; column FFTs of xt^i (row transforms), where the
+                                plan takes the lag sums along x from them */
+    SFFT_STAGE_GATHER = 2,   /* lag sums along x: spectrum products and pruned inverse DFT,
+                                or from short windows of the row transforms, or directly */
     SFFT_STAGE_LAGS = 3,     /* frequency sums along y to the lag tables; assembly of M, rhs */
     SFFT_STAGE_SOLVE = 4,    /* Cholesky and refinement */
     SFFT_STAGE_SUBTRACT = 5  /* the difference image (after a masked build, preceded by

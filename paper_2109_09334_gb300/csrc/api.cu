@@ -452,7 +452,7 @@ int plan_new(const sfft_config *cfg, cudaStream_t s, Plan **out) {
     }
     SFFT_ALLOC(p->dscale, n * sizeof(double));
     SFFT_ALLOC(p->r, n * sizeof(double));
-    SFFT_ALLOC(p->xw, (n + kSolveTail + 64) * sizeof(double));  // x, stats, per-block partials, kernel sums
+    SFFT_ALLOC(p->xw, (n + kSolveTail) * sizeof(double));
     SFFT_ALLOC(p->zv, solve_vec_elems((int)n) * rsz);
     SFFT_ALLOC(p->flag, 4 * sizeof(int));
     SFFT_ALLOC(p->M_own, n * n * sizeof(double));
@@ -995,7 +995,8 @@ cudaError_t enqueue_pairs(const sfft_plan_t *plans, int32_t count, const void *c
     // kLanes of the plans' own streams: the small kernels of a pair leave most
     // multiprocessors idle, and the builds of one group of systems run during
     // the solve of the group before.  Every lane is joined to s again whatever
-    // fails.  Sixteen sectors of 512 to 2048 pixels: 4.76 -> 3.31 ms on four lanes.
+    // fails.  Sixteen sectors of 512 to 2048 pixels: 4.76 -> 3.31 ms on four lanes
+    // (3.56 on two, 3.26 on eight, which twice the streams are not worth).
     // Pairs that share a buffer one of them writes (the difference image of one
     // over the reference of another, say) keep the order of one stream: every
     // build, every solve, then the subtractions as listed.

@@ -1,23 +1,29 @@
 // build.cu -- construction of the normal equations (Eq. 18-24 via App. B).
 //
-// Pipeline (all on the plan's stream):
-//   k_rows     row pass: zero-fill with the mask, weight by yt^j, real FFT of
-//              every row along y for j = 0..dk and of S; writes the row
-//              transforms transposed ([image][m][x], x contiguous) and the
-//              per-row moment sums used for the lag-zero entries.
-//   k_moments  FP64 moments sum_x xt^u * (row moment) (Eq. B11, B15 and the
-//              lag-zero values of Omega, Lambda, Theta).
-//   k_cols     column pass: weight by xt^i, FFT along x, and store every
-//              spectrum permuted so that the bins l = lb + NB*r (r < NA) of one
-//              residue class lb are contiguous.
-//   k_gather   for each column m and residue class lb: spectrum products
-//              conj(U_a) U_b with the DC bin removed, an NA-point inverse DFT
-//              over r, and the outer sum over lb with twiddles exp(2 pi i lb
-//              rho/N0), accumulated with two-sum compensation (pruned inverse
-//              DFT along x, only |rho| <= 2w (Omega) or w (Lambda, Theta)).
+// Transforms and lag sums, on the caller's stream:
+//   rows       zero-fill with the mask, weight by yt^j, real DFT of every row
+//              along y for j = 0..dk and of S, written transposed ([image][m][x],
+//              x contiguous): k_rows (FFT), k_rows_blu (Bluestein, other lengths
+//              than powers of two) or k_rows_seg (segment.cu, by segments).
+//   lag sums along x, |rho| <= 2w (Omega) or w (Lambda, Theta), in one of three
+//   forms (api.cu, plan_new, chooses):
+//     k_lagx     (segment.cu) from windows of 128 of the row transforms:
+//                polynomial fits of up to six terms, half-widths up to 16.
+//     k_cols,    column pass (weight by xt^i, FFT along x, spectra permuted so
+//     k_gather   that the bins l = lb + NB*r, r < NA, of one residue class lb are
+//                contiguous), then per column m and class lb the spectrum products
+//                conj(U_a) U_b with the DC bin removed, an NA-point inverse DFT
+//                over r, and the outer sum over lb with twiddles exp(2 pi i lb
+//                rho/N0), compensated: n0 a power of two.
+//     k_xcorr    direct sums at the needed lags: other n0.
 //   k_stage2   the remaining sum over m with exp(2 pi i m rho/N1) (and the
 //              1-D spectrum of y^q for Lambda), compensated, to FP64 lag tables.
-//   k_assemble the index maps of Eq. B5, B7, B9, B11, B13, B15 into M and rhs.
+// Beside them, on the plan's own stream (build_system):
+//   k_row_moments, k_boundary   FP64 moment sums of each row and of the boundary
+//              columns; k_row_moments_tab for B-splines.
+//   k_zero_lag the lag-zero values of Omega, Lambda and Theta, and Eq. B15.
+//   k_lambda_closed   Lambda in closed form (polynomial basis, w <= 16).
+// Then k_assemble: the index maps of Eq. B5, B7, B9, B11, B13, B15 into M and rhs.
 #include <cuda_runtime.h>
 
 #include "common.cuh"

@@ -18,11 +18,10 @@ constexpr int kSegLen = 256;
 // Window length of the lag sums along x (segment.cu).
 constexpr int kLagLen = 128;
 
-// Cooperative solve grid: at most kMaxSolveGrid blocks.  The plan's vector
-// xw holds x (n), then the solve's statistics (8) and per-block partial sums
-// (2 per block), then the subtraction's kernel sums.
+// Cooperative solve grid: at most kMaxSolveGrid blocks.  The vector xw holds x
+// (n), then kSolveTail values: the solve's statistics.
 constexpr int kMaxSolveGrid = 512;
-constexpr int kSolveTail = 8 + 2 * kMaxSolveGrid;
+constexpr int kSolveTail = 8;
 // Limit of a wait on the solve's grid barrier, in cycles (about two seconds).
 constexpr long long kSolveWaitCycles = 4000000000LL;
 // Systems solved together by one launch of the batched solve.
@@ -262,7 +261,7 @@ size_t solve_vec_elems(int n);
 size_t solve_matrix_elems(int n, bool fp64);
 // Solve workspace given by the caller instead of a plan (sizes for n
 // unknowns in the compute type: A solve_matrix_elems(n); zv solve_vec_elems(n); dsc, r n
-// doubles; xw n + 8 + 2*grid doubles; flag 4 ints).
+// doubles; xw n + kSolveTail doubles; flag 4 ints).
 struct SolveBuffers {
     int n, grid;
     bool fp64;

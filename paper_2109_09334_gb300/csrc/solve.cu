@@ -1484,8 +1484,10 @@ static cudaError_t solve_batch_t(Plan *const *plans, int count, const double *co
         grid = sg;  // set by hand
     } else if (count == 1 && !tc && sizeof(T) == 4 && full >= 2 * kMaxSolveBatch) {
         // one system alone: one block per SM (the step's latency, not the
-        // tile throughput, sets its time: 582 us on 304 blocks, 515 on 152 at
-        // n = 1735); several: every resident block
+        // tile throughput, sets its time; us on 152 and on 304 blocks: 70 and 75 at
+        // n = 84, 156 and 163 at 508, 471 and 515 at 1732, 1137 and 1154 at 2884; only
+        // systems far above those of the fits in use are the other way round, 4851
+        // and 4143 at 5284); several: every resident block
         grid = full / kBlocksPerSM;
     }
     const cudaError_t err = launch_batch(ba, grid, st, tc);
@@ -1514,7 +1516,7 @@ int solve_grid_size(bool fp64, bool tc) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const size_t dsm = solve_dyn_smem(fp64);
     // all of the unified L1/shared storage as shared memory, so that two FP32
-    // blocks (64 KB of shared memory each) fit on an SM
+    // blocks (76.8 KB of shared memory each) fit on an SM
     const void *kern = solve_kernel(fp64, tc);
     cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsm);

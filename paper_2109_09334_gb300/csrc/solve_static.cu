@@ -20,7 +20,7 @@
 namespace {
 
 constexpr size_t kMaxN = SFFT_SOLVE_STATIC_MAX_N;
-constexpr int kMaxGrid = sfft::kMaxSolveGrid;  // per-block partial sums: 2 doubles per block
+constexpr int kMaxGrid = sfft::kMaxSolveGrid;
 constexpr int kMaxDevices = 64;  // devices with their own setup record
 constexpr size_t kAlign = 256;
 constexpr size_t kScratchBytes = 2 * kMaxN * kMaxN * sizeof(double) + 256 * 1024;
@@ -103,7 +103,7 @@ int sfft_solve_static(const double *d_M, const double *d_rhs, int32_t n, int32_t
     b.zv = take(sfft::solve_vec_elems(n) * rsz);
     b.dsc = reinterpret_cast<double *>(take(nn * sizeof(double)));
     b.r = reinterpret_cast<double *>(take(nn * sizeof(double)));
-    b.xw = reinterpret_cast<double *>(take((nn + 8 + 2 * kMaxGrid) * sizeof(double)));
+    b.xw = reinterpret_cast<double *>(take((nn + sfft::kSolveTail) * sizeof(double)));
     b.flag = reinterpret_cast<int *>(take(4 * sizeof(int)));
     if (off > kScratchBytes) return SFFT_ERR_UNSUPPORTED;  // not reached for n <= SFFT_SOLVE_STATIC_MAX_N
     e = sfft::solve_on_buffers(b, d_M, d_rhs, d_x, d_info, (cudaStream_t)stream);
