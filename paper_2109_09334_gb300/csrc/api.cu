@@ -181,10 +181,11 @@ int plan_validate(const sfft_config *c) {
 
 void plan_free(Plan *p) {
     void *bufs[] = {p->tw0, p->tw1, p->twp0, p->twp1, p->chirp1, p->bfilt1, p->twpm1, p->chirp0, p->bfilt0,
-                    p->twpm0, p->kimg, p->xhat, p->yhat, p->F, p->U, p->Q, p->pairs, p->rowmom, p->lag, p->A,
+                    p->twpm0, p->kimg, p->xhat, p->build.yhat, p->F, p->U, p->Q, p->pairs, p->rowmom, p->lag, p->A,
                     p->dscale, p->r, p->xw, p->zv, p->flag, p->M_own, p->rhs_own, p->x_own, p->info_own,
                     p->img_ref, p->img_sci, p->img_diff, p->img_mask, p->kap, p->d_int, p->ftab, p->ftab64, p->tw128,
-                    p->segy ? p->twy : nullptr,
+                    p->build.seg ? p->build.twy : nullptr, p->own.seg && !p->build.seg ? p->own.twy : nullptr,
+                    p->own.seg && !p->build.seg ? p->own.yhat : nullptr,
                     p->bxy64, p->d_zdesc, p->d_rdesc, p->z0, p->cmat, p->unk, p->gam, p->bnd};
     for (void *b : bufs)
         if (b) cudaFree(b);
@@ -237,7 +238,7 @@ static std::mutex g_tune_mu;
 static bool tune_key_eq(const TuneEntry &e, const Plan *p) {
     const sfft_config *c = &p->cfg;
     return e.n0 == c->n0 && e.n1 == c->n1 && e.dtype == c->dtype && e.precision == c->precision && e.dk == c->dk &&
-           e.basis == c->basis && e.kdeg == c->kdeg && e.kint == c->kint && e.segx == p->segx && e.segy == p->segy;
+           e.basis == c->basis && e.kdeg == c->kdeg && e.kint == c->kint && e.segx == p->segx && e.segy == p->build.seg;
 }
 
 static void tune_lookup(Plan *p) {
@@ -255,8 +256,20 @@ static void tune_store(const Plan *p) {
         else ++g_ntune;
     }
     const sfft_config &c = p->cfg;
-    g_tune[k] = TuneEntry{c.n0, c.n1, c.dtype, c.precision, c.dk, c.basis, c.kdeg, c.kint, p->segx, p->segy, {}};
+    g_tune[k] = TuneEntry{c.n0, c.n1, c.dtype, c.precision, c.dk, c.basis, c.kdeg, c.kint, p->segx, p->build.seg, {}};
     get_shapes(p, g_tune[k].shapes);
+}
+
+// spectra of the background functions of y (tab, FP64) and twiddles of one form
+template <typename T>
+static void form_tables(Plan *p, const RowForm &f, const cpx<double> *tw64, const double *tab, cudaStream_t s) {
+    const int blocks = (p->nby * f.ncol + 127) / 128;
+    if (!f.seg) {
+        k_poly_dft<T><<<blocks, 128, 0, s>>>(p->n1, p->h1c, p->nby, tw64, 0, 1, 0, tab, (cpx<T> *)f.yhat);
+        return;
+    }
+    k_seg_dft<T><<<blocks, 128, 0, s>>>(p->n1, f.hop, f.halo, f.hc, f.ncol, p->nby, tab, (cpx<T> *)f.yhat);
+    k_twiddle<T><<<1, 256, 0, s>>>(f.ylen, (cpx<T> *)f.twy);
 }
 
 int plan_new(const sfft_config *cfg, cudaStream_t s, Plan **out) {
@@ -327,21 +340,34 @@ int plan_new(const sfft_config *cfg, cudaStream_t s, Plan **out) {
     // by segments and by Bluestein: 9.2e-6 and 4.1e-6 at 240 pixels, 7.4e-6 and 5.2e-6
     // at 300, 5.2e-6 and 4.9e-6 at 500; from 600 up it is the other way round (400 x
     // 600: 4.5e-6 and 6.8e-6), Bluestein's own roundings growing with its length.
-    const int blu_most = !p->fp64 ? (p->nk == 1 ? 0 : 1024) : p->nk == 6 ? 256 : p->nk == 3 ? 128 : 0;
+    const int blu_most = !p->fp64 ? (p->nk == 1 ? 0 : 1024) : p->nk == 6 ? 256 : p->nk == 3 ? 128 : 64;
     const bool blu = p->m1 <= blu_most;
-    p->segy = p->segx && p->gen1 && !blu;
-    p->ylen = p->segy ? kSegLen : p->n1;
-    p->hc = p->ylen / 2 + 1;
-    p->nsy = 1;
-    if (p->segy) {
-        p->halo = 2 * cfg->w1;
-        const int most = kSegLen - 2 * p->halo;
-        p->nsy = (p->n1 + most - 1) / most;
-        p->hop = (p->n1 + p->nsy - 1) / p->nsy;
-        p->nsy = (p->n1 + p->hop - 1) / p->hop;  // no empty segment
-        p->offb = p->nfy;
-    }
-    p->ncol = p->nsy * p->hc;
+    // A subtraction that transforms the rows itself takes segments where they are
+    // faster (FP32 2000 x 300, 6 terms, w = 8: 50 us by segments, 76 by Bluestein; FP64
+    // 64 x 65, 6 terms: 172 and 184; 64 x 48: 185 and 158): no sums over them are at
+    // stake, and its own error is no larger so (1500 x 450: 7.7e-7 and 9.9e-7).
+    const bool blu_own = p->fp64 && p->m1 <= (p->nk == 1 ? 64 : 128);
+    auto rows_form = [&](bool seg) {
+        RowForm f{};
+        f.seg = seg;
+        f.ylen = seg ? kSegLen : p->n1;
+        f.hc = f.ylen / 2 + 1;
+        f.nsy = 1;
+        if (seg) {
+            f.halo = 2 * cfg->w1;
+            const int most = kSegLen - 2 * f.halo;
+            f.nsy = (p->n1 + most - 1) / most;
+            f.hop = (p->n1 + f.nsy - 1) / f.nsy;
+            f.nsy = (p->n1 + f.hop - 1) / f.hop;  // no empty segment
+            f.offb = p->nfy;
+        }
+        f.ncol = f.nsy * f.hc;
+        return f;
+    };
+    p->build = rows_form(p->segx && p->gen1 && !blu);
+    p->own = rows_form(p->segx && p->gen1 && !blu_own);
+    RowForm *const forms[2] = {&p->build, &p->own};
+    const int nforms = p->own.seg == p->build.seg ? 1 : 2;  // forms with tables of their own
     // gather pairs
     const int maxp = p->nk * (p->nk + 1) / 2 + p->nk * p->nbx + p->nk;
     p->host_pairs = (PairDesc *)malloc((size_t)2 * maxp * sizeof(PairDesc));
@@ -398,7 +424,7 @@ int plan_new(const sfft_config *cfg, cudaStream_t s, Plan **out) {
     }
 
     const size_t P = (size_t)p->n0 * p->n1;
-    const size_t half = (size_t)p->ncol * p->n0;
+    const size_t half = (size_t)p->build.ncol * p->n0;
     const size_t csz = p->csz;
     const size_t rsz = p->fp64 ? sizeof(double) : sizeof(float);
     const int npo = p->nk * (p->nk + 1) / 2;
@@ -416,17 +442,25 @@ int plan_new(const sfft_config *cfg, cudaStream_t s, Plan **out) {
     SFFT_ALLOC(p->twp0, p->n0 * csz);
     SFFT_ALLOC(p->twp1, p->n1 * csz);
     if (!p->lam_closed) SFFT_ALLOC(p->xhat, (size_t)p->nbx * p->n0 * csz);
-    SFFT_ALLOC(p->yhat, (size_t)p->nby * p->ncol * csz);
-    SFFT_ALLOC(p->F, (size_t)(p->offb + p->nfy + 1) * half * csz);
+    size_t fcols = 0, dcols = p->h1c, kcols = 0;  // columns of F, of D~, of the kernel spectra
+    for (RowForm *f : forms) {
+        fcols = std::max(fcols, (size_t)(f->offb + p->nfy + 1) * f->ncol);
+        dcols = std::max(dcols, (size_t)f->ncol);
+        kcols = std::max(kcols, (size_t)f->hc);
+    }
+    for (int k = 0; k < nforms; ++k) SFFT_ALLOC(forms[k]->yhat, (size_t)p->nby * forms[k]->ncol * csz);
+    SFFT_ALLOC(p->F, fcols * p->n0 * csz);
     // the column spectra (power-of-two n0, unless segx); the subtraction
     // and the noise decorrelation reuse U for D~
     {
-        const size_t dt = std::max(half, (size_t)p->h1c * p->n0);
+        const size_t dt = dcols * p->n0;
         SFFT_ALLOC(p->U, (p->gen0 || p->segx ? dt : (size_t)p->nimg * half) * csz);
     }
     if (p->segx) SFFT_ALLOC(p->tw128, p->fp64 ? sizeof(LagTab<double>) : sizeof(LagTab<float>));
-    if (p->segy) SFFT_ALLOC(p->twy, (size_t)p->ylen * csz);
-    else p->twy = p->tw1;
+    for (int k = 0; k < nforms; ++k) {
+        if (forms[k]->seg) SFFT_ALLOC(forms[k]->twy, (size_t)kSegLen * csz);
+        else forms[k]->twy = p->tw1;
+    }
     SFFT_ALLOC(p->kimg, (size_t)p->L0 * p->L1 * sizeof(double));
     if (p->gen0) {
         SFFT_ALLOC(p->chirp0, (size_t)p->n0 * csz);
@@ -438,7 +472,7 @@ int plan_new(const sfft_config *cfg, cudaStream_t s, Plan **out) {
         SFFT_ALLOC(p->bfilt1, (size_t)p->m1 * csz);
         SFFT_ALLOC(p->twpm1, (size_t)p->m1 * csz);
     }
-    SFFT_ALLOC(p->Q, (size_t)p->nrows * p->ncol * csz);
+    SFFT_ALLOC(p->Q, (size_t)p->nrows * p->build.ncol * csz);
     SFFT_ALLOC(p->pairs, (size_t)(np + p->ngpairs) * sizeof(PairDesc));
     p->gpairs = p->pairs + np;
     SFFT_ALLOC(p->rowmom, (size_t)p->n0 * p->nmom * sizeof(double));
@@ -459,7 +493,7 @@ int plan_new(const sfft_config *cfg, cudaStream_t s, Plan **out) {
     SFFT_ALLOC(p->rhs_own, n * sizeof(double));
     SFFT_ALLOC(p->x_own, n * sizeof(double));
     SFFT_ALLOC(p->info_own, sizeof(sfft_solve_info));
-    SFFT_ALLOC(p->kap, std::max((size_t)p->nk * p->L0 * p->hc, (size_t)p->L0 * p->h1c) * csz);
+    SFFT_ALLOC(p->kap, std::max((size_t)p->nk * p->L0 * kcols, (size_t)p->L0 * p->h1c) * csz);
 
     // constant tables
     cudaError_t err;
@@ -478,7 +512,7 @@ int plan_new(const sfft_config *cfg, cudaStream_t s, Plan **out) {
     }
     k_twiddle64<<<(p->n0 + 255) / 256, 256, 0, s>>>(p->n0, t64a);
     k_twiddle64<<<(p->n1 + 255) / 256, 256, 0, s>>>(p->n1, t64b);
-    const int bx = (p->nbx * p->n0 + 127) / 128, by = (p->nby * p->ncol + 127) / 128;
+    const int bx = (p->nbx * p->n0 + 127) / 128;
     // the tabulated background functions (FP64)
     const double *tbx = p->bxy64, *tby = p->bxy64 + (size_t)p->nbx * p->n0;
     if (p->fp64) {
@@ -489,13 +523,8 @@ int plan_new(const sfft_config *cfg, cudaStream_t s, Plan **out) {
         if (p->xhat)
             k_poly_dft<double><<<bx, 128, 0, s>>>(p->n0, p->n0, p->nbx, t64a, p->na, p->nbk, 1, tbx,
                                                   (cpx<double> *)p->xhat);
-        if (p->segy)
-            k_seg_dft<double><<<by, 128, 0, s>>>(p->n1, p->hop, p->halo, p->hc, p->ncol, p->nby, tby,
-                                             (cpx<double> *)p->yhat);
-        else
-            k_poly_dft<double><<<by, 128, 0, s>>>(p->n1, p->h1c, p->nby, t64b, 0, 1, 0, tby, (cpx<double> *)p->yhat);
+        for (int k = 0; k < nforms; ++k) form_tables<double>(p, *forms[k], t64b, tby, s);
         if (p->segx) k_lag_tables<<<1, kLagLen, 0, s>>>((LagTab<double> *)p->tw128);
-        if (p->segy) k_twiddle<double><<<1, 256, 0, s>>>(p->ylen, (cpx<double> *)p->twy);
     } else {
         k_round<float><<<(p->n0 + 255) / 256, 256, 0, s>>>(p->n0, t64a, (cpx<float> *)p->tw0);
         k_round<float><<<(p->n1 + 255) / 256, 256, 0, s>>>(p->n1, t64b, (cpx<float> *)p->tw1);
@@ -504,13 +533,8 @@ int plan_new(const sfft_config *cfg, cudaStream_t s, Plan **out) {
         if (p->xhat)
             k_poly_dft<float><<<bx, 128, 0, s>>>(p->n0, p->n0, p->nbx, t64a, p->na, p->nbk, 1, tbx,
                                                  (cpx<float> *)p->xhat);
-        if (p->segy)
-            k_seg_dft<float><<<by, 128, 0, s>>>(p->n1, p->hop, p->halo, p->hc, p->ncol, p->nby, tby,
-                                             (cpx<float> *)p->yhat);
-        else
-            k_poly_dft<float><<<by, 128, 0, s>>>(p->n1, p->h1c, p->nby, t64b, 0, 1, 0, tby, (cpx<float> *)p->yhat);
+        for (int k = 0; k < nforms; ++k) form_tables<float>(p, *forms[k], t64b, tby, s);
         if (p->segx) k_lag_tables<<<1, kLagLen, 0, s>>>((LagTab<float> *)p->tw128);
-        if (p->segy) k_twiddle<float><<<1, 256, 0, s>>>(p->ylen, (cpx<float> *)p->twy);
     }
     for (int ax = 0; ax < 2; ++ax) {  // Bluestein tables of the axes that are not powers of two
         const bool gen = ax == 0 ? p->gen0 : p->gen1;
@@ -551,6 +575,7 @@ int plan_new(const sfft_config *cfg, cudaStream_t s, Plan **out) {
         plan_free(p);
         return SFFT_ERR_CUDA;
     }
+    if (nforms == 1) p->own = p->build;
     tune_lookup(p);
     *out = p;
     return SFFT_OK;
@@ -597,7 +622,7 @@ static int run_pair(Plan *p, const void *ref, const void *sci, const uint8_t *ma
     } else if (e == cudaSuccess) {
         e = solve_system(p, M, rhs, x, info, s);
     }
-    if (e == cudaSuccess) e = subtract_from_rows(p, x, diff, s);
+    if (e == cudaSuccess) e = subtract_from_rows(p, mask ? p->own : p->build, x, diff, s);
     p->last_stream = s;
     return status_of(e);
 }
@@ -697,7 +722,8 @@ int sfft_replay_stage(sfft_plan_t plan, int stage, sfft_stream_t stream) {
         case SFFT_STAGE_SOLVE: e = solve_system(p, p->last_M, p->last_rhs, p->last_x, p->last_info, s); break;
         case SFFT_STAGE_SUBTRACT:  // as in sfft_run_pair: unmasked row FFTs only after a masked build
             e = p->last_mask ? row_transform(p, p->last_ref, p->last_sci, nullptr, false, s) : cudaSuccess;
-            if (e == cudaSuccess) e = subtract_from_rows(p, p->last_x, p->last_diff, s);
+            if (e == cudaSuccess)
+                e = subtract_from_rows(p, p->last_mask ? p->own : p->build, p->last_x, p->last_diff, s);
             break;
         default: return SFFT_ERR_INVALID;
     }
@@ -751,7 +777,7 @@ int sfft_subtract(sfft_plan_t plan, const void *d_ref, const void *d_sci, const 
     cudaStream_t s = (cudaStream_t)stream;
     p->last_stream = s;
     cudaError_t e = row_transform(p, d_ref, d_sci, nullptr, false, s);
-    if (e == cudaSuccess) e = subtract_from_rows(p, d_x, d_diff, s);
+    if (e == cudaSuccess) e = subtract_from_rows(p, p->own, d_x, d_diff, s);
     return status_of(e);
 }
 
@@ -797,7 +823,7 @@ int sfft_plan_autotune(sfft_plan_t plan, const void *d_ref, const void *d_sci, v
     // sets it by hand).
     for (Knob &kb : knobs) {
         if (kb.stage == SFFT_STAGE_COLS && (p->gen0 || p->segx)) continue;  // no column FFT
-        if (kb.stage != SFFT_STAGE_COLS && p->segy) continue;  // rows by segments: one shape
+        if (kb.stage != SFFT_STAGE_COLS && p->build.seg) continue;  // rows by segments: one shape
         int best = 0;
         float best_ms = 1e30f;
         for (int c : kb.cand) {
@@ -1010,7 +1036,8 @@ cudaError_t enqueue_pairs(const sfft_plan_t *plans, int32_t count, const void *c
     auto lane = [&](int q) { return apart ? ((Plan *)plans[q % lanes])->side : s; };
     auto subtract = [&](Plan *p, cudaStream_t st) {
         if (e == cudaSuccess && p->last_mask) first(row_transform(p, p->last_ref, p->last_sci, nullptr, false, st));
-        if (e == cudaSuccess) first(subtract_from_rows(p, p->last_x, p->last_diff, st));
+        if (e == cudaSuccess)
+            first(subtract_from_rows(p, p->last_mask ? p->own : p->build, p->last_x, p->last_diff, st));
     };
     Plan *head = (Plan *)plans[0];
     first(cudaEventRecord(head->ev_fork, s));

@@ -1226,7 +1226,8 @@ static cudaError_t launch_rows(Plan *p, const void *ref, const void *sci, const 
                                cudaStream_t s) {
     const int nfft = (p->nfy + 2) / 2;
     const FTab<T> ft = ftab_of<T>(p);
-    if (p->segy) {
+    const bool seg = core ? p->build.seg : p->own.seg;
+    if (seg) {
         const cudaError_t e = rows_segments(p, ref, sci, mask, core, s);
         if (e != cudaSuccess) return e;
     } else if (p->gen1) {
@@ -1261,7 +1262,7 @@ static cudaError_t launch_rows(Plan *p, const void *ref, const void *sci, const 
                                                               (const cpx<T> *)p->twp1, p->bspline ? ft.fy : nullptr,
                                                               kRowsPrefetch * p->sms);
     }
-    if (!p->segy) p->launches++;
+    if (!seg) p->launches++;
     return cudaGetLastError();
 }
 
@@ -1366,9 +1367,11 @@ static cudaError_t launch_gather(Plan *p, cudaStream_t s) {
 
 template <typename T>
 static cudaError_t launch_stage2(Plan *p, cudaStream_t s) {
-    k_stage2<T><<<p->nrows, 256, 0, s>>>(1.0 / ((double)lag_norm(p) * (double)p->ylen), p->ylen, p->hc, p->ncol, p->cfg.w0,
-                                         p->cfg.w1, p->bv, p->npairs, p->pairs, (const cpx<T> *)p->Q, (const cpx<T> *)p->yhat,
-                                         (const cpx<T> *)p->twy, p->lag, p->lag_om, p->lag_la, p->lag_th);
+    const RowForm &f = p->build;
+    k_stage2<T><<<p->nrows, 256, 0, s>>>(1.0 / ((double)lag_norm(p) * (double)f.ylen), f.ylen, f.hc, f.ncol, p->cfg.w0,
+                                         p->cfg.w1, p->bv, p->npairs, p->pairs, (const cpx<T> *)p->Q,
+                                         (const cpx<T> *)f.yhat, (const cpx<T> *)f.twy, p->lag, p->lag_om, p->lag_la,
+                                         p->lag_th);
     p->launches++;
     return cudaGetLastError();
 }
@@ -1421,7 +1424,7 @@ cudaError_t build_stage(Plan *p, int stage, double *M, double *rhs, cudaStream_t
     }
 }
 
-// the row transforms (core: with the core sequences that the lag sums need)
+// the row transforms (core: those of a build, with the core sequences that the lag sums need)
 static cudaError_t rows_of(Plan *p, const void *ref, const void *sci, const uint8_t *mask, bool core,
                            cudaStream_t s) {
     const bool img64 = p->cfg.dtype == SFFT_F64;

@@ -99,6 +99,17 @@ constexpr int kMaxFun = 8;
 // Largest number of science (and of reference) images in the co-added form of the decorrelation.
 constexpr int kMaxCoadd = 16;
 
+// Row transforms along y.  seg: by nsy segments of kSegLen (segment.cu; core length
+// hop, halo 2 w1), else of the whole row.  The table F has ncol columns: column c is
+// frequency c mod hc of a transform of length ylen (of segment c / hc).
+struct RowForm {
+    int seg, nsy, hop, halo;
+    int ylen, hc, ncol;
+    int offb;    // first window sequence in F (seg: after the nfy core sequences)
+    void *twy;   // twiddles of length ylen (the plan's tw1 unless seg)
+    void *yhat;  // [q][c] 1-D spectra of the background y-functions (compute type)
+};
+
 struct Plan {
     sfft_config cfg;
     int n0, n1, h1c;       // h1c = n1/2 + 1 half-spectrum columns
@@ -119,17 +130,13 @@ struct Plan {
     // Bluestein DFTs of length n1 through FFTs of length m1; gen0: the lag
     // sums along x are direct circular correlations (k_xcorr), no column FFT.
     int gen0, gen1, m0, m1;
-    // Overlap-save transforms (segment.cu).  segx: the lag sums along x by
-    // k_lagx (polynomial basis, n_K <= 6 terms, w0 <= 16); else the column
-    // FFT and gather, or k_xcorr.  segy: the rows by segments of kSegLen
-    // (gen1 only; nsy segments of core length hop, halo 2 w1).  The row
-    // transform table F has ncol columns: column c is frequency c mod hc of a
-    // transform of length ylen (of segment c / hc).
-    int segx, segy, nsy, hop, halo;
-    int ylen, hc, ncol;
-    int offb;              // first window sequence in F (segy: after the nfy core sequences)
-    void *twy;             // twiddles of length ylen (= tw1 unless segy)
-    void *tw128;           // twiddles of length 128 (segx)
+    // segx: the lag sums along x by k_lagx (segment.cu; polynomial basis, n_K <= 6
+    // terms, w0 <= 16); else the column FFT and gather, or k_xcorr.
+    int segx;
+    void *tw128;           // its tables (LagTab)
+    // the row transforms of a build, which the subtraction after an unmasked one
+    // reads too, and those that a subtraction makes of its own
+    RowForm build, own;
     void *chirp1, *bfilt1, *twpm1;  // Bluestein tables for n1 (compute type)
     void *chirp0, *bfilt0, *twpm0;  // Bluestein tables for n0 (noise decorrelation only)
     double *kimg;                   // L0 x L1 kernel image (noise decorrelation)
@@ -165,7 +172,6 @@ struct Plan {
     double *bnd;
     void *xhat;            // [p][lb][r] 1-D spectra of the background x-functions, permuted (compute
                            // type); only where Lambda goes through the gather (not lam_closed)
-    void *yhat;            // [q][m] 1-D spectra of the background y-functions, m < h1c (compute type)
     void *F;               // [(nfy+1)][m][x] row transforms (compute type)
     void *U;               // [nimg][m][lb][r] full spectra, permuted (compute type); reused for Dt
     void *Q;               // [nrows][m] stage-1 results (compute type complex)
@@ -240,13 +246,14 @@ int basis_build(Plan *p, cudaStream_t s);  // p->n, sizes and cfg set; allocatio
 void basis_term_weights(const Plan *p, double xt0, double yt0, double *w);
 
 // The stage-1 table holds the lag sums along x times this.
-inline int lag_norm(const Plan *p) { return p->segy ? kLagLen : p->n0; }
+inline int lag_norm(const Plan *p) { return p->build.seg ? kLagLen : p->n0; }
 
 // launchers (return cudaError_t of the last launch)
 // side: a second stream for the kernels beside the transforms (the plan's, or
 // null: all on s); p->ev_fork is then recorded where F may be overwritten
 cudaError_t build_system(Plan *p, const void *ref, const void *sci, const uint8_t *mask, double *M,
                          double *rhs, cudaStream_t s, cudaStream_t side = nullptr);
+// (for a build, with the moments, or for a subtraction)
 cudaError_t row_transform(Plan *p, const void *ref, const void *sci, const uint8_t *mask,
                           bool moments, cudaStream_t s);
 cudaError_t build_stage(Plan *p, int stage, double *M, double *rhs, cudaStream_t s);
@@ -285,8 +292,9 @@ cudaError_t decorrelate(Plan *p, const double *x, double xt0, double yt0, double
 cudaError_t lag_sums_x(Plan *p, cudaStream_t s);
 cudaError_t rows_segments(Plan *p, const void *ref, const void *sci, const uint8_t *mask, bool core,
                           cudaStream_t s);
-cudaError_t rows_inv_segments(Plan *p, void *diff, cudaStream_t s);
-cudaError_t subtract_from_rows(Plan *p, const double *x, void *diff, cudaStream_t s);
+cudaError_t rows_inv_segments(Plan *p, const RowForm &f, void *diff, cudaStream_t s);
+// f: of the row transforms in F (p->build or p->own)
+cudaError_t subtract_from_rows(Plan *p, const RowForm &f, const double *x, void *diff, cudaStream_t s);
 cudaError_t plan_tables(Plan *p, cudaStream_t s);
 
 }  // namespace sfft

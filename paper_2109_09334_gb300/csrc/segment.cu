@@ -507,14 +507,15 @@ __global__ void __launch_bounds__(LagShape<NK>::kThreads, sizeof(T) == 4 ? (NK =
 template <typename T, int NK>
 static cudaError_t lagx_nk(Plan *p, cudaStream_t s) {
     using Sh = LagShape<NK>;
-    const size_t smem = (size_t)Sh::kSeg * ((Sh::kSeq * kLagRow + (p->offb + p->nfy + 1) * kLagWin) * sizeof(cpx<T>) +
+    const RowForm &f = p->build;
+    const size_t smem = (size_t)Sh::kSeg * ((Sh::kSeq * kLagRow + (f.offb + p->nfy + 1) * kLagWin) * sizeof(cpx<T>) +
                                             (p->nfy - 1) * kLagWin * sizeof(T));
     // the epilogue's tables lie over the transforms and windows
     const size_t epi = (size_t)(Sh::kPairs * (kLagL + 136) + 16 * (4 * p->cfg.w0 + 1)) * sizeof(cpx<T>);
     if (epi > smem) return cudaErrorInvalidConfiguration;
     auto kern = k_lagx<T, NK>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    kern<<<p->ncol, Sh::kThreads, smem, s>>>(p->n0, p->hc, p->ncol, p->cfg.w0, p->offb, p->nfy,
+    kern<<<f.ncol, Sh::kThreads, smem, s>>>(p->n0, f.hc, f.ncol, p->cfg.w0, f.offb, p->nfy,
                                              (const cpx<T> *)p->F, ftab_of<T>(p).fx, (const LagTab<T> *)p->tw128, lag_norm(p),
                                              (cpx<T> *)p->Q);
     p->launches++;
@@ -700,10 +701,11 @@ __global__ void __launch_bounds__(128) k_rows_inv_seg(int n0, int n1, int hop, i
 template <typename T, typename I>
 static cudaError_t rows_seg_t(Plan *p, const void *ref, const void *sci, const uint8_t *mask, bool core,
                               cudaStream_t s) {
-    const dim3 grid((p->n0 + kSegRows - 1) / kSegRows, p->nsy);
-    k_rows_seg<T, I><<<grid, 128, 0, s>>>(p->n0, p->n1, p->hop, p->halo, p->nfy, core ? 1 : 0, (const I *)ref,
-                                          (const I *)sci, mask, ftab_of<T>(p).fy, (const cpx<T> *)p->twy,
-                                          (cpx<T> *)p->F, (size_t)p->ncol * p->n0);
+    const RowForm &f = core ? p->build : p->own;
+    const dim3 grid((p->n0 + kSegRows - 1) / kSegRows, f.nsy);
+    k_rows_seg<T, I><<<grid, 128, 0, s>>>(p->n0, p->n1, f.hop, f.halo, p->nfy, core ? 1 : 0, (const I *)ref,
+                                          (const I *)sci, mask, ftab_of<T>(p).fy, (const cpx<T> *)f.twy,
+                                          (cpx<T> *)p->F, (size_t)f.ncol * p->n0);
     p->launches++;
     return cudaGetLastError();
 }
@@ -719,17 +721,17 @@ cudaError_t rows_segments(Plan *p, const void *ref, const void *sci, const uint8
 }
 
 template <typename T, typename I>
-static cudaError_t rows_inv_seg_t(Plan *p, void *diff, cudaStream_t s) {
-    const dim3 grid((p->n0 + kSegRows - 1) / kSegRows, p->nsy);
-    k_rows_inv_seg<T, I><<<grid, 128, 0, s>>>(p->n0, p->n1, p->hop, p->halo, (const cpx<T> *)p->U,
-                                              (const cpx<T> *)p->twy, (I *)diff);
+static cudaError_t rows_inv_seg_t(Plan *p, const RowForm &f, void *diff, cudaStream_t s) {
+    const dim3 grid((p->n0 + kSegRows - 1) / kSegRows, f.nsy);
+    k_rows_inv_seg<T, I><<<grid, 128, 0, s>>>(p->n0, p->n1, f.hop, f.halo, (const cpx<T> *)p->U,
+                                              (const cpx<T> *)f.twy, (I *)diff);
     return cudaGetLastError();
 }
 
-cudaError_t rows_inv_segments(Plan *p, void *diff, cudaStream_t s) {
+cudaError_t rows_inv_segments(Plan *p, const RowForm &f, void *diff, cudaStream_t s) {
     const bool img64 = p->cfg.dtype == SFFT_F64;
-    if (p->fp64) return img64 ? rows_inv_seg_t<double, double>(p, diff, s) : rows_inv_seg_t<double, float>(p, diff, s);
-    return img64 ? rows_inv_seg_t<float, double>(p, diff, s) : rows_inv_seg_t<float, float>(p, diff, s);
+    if (p->fp64) return img64 ? rows_inv_seg_t<double, double>(p, f, diff, s) : rows_inv_seg_t<double, float>(p, f, diff, s);
+    return img64 ? rows_inv_seg_t<float, double>(p, f, diff, s) : rows_inv_seg_t<float, float>(p, f, diff, s);
 }
 
 }  // namespace sfft

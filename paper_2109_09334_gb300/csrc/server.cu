@@ -226,7 +226,7 @@ int flush(Server *v) {
         Slot &s = v->slots[seq % v->depth];
         Plan *p = s.plan;
         if (s.in_mask) e = row_transform(p, s.in_ref, s.in_sci, nullptr, false, v->ss);
-        if (e == cudaSuccess) e = subtract_from_rows(p, s.x, s.diff_out, v->ss);
+        if (e == cudaSuccess) e = subtract_from_rows(p, s.in_mask ? p->own : p->build, s.x, s.diff_out, v->ss);
         cudaStream_t last = v->ss;  // the stream of this request's last operation
         if (s.host) {  // results back to the host on so, overlapping the next group's work on ss
             const sfft_request &r = s.req;

@@ -437,12 +437,12 @@ static cudaError_t launch_rows_inv(Plan *p, void *diff, cudaStream_t s) {
 }
 
 template <typename T>
-static cudaError_t sub_t(Plan *p, const double *x, void *diff, cudaStream_t s) {
+static cudaError_t sub_t(Plan *p, const RowForm &f, const double *x, void *diff, cudaStream_t s) {
     cudaError_t err;
     p->launches += 3;
     const size_t csmem = (size_t)p->L1 * sizeof(T);
-    k_kernel_table<T><<<dim3((p->hc + 255) / 256, p->nk * p->L0), 256, csmem, s>>>(
-        p->ylen, p->bv, x, (const cpx<T> *)p->twy, (cpx<T> *)p->kap);
+    k_kernel_table<T><<<dim3((f.hc + 255) / 256, p->nk * p->L0), 256, csmem, s>>>(
+        f.ylen, p->bv, x, (const cpx<T> *)f.twy, (cpx<T> *)p->kap);
     if ((err = cudaGetLastError())) return err;
     {
         const SubShape h = sub_shape<T>(p);
@@ -461,12 +461,12 @@ static cudaError_t sub_t(Plan *p, const double *x, void *diff, cudaStream_t s) {
             }
         }
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h.smem);
-        kern<<<dim3(p->ncol, (p->n0 + seg - 1) / seg), h.threads, h.smem, s>>>(
-            p->n0, p->hc, p->ncol, p->offb, p->bv, ftab_of<T>(p), p->cfg.w0, nbkg_off, (const cpx<T> *)p->F,
-            (const cpx<T> *)p->kap, (const cpx<T> *)p->yhat, x, (cpx<T> *)p->U);
+        kern<<<dim3(f.ncol, (p->n0 + seg - 1) / seg), h.threads, h.smem, s>>>(
+            p->n0, f.hc, f.ncol, f.offb, p->bv, ftab_of<T>(p), p->cfg.w0, nbkg_off, (const cpx<T> *)p->F,
+            (const cpx<T> *)p->kap, (const cpx<T> *)f.yhat, x, (cpx<T> *)p->U);
         if ((err = cudaGetLastError())) return err;
     }
-    if (p->segy) return rows_inv_segments(p, diff, s);
+    if (f.seg) return rows_inv_segments(p, f, diff, s);
     return launch_rows_inv<T>(p, diff, s);
 }
 
@@ -768,8 +768,8 @@ cudaError_t decorrelate(Plan *p, const double *x, double xt0, double yt0, double
                    : decorr_t<float>(p, x, xt0, yt0, sigma_ref, sigma_sci, diff, out, co, s);
 }
 
-cudaError_t subtract_from_rows(Plan *p, const double *x, void *diff, cudaStream_t s) {
-    return p->fp64 ? sub_t<double>(p, x, diff, s) : sub_t<float>(p, x, diff, s);
+cudaError_t subtract_from_rows(Plan *p, const RowForm &f, const double *x, void *diff, cudaStream_t s) {
+    return p->fp64 ? sub_t<double>(p, f, x, diff, s) : sub_t<float>(p, f, x, diff, s);
 }
 
 }  // namespace sfft

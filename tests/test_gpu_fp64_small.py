@@ -31,7 +31,8 @@ CASES = [
     (64, 65, 2, 2, 1, 1, 1, False),     # segments
     (64, 127, 2, 2, 2, 1, 1, False),    # six terms: Bluestein rows of 256
     (64, 129, 2, 2, 2, 1, 1, False),    # segments
-    (64, 33, 2, 2, 0, 1, 1, False),     # one term: segments
+    (64, 31, 2, 2, 0, 1, 1, False),     # one term: Bluestein rows of 64
+    (64, 33, 2, 2, 0, 1, 1, False),     # segments
 ]
 
 
