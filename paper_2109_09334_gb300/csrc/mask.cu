@@ -22,8 +22,16 @@ constexpr int kMaxGrow = 16;
 constexpr int kMaskBlocks = 200;
 
 __host__ __device__ constexpr int mask_threads(int rows) { return rows == 64 ? 256 : 512; }
+// Resident blocks per SM.  Tall tiles run where the image makes many of them:
+// 8 blocks of 256 threads (32 registers) take the 1024 tiles of 4096 x 4096 in
+// one wave, 6 (40 registers) leave a second, nearly empty one: 54 -> 45 us,
+// halo 0.  FP64 at 6 instead of 5: 3500 x 4000 98 -> 70 us.
+template <typename I>
+__host__ __device__ constexpr int mask_blocks(int rows) {
+    return rows == 64 ? (sizeof(I) == 4 ? 8 : 6) : 2;
+}
 template <typename I, int ROWS>
-__global__ void __launch_bounds__(mask_threads(ROWS), ROWS == 64 ? 1 : 2)
+__global__ void __launch_bounds__(mask_threads(ROWS), mask_blocks<I>(ROWS))
     k_sat_mask(int n0, int n1, const I *__restrict__ R, const I *__restrict__ S, I sat_r, I sat_s, int grow, bool vec,
                const uint8_t *mask_in, uint8_t *mask_out) {
     constexpr int kMaskThreads = mask_threads(ROWS);

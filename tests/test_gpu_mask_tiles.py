@@ -38,3 +38,30 @@ def test_tiles_match_oracle(n0, n1, grow, dtype):
     B.sfft_saturation_mask(torch.from_numpy(R).cuda(), torch.from_numpy(S).cuda(), sat, sat, grow, m, d_mask_in=m)
     torch.cuda.synchronize()
     assert np.array_equal(m.cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("dtype,small,large", [("float32", (3500, 4000), (4096, 4096)),
+                                               ("float64", (3001, 2048), (3500, 4000))])
+def test_time_grows_no_faster_than_pixels(dtype, small, large):
+    """The larger image's tiles run in one wave too (1024 of 64 rows in FP32, 880
+    in FP64): its time against the smaller's is at most their pixels', and a
+    tenth for noise.  With fewer resident blocks its last tiles took a wave of
+    their own: 1.38 times for 1.20 times the pixels, 2.65 for 2.28."""
+    from paper_2109_09334_gb300 import binding as B
+
+    def best(n0, n1):
+        R, S = (torch.rand((n0, n1), device="cuda", dtype=getattr(torch, dtype)) for _ in range(2))
+        m = torch.empty((n0, n1), dtype=torch.uint8, device="cuda")
+        ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        times = []
+        for _ in range(8):
+            ev[0].record()
+            for _ in range(20):
+                B.sfft_saturation_mask(R, S, 0.999, 0.999, 0, m)
+            ev[1].record()
+            torch.cuda.synchronize()
+            times.append(ev[0].elapsed_time(ev[1]))
+        return min(times)
+
+    pixels = large[0] * large[1] / (small[0] * small[1])
+    assert best(*large) <= 1.1 * pixels * best(*small)
